@@ -244,6 +244,7 @@ void split_any(const Src &src, int rows, int K, int row0, Sliced &o, cudaStream_
     case 2: k_digits<2, Src><<<gd, 256, 0, s>>>(src, K, kpad, row0, plane, o.expo, dig); break;
     case 3: k_digits<3, Src><<<gd, 256, 0, s>>>(src, K, kpad, row0, plane, o.expo, dig); break;
     case 4: k_digits<4, Src><<<gd, 256, 0, s>>>(src, K, kpad, row0, plane, o.expo, dig); break;
+    case S_WIDE: k_digits<S_WIDE, Src><<<gd, 256, 0, s>>>(src, K, kpad, row0, plane, o.expo, dig); break;
     default: k_digits<5, Src><<<gd, 256, 0, s>>>(src, K, kpad, row0, plane, o.expo, dig); break;
   }
   ++launch_counter();
@@ -308,36 +309,42 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 }
 
 
-// instruction descriptors: D = F32, A and B K-major, M = 128, N = BN; A/B format 1 = BF16
-// (kind::f16) or 2 = TF32 (kind::tf32)
-constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                           ((uint32_t)(BM >> 4) << 24);
-constexpr uint32_t IDESC_TF32 = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                                ((uint32_t)(BM >> 4) << 24);
+// instruction descriptor: D = F32, A and B K-major, M = 128, N = n; A/B format 1 = BF16 (kind::f16)
+// or 2 = TF32 (kind::tf32)
+__host__ __device__ constexpr uint32_t idesc(uint32_t n, bool tf32) {
+  return (1u << 4) | ((tf32 ? 2u : 1u) << 7) | ((tf32 ? 2u : 1u) << 10) | ((n >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+}
 
-__device__ __forceinline__ void umma(uint32_t d, uint64_t a, uint64_t b, uint32_t acc) {
+__device__ __forceinline__ void umma(uint32_t d, uint64_t a, uint64_t b, uint32_t desc, uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-      ::"r"(d), "l"(a), "l"(b), "r"(IDESC), "r"(acc)
+      ::"r"(d), "l"(a), "l"(b), "r"(desc), "r"(acc)
       : "memory");
 }
-__device__ __forceinline__ void umma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t acc) {
+__device__ __forceinline__ void umma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t desc, uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n"
-      ::"r"(d), "l"(a), "l"(b), "r"(IDESC_TF32), "r"(acc)
+      ::"r"(d), "l"(a), "l"(b), "r"(desc), "r"(acc)
       : "memory");
 }
 __device__ __forceinline__ void umma_commit(uint64_t *bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
 }
+// 16 columns of the warp's 32 TMEM lanes; the registers are valid after tmem_ld_wait on them
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
 }
 
 // An output tile; c_n >= 0: only the K stages listed at chunks[c_off .. + c_n) (in units of the
@@ -421,26 +428,67 @@ __device__ __forceinline__ float2 i64_to_f32x2(long long a, int sh) {
   return neg ? make_float2(-hi, -lo) : make_float2(hi, lo);
 }
 
+// (hi 2^32 + lo) 2^sh as FP64, rounded to nearest even (|hi|, |lo| < 2^62): the two words are carried
+// into one sign and a 96-bit magnitude, whose leading 64 bits (with a sticky bit) are rounded
+__device__ __forceinline__ double i96_to_f64(long long hi, long long lo, int sh) {
+  hi += lo >> 32;
+  unsigned l = (unsigned)(unsigned long long)lo;
+  const bool neg = hi < 0;
+  if (neg) {
+    l = 0u - l;
+    hi = l ? ~hi : -hi;
+  }
+  const unsigned long long h = (unsigned long long)hi;
+  if (h == 0) {
+    const double v = i64_to_f64((long long)l, sh);
+    return neg ? -v : v;
+  }
+  const int lz = __clzll((long long)h);
+  unsigned long long m = h << lz;   // leading one at bit 63 of the upper 64 of 96 bits
+  unsigned rest = 0;
+  if (lz <= 32) {
+    m |= (unsigned long long)l >> (32 - lz);
+    rest = lz < 32 ? l << lz : 0u;
+  } else {
+    m |= (unsigned long long)l << (lz - 32);
+  }
+  unsigned long long mant = m >> 11;
+  const unsigned rem = (unsigned)(m & 0x7FFull);
+  int e = 1086 - lz + 32 + sh;
+  if (rem > 0x400u || (rem == 0x400u && (rest != 0u || (mant & 1ull)))) {
+    ++mant;
+    if (mant >> 53) {
+      mant >>= 1;
+      ++e;
+    }
+  }
+  if (e <= 0 || e >= 2047) {   // outside the normal range (rare)
+    const double v = ldexp((double)m, sh + 32 - lz);
+    return neg ? -v : v;
+  }
+  return __longlong_as_double(
+      (long long)((neg ? 0x8000000000000000ull : 0ull) | ((unsigned long long)e << 52) | (mant & 0xFFFFFFFFFFFFFull)));
+}
+
 template <int S>
 __host__ __device__ constexpr uint32_t tmem_cols() {
   return S * BN <= 64 ? 64 : S * BN <= 128 ? 128 : S * BN <= 256 ? 256 : 512;
 }
 constexpr uint64_t WAIT_NS = 2000000000ull;   // 2 s
 
-// Pipelined, warp-specialised kernel (one CTA = one 128 x 64 output tile of one GEMM entry):
-//   warp EW (one lane): TMA producer over a ring of NST shared-memory stages, each holding the
-//     NP digit planes of a 128 x 32 A slice and a 64 x 32 B slice (SWIZZLE_64B, K-major);
-//   warp EW + 1 (one lane): tcgen05.mma issuer; commits free a stage when its MMAs complete
-//     and, at the end of a flush group, signal the epilogue;
-//   warps 0..EW-1: epilogue; warp w owns TMEM lanes 32 (w % 4) .. + 31 (= tile rows).  With
-//     EW = 8 (digit planes) warp w takes columns 32 (w / 4) .. + 31: after each flush group it
-//     moves the diagonal accumulators into exact int64 register sums (32 per thread) and hands
-//     the TMEM columns back to the issuer.  With EW = 4 (plain BF16 / TF32, one drain at the
-//     end) each warp takes all 64 columns.
 constexpr int PBK = 32;   // K per stage: one 64-byte swizzle row of BF16 (16 TF32 values)
-constexpr int NST = 3;    // pipeline depth
+// pipeline depth: 3 stages (180 KB with 5 planes); 2 with more planes (8 planes: 96 KB a stage)
+__host__ __device__ constexpr int ring_stages(int S) { return S == S_WIDE ? 2 : 3; }
 // epilogue warps of the S variant
-__host__ __device__ constexpr int epi_warps(int S) { return (S == 0 || S == S_TF32 || S == S_TF32X3) ? 4 : 8; }
+__host__ __device__ constexpr int epi_warps(int S) { return is_digits(S) ? 8 : 4; }
+// columns the epilogue stages at a time, and bytes of its staging area: 16 columns of int64 sums, pitch
+// 17 (conflict-free by rows and by columns), or 4 columns of two-word sums, pitch 5
+__host__ __device__ constexpr int stage_cols(int S) { return S == S_WIDE ? 4 : 16; }
+__host__ __device__ constexpr int stage_bytes(int S) {
+  return is_digits(S) ? epi_warps(S) * 32 * (stage_cols(S) + 1) * (S == S_WIDE ? 16 : 8) : 0;
+}
+// digit planes of B multiplied by one MMA: at most 256 columns
+constexpr int kStack = 256 / BN;
 
 // shared-memory matrix descriptor: K-major, 64-byte swizzle, 8-row groups 512 bytes apart
 __device__ __forceinline__ uint64_t smem_desc64(uint32_t saddr) {
@@ -472,13 +520,19 @@ struct alignas(128) MapPair {
 //     across tiles, so the next tile's loads overlap this tile's MMAs and epilogue;
 //   warp EW + 1 (one lane): tcgen05.mma issuer; commits free a stage when its MMAs complete and, at
 //     the end of a flush group, signal the epilogue; the next group (of this or the next tile)
-//     starts once the epilogue has drained the accumulators;
+//     starts once the epilogue has drained the accumulators.  The B planes lie one after the other in a
+//     stage and the accumulators of consecutive diagonals in consecutive columns, so plane s of A
+//     meets up to four planes of B in one MMA of N = 256: 6 MMAs per K step of 16 with 5 planes in place of 15
+//     of N = 64, and A read from shared memory 6 times instead of 15 (54 KB a step, below what the
+//     MMAs' 480 cycles can take; at N = 64 the 90 KB held the tensor pipe at two thirds);
 //   warps 0..EW-1: epilogue; warp w owns TMEM lanes 32 (w % 4) .. + 31 (= tile rows).  With EW = 8
 //     (digit planes) warp w takes columns 32 (w / 4) .. + 31 and after each flush group moves the
-//     diagonal accumulators into exact int64 register sums (32 per thread); with EW = 4 (plain
-//     BF16 / TF32, one group) each warp takes all 64 columns into registers.  The TMEM columns go
-//     back to the issuer before the values are converted and stored, so conversion and stores
-//     overlap the next tile's MMAs.
+//     diagonal accumulators into exact int64 register sums (32 per thread, two words each with 8
+//     planes); with EW = 4 (plain BF16 / TF32, one group) each warp takes all 64 columns into
+//     registers.  The TMEM columns go back to the issuer before the values are converted and stored, so
+//     conversion and stores overlap the next tile's MMAs.  The sums go through a per-warp staging area into
+//     short rolled loops that convert and store: the conversion is ~50 instructions, and unrolled over
+//     a thread's 32 sums it ran from outside the instruction cache.
 // stall_ns > 0 (testing only): the MMA issuer first waits that long on an mbarrier nothing arrives
 // at, so the CTA takes the bounded-wait failure path.  On any failure the CTA sets *err, stops
 // issuing, waits (with the full limit) for the TMA copies and MMAs it has already issued, frees its
@@ -488,8 +542,10 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
     k_ozgemm(const MapPair *__restrict__ maps, const Entry *__restrict__ entries, const Tile *__restrict__ tiles,
              const int *__restrict__ chunks, int ntiles, int *err, uint64_t stall_ns, int stage_in_ring) {
   constexpr bool TF = S == S_TF32 || S == S_TF32X3;   // kind::tf32
-  constexpr bool PLAIN = S == 0 || TF;                 // one FP32 accumulator over all K
-  constexpr int NP = S == S_TF32X3 ? 2 : PLAIN ? 1 : S;   // planes per operand
+  constexpr bool PLAIN = !is_digits(S);                // one FP32 accumulator over all K
+  constexpr bool WIDE = S == S_WIDE;                   // two-word sums
+  constexpr int NP = planes(S);                        // planes per operand
+  constexpr int NST = ring_stages(S);
   constexpr int KS = TF ? PBK / 2 : PBK;               // K elements per stage (64 bytes per row)
   constexpr uint32_t A_BYTES = BM * 64, B_BYTES = BN * 64;
   constexpr uint32_t STAGE = NP * (A_BYTES + B_BYTES);
@@ -498,7 +554,6 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
   constexpr int G = PLAIN ? (1 << 30) : 32 / NP;
   constexpr int EPI_WARPS = epi_warps(S), HALF = BN * 4 / EPI_WARPS;   // HALF: columns per epilogue warp
   constexpr uint32_t TMEM_COLS = tmem_cols<PLAIN ? 1 : NP>();
-  constexpr int SPITCH = 17;   // staging: 32 rows x 16 columns (+1) of 8-byte values per epilogue warp
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t full[NST], empty[NST], tfull, tempty, mdone, never;
   __shared__ uint32_t tmem_slot;
@@ -507,7 +562,7 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   // the epilogue's staging area: in the pipeline's stages when the CTA has a single tile (they are
   // idle once its last MMA completed), else after them
-  double *stage_out = reinterpret_cast<double *>(stage_in_ring ? smem : smem + NST * STAGE);
+  uint8_t *stage_out = stage_in_ring ? smem : smem + NST * STAGE;
   if (tid == 0) {
 #pragma unroll
     for (int s = 0; s < NST; ++s) {
@@ -539,7 +594,7 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
       long long it = 0;   // stages issued so far (all tiles)
       for (int t = blockIdx.x; t < ntiles && !abort_flag; t += gridDim.x) {
         const Tile tl = tiles[t];
-        const Entry en = entries[tl.e];
+        const Entry &en = entries[tl.e];
         const MapPair *mp = maps + en.pair;
         int kbeg;
         const int nsteps = steps_of(en, tl, kbeg);
@@ -574,9 +629,8 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
       long long it = 0, g = 0;   // stages consumed, flush groups committed (all tiles)
       for (int t = blockIdx.x; t < ntiles && !abort_flag; t += gridDim.x) {
         const Tile tl = tiles[t];
-        const Entry en = entries[tl.e];
         int kbeg;
-        const int nsteps = steps_of(en, tl, kbeg);
+        const int nsteps = steps_of(entries[tl.e], tl, kbeg);
         for (int i = 0; i < nsteps; ++i, ++it) {
           const int st = (int)(it % NST), c = i % G;
           // a new group needs the accumulators drained by the epilogue (previous group, any tile)
@@ -590,22 +644,36 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
           }
           tc_fence_after();
           const uint32_t sa = smem_u32(smem + st * STAGE), sb = sa + NP * A_BYTES;
+          if constexpr (PLAIN) {
+            // one accumulator for all products: hi hi (and hi lo, lo hi of the 3xTF32 split)
 #pragma unroll
-          for (int s = 1; s <= NP; ++s)
+            for (int s = 1; s <= NP; ++s)
 #pragma unroll
-            for (int u = 1; u + s <= NP + 1; ++u)
+              for (int u = 1; u + s <= NP + 1; ++u)
 #pragma unroll
-              for (int j = 0; j < 2; ++j) {   // two MMAs of 32 bytes of K per 64-byte row
-                const uint64_t da = smem_desc64(sa + (s - 1) * A_BYTES + 32 * j);
-                const uint64_t db = smem_desc64(sb + (u - 1) * B_BYTES + 32 * j);
-                // digit planes: one accumulator per diagonal s + u; plain forms: one for all
-                const uint32_t col = PLAIN ? 0u : (uint32_t)(s + u - 2) * BN;
-                const uint32_t accum = (c == 0 && j == 0 && s == 1 && (!PLAIN || u == 1)) ? 0u : 1u;
-                if constexpr (TF)
-                  umma_tf32(tmem + col, da, db, accum);
-                else
-                  umma(tmem + col, da, db, accum);
-              }
+                for (int j = 0; j < 2; ++j) {   // two MMAs of 32 bytes of K per 64-byte row
+                  const uint64_t da = smem_desc64(sa + (s - 1) * A_BYTES + 32 * j);
+                  const uint64_t db = smem_desc64(sb + (u - 1) * B_BYTES + 32 * j);
+                  const uint32_t accum = (c == 0 && j == 0 && s == 1 && u == 1) ? 0u : 1u;
+                  if constexpr (TF)
+                    umma_tf32(tmem, da, db, idesc(BN, true), accum);
+                  else
+                    umma(tmem, da, db, idesc(BN, false), accum);
+                }
+          } else {
+            // plane s of A by planes u .. u + w - 1 of B (N = 64 w), into the diagonals s + u ..
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+              for (int s = 1; s <= NP; ++s)
+#pragma unroll
+                for (int u = 1; u + s <= NP + 1; u += kStack) {
+                  const int w = NP + 2 - s - u < kStack ? NP + 2 - s - u : kStack;
+                  const uint64_t da = smem_desc64(sa + (s - 1) * A_BYTES + 32 * j);
+                  const uint64_t db = smem_desc64(sb + (u - 1) * B_BYTES + 32 * j);
+                  umma(tmem + (uint32_t)(s + u - 2) * BN, da, db, idesc(BN * w, false), (c == 0 && j == 0 && s == 1) ? 0u : 1u);
+                }
+          }
           umma_commit(&empty[st]);
           if (c == G - 1 || i == nsteps - 1) {
             umma_commit(&tfull);
@@ -622,24 +690,27 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
     }
   } else {
     const int quad = warp & 3, half = warp >> 2;   // TMEM lane quadrant, column half
-    double *stg = stage_out + (size_t)warp * 32 * SPITCH;
+    const uint32_t tbase = tmem + ((uint32_t)(32 * quad) << 16) + half * HALF;
     long long g = 0;   // flush groups drained (all tiles)
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
       const Tile tl = tiles[t];
-      const Entry en = entries[tl.e];
+      const Entry &en = entries[tl.e];
       int kbeg;
       const int nsteps = steps_of(en, tl, kbeg);
       const int ngroups = (nsteps + G - 1) / G;
       const int m0 = tl.m0, n0 = tl.n0;
-      long long acc[HALF];       // digit planes: exact int64 sums of the diagonals, or (fpath) an FP32 pair
+      // digit planes: exact sums of the diagonals, in units of the last one's scale (WIDE: the first four
+      // diagonals in acch, in units of the fourth's, the last four in acc)
+      long long acc[PLAIN ? 1 : HALF], acch[WIDE ? HALF : 1];
       uint32_t fa[PLAIN ? HALF : 1];   // plain forms: the FP32 accumulators
+      if constexpr (!PLAIN) {
 #pragma unroll
-      for (int j = 0; j < HALF; ++j) acc[j] = 0;
-      // FP32-pair outputs of a tile with a single flush group (the short-K GEMMs of the chi0 steps):
-      // the diagonal sums, exact integers below 2^24 times their powers of two, are summed into an
-      // unevaluated FP32 pair (hi, lo) by exact two-sums, held in the int64 slot's two halves --
-      // FP32 arithmetic instead of the int64 sum and its conversion
-      const bool fpath = !PLAIN && ngroups == 1 && en.mode == 3 && en.alpha_shift != kNoShift;
+        for (int j = 0; j < HALF; ++j) acc[j] = 0;
+        if constexpr (WIDE) {
+#pragma unroll
+          for (int j = 0; j < HALF; ++j) acch[j] = 0;
+        }
+      }
       bool ok_all = true;
       for (int gi = 0; gi < ngroups; ++gi, ++g) {
         bool ok = !abort_flag && mbar_wait(&tfull, (uint32_t)(g & 1), WAIT_NS, &abort_flag);
@@ -651,37 +722,30 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
         }
         tc_fence_after();
         if constexpr (!PLAIN) {
-          if (fpath) {
-#pragma unroll 1
-            for (int d = 2; d <= S + 1; ++d) {
-              const float mulf = __uint_as_float((uint32_t)(127 + 8 * (S + 1 - d)) << 23);   // 2^(8(S+1-d))
+          // 16 columns of one diagonal at a time, the next load in flight while these are added
+          // (registers for one load only with the two-word sums)
+          constexpr int CB = HALF / 16, NL = S * CB, RB = WIDE ? 1 : 2;
+          uint32_t r[RB][16];
+          if (!WIDE) tmem_ld16(tbase, r[0]);
 #pragma unroll
-              for (int cb = 0; cb < HALF / 16; ++cb) {
-                uint32_t r[16];
-                tmem_ld16(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(d - 2) * BN + half * HALF + cb * 16, r);
+          for (int l = 0; l < NL; ++l) {
+            const int d = l / CB, cb = l % CB;
+            if (WIDE) tmem_ld16(tbase + (uint32_t)d * BN + cb * 16, r[0]);
+            tmem_ld_wait(r[l % RB]);
+            if (!WIDE && l + 1 < NL)
+              tmem_ld16(tbase + (uint32_t)((l + 1) / CB) * BN + ((l + 1) % CB) * 16, r[(l + 1) % RB]);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                  const int c = cb * 16 + j;
-                  const float t = __uint_as_float(r[j]) * mulf;   // exact
-                  const float hi = __int_as_float((int)(acc[c] & 0xFFFFFFFFll));
-                  float lo = __int_as_float((int)(acc[c] >> 32));
-                  const float sm = hi + t, bb = sm - hi;
-                  lo += (hi - (sm - bb)) + (t - bb);
-                  acc[c] = ((long long)__float_as_int(lo) << 32) | (long long)(uint32_t)__float_as_int(sm);
-                }
-              }
-            }
-          } else {
-#pragma unroll 1
-            for (int d = 2; d <= S + 1; ++d) {
-              const long long mul = 1LL << (8 * (S + 1 - d));
-#pragma unroll
-              for (int cb = 0; cb < HALF / 16; ++cb) {
-                uint32_t r[16];
-                tmem_ld16(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(d - 2) * BN + half * HALF + cb * 16, r);
-#pragma unroll
-                for (int j = 0; j < 16; ++j)
-                  acc[cb * 16 + j] += (long long)__float2int_rn(__uint_as_float(r[j])) * mul;
+            for (int j = 0; j < 16; ++j) {
+              const int v = __float2int_rn(__uint_as_float(r[l % RB][j]));
+              if constexpr (WIDE) {
+                if (d < 4)
+                  acch[cb * 16 + j] += (long long)v * (1 << (8 * (3 - d)));
+                else
+                  acc[cb * 16 + j] += (long long)v * (1 << (8 * (7 - d)));
+              } else if (S == 5 && d == 0) {
+                acc[cb * 16 + j] += (long long)((unsigned long long)(unsigned)v << 32);   // 2^32 v (mod 2^64)
+              } else {
+                acc[cb * 16 + j] += (long long)v * (1 << (8 * (S - 1 - d) % 32));
               }
             }
           }
@@ -689,7 +753,8 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
 #pragma unroll
           for (int cb = 0; cb < HALF / 16; ++cb) {
             uint32_t r[16];
-            tmem_ld16(tmem + ((uint32_t)(32 * quad) << 16) + half * HALF + cb * 16, r);
+            tmem_ld16(tbase + cb * 16, r);
+            tmem_ld_wait(r);
 #pragma unroll
             for (int j = 0; j < 16; ++j) fa[cb * 16 + j] = r[j];
           }
@@ -699,116 +764,123 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
         if (lane == 0) mbar_arrive(&tempty);   // the accumulators may be overwritten now
       }
       if (!ok_all) break;
+      const int eM = en.M, eN = en.N, mode = en.mode;
+      const long long ldc = en.ldc;
+      double *const C = en.C;
+      const double alpha = en.alpha, beta = en.beta;
+      const bool pow2 = en.alpha_shift != kNoShift;   // alpha = +-2^alpha_shift: folded into the exponent
+      const int row = m0 + 32 * quad + lane;          // thread = tile row (the TMEM lane layout)
+      const bool row_ok = row < eM;
+      // one output element (modes 0, 1, 2, 4)
+      auto store = [&](int r_, int c_, double v) {
+        double *p = mode == 0   ? C + (long long)r_ * ldc + c_
+                    : mode == 1 ? C + 2 * ((long long)(r_ >> 1) * ldc + c_) + (r_ & 1)
+                    : mode == 4 ? C + (long long)c_ * ldc + r_
+                                : C + 2 * ((long long)c_ * ldc + (r_ >> 1)) + (r_ & 1);
+        *p = beta == 0.0 ? v : v + beta * *p;
+      };
       if constexpr (PLAIN) {
         // plain forms: one FP32 sum per element, scaled in FP64 and stored from the registers,
         // thread = tile row
-        const int row = m0 + 32 * quad + lane;
-        if (row < en.M) {
+        if (row_ok) {
 #pragma unroll
           for (int c = 0; c < HALF; ++c) {
             const int col = n0 + half * HALF + c;
-            if (col >= en.N) break;
-            if (en.mode == 3 && en.alpha_shift != kNoShift) {   // the FP32 sum times +-2^k: exact in FP32
-              const float f = nsteps > 0 ? __uint_as_float(fa[c]) * (float)en.alpha : 0.f;
-              reinterpret_cast<float2 *>(en.C)[(long long)row * en.ldc + col] = make_float2(f, 0.f);
+            if (col >= eN) break;
+            if (mode == 3 && pow2) {   // the FP32 sum times +-2^k: exact in FP32
+              const float f = nsteps > 0 ? __uint_as_float(fa[c]) * (float)alpha : 0.f;
+              reinterpret_cast<float2 *>(C)[(long long)row * ldc + col] = make_float2(f, 0.f);
               continue;
             }
-            const double v = nsteps > 0 ? en.alpha * (double)__uint_as_float(fa[c]) : 0.0;
-            if (en.mode == 3) {   // real, as an unevaluated pair of FP32 numbers (hi, lo)
+            const double v = nsteps > 0 ? alpha * (double)__uint_as_float(fa[c]) : 0.0;
+            if (mode == 3) {   // real, as an unevaluated pair of FP32 numbers (hi, lo)
               const float hi = __double2float_rn(v);
-              reinterpret_cast<float2 *>(en.C)[(long long)row * en.ldc + col] =
+              reinterpret_cast<float2 *>(C)[(long long)row * ldc + col] =
                   make_float2(hi, __double2float_rn(v - (double)hi));
               continue;
             }
-            double *p = en.mode == 0   ? en.C + (long long)row * en.ldc + col
-                        : en.mode == 1 ? en.C + 2 * ((long long)(row >> 1) * en.ldc + col) + (row & 1)
-                        : en.mode == 4 ? en.C + (long long)col * en.ldc + row
-                                       : en.C + 2 * ((long long)col * en.ldc + (row >> 1)) + (row & 1);
-            *p = en.beta == 0.0 ? v : v + en.beta * *p;
+            store(row, col, v);
           }
         }
-        continue;
-      }
-      // Digit planes: values are formed with thread = tile row (the TMEM lane layout).  Row-major outputs
-      // (modes 0, 1, 3) go through a per-warp staging area, 16 columns at a time, and are written
-      // with lanes along the row (two rows of 16 columns per warp store); the transposed outputs
-      // (modes 2, 4) are consecutive along rows already and are stored directly.
-      const int row = m0 + 32 * quad + lane;
-      const bool row_ok = row < en.M;
-      const int ea = (!PLAIN && row_ok) ? maps[en.pair].ea[en.a_row0 + row] : 0;
-      const int *eb = maps[en.pair].eb;
-      const int cbase = n0 + half * HALF;
-      const bool pow2 = en.alpha_shift != kNoShift;   // alpha = +-2^alpha_shift: folded into the exponent
-      const int ash = pow2 ? en.alpha_shift : 0;
-      const bool aneg = pow2 && en.alpha < 0.0;
-      const bool staged = en.mode != 2 && en.mode != 4;
+      } else {
+        constexpr int SC = stage_cols(S);
+        const MapPair &mp = maps[en.pair];
+        const int ea = row_ok ? mp.ea[en.a_row0 + row] : 0;
+        const int *eb = mp.eb + en.b_row0;
+        const int ash = (pow2 ? en.alpha_shift : 0) - 14 - 8 * (S - 1);
+        const bool aneg = pow2 && alpha < 0.0;
+        const int cbase = n0 + half * HALF;
+        // value of a sum: its scale from the row's and the column's exponents; a row or column with an
+        // infinity or a NaN (exponent 1025) gives NaN
+        auto value = [&](long long hi, long long lo, int e_a, int e_b) {
+          const int sh = e_a + e_b + ash;
+          double v;
+          if constexpr (WIDE)
+            v = i96_to_f64(aneg ? -hi : hi, aneg ? -lo : lo, sh);
+          else
+            v = i64_to_f64(aneg ? -lo : lo, sh);
+          if (!pow2) v *= alpha;
+          return e_a > 1024 || e_b > 1024 ? __longlong_as_double(0x7FF8000000000000ll) : v;
+        };
+        long long *stg = reinterpret_cast<long long *>(stage_out + (size_t)warp * (stage_bytes(S) / EPI_WARPS));
 #pragma unroll
-      for (int cb = 0; cb < HALF / 16; ++cb) {
+        for (int cb = 0; cb < HALF / SC; ++cb) {
+          const int col0 = cbase + cb * SC;
+          if (col0 >= eN) break;   // the same for the whole warp
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int c = cb * 16 + j, col = cbase + c;
-          const bool ok = row_ok && col < en.N;
-          double v = 0.0;
-          float2 pr = make_float2(0.f, 0.f);
-          if (ok) {
-            {
-              const int sh = ea + eb[en.b_row0 + col] - 14 - 8 * (S - 1) + ash;
-              const long long a = aneg ? -acc[c] : acc[c];
-              if (fpath) {
-                // renormalise the pair, then scale it by 2^sh (exact in the normal range)
-                float hi = __int_as_float((int)(acc[c] & 0xFFFFFFFFll)), lo = __int_as_float((int)(acc[c] >> 32));
-                const float sm = hi + lo;
-                lo = lo - (sm - hi);
-                hi = sm;
-                if (aneg) {
-                  hi = -hi;
-                  lo = -lo;
+          for (int j = 0; j < SC; ++j) {
+            if constexpr (WIDE)
+              reinterpret_cast<longlong2 *>(stg)[lane * (SC + 1) + j] = make_longlong2(acch[cb * SC + j], acc[cb * SC + j]);
+            else
+              stg[lane * (SC + 1) + j] = acc[cb * SC + j];
+          }
+          __syncwarp();
+          if (WIDE || mode == 2 || mode == 4) {
+            // thread = tile row: the transposed outputs are consecutive along the lanes; with the two-word sums
+            // a lane writes 4 columns, one 32-byte sector of a row-major output
+            const int nc = min(SC, eN - col0);
+            if (row_ok) {
+#pragma unroll 1
+              for (int j = 0; j < nc; ++j) {
+                double v;
+                if constexpr (WIDE) {
+                  const longlong2 a = reinterpret_cast<const longlong2 *>(stg)[lane * (SC + 1) + j];
+                  v = value(a.x, a.y, ea, eb[col0 + j]);
+                } else {
+                  v = value(0, stg[lane * (SC + 1) + j], ea, eb[col0 + j]);
                 }
-                const int eh = (int)((__float_as_uint(hi) >> 23) & 0xFF);
-                if (sh >= -126 && sh <= 127 && (hi == 0.f || (eh + sh >= 1 && eh + sh <= 254))) {
-                  const float sc = __uint_as_float((uint32_t)(sh + 127) << 23);
-                  pr = make_float2(hi * sc, lo * sc);
-                } else {   // outside the FP32 range of a direct scaling: through FP64
-                  const double dv = ldexp((double)hi + (double)lo, sh);
-                  pr.x = __double2float_rn(dv);
-                  pr.y = __double2float_rn(dv - (double)pr.x);
-                }
-              } else if (en.mode == 3 && pow2) {
-                pr = i64_to_f32x2(a, sh);
-              } else {
-                v = i64_to_f64(a, sh);
-                if (!pow2) v *= en.alpha;
-                if (en.mode == 3) {
-                  pr.x = __double2float_rn(v);
-                  pr.y = __double2float_rn(v - (double)pr.x);
+                if (WIDE && mode == 3) {
+                  const float h = __double2float_rn(v);
+                  reinterpret_cast<float2 *>(C)[(long long)row * ldc + col0 + j] =
+                      make_float2(h, __double2float_rn(v - (double)h));
+                } else {
+                  store(row, col0 + j, v);
                 }
               }
             }
-          }
-          if (en.mode == 3)
-            v = __longlong_as_double(
-                (long long)(((unsigned long long)__float_as_uint(pr.y) << 32) | __float_as_uint(pr.x)));
-          if (staged) {
-            stg[lane * SPITCH + j] = v;
-          } else if (ok) {
-            double *p = en.mode == 4 ? en.C + (long long)col * en.ldc + row
-                                     : en.C + 2 * ((long long)col * en.ldc + (row >> 1)) + (row & 1);
-            *p = en.beta == 0.0 ? v : v + en.beta * *p;
-          }
-        }
-        if (staged) {
-          __syncwarp();
-          const int cl = lane & 15, col = cbase + cb * 16 + cl;
-          for (int rr = lane >> 4; rr < 32; rr += 2) {
-            const int grow = m0 + 32 * quad + rr;
-            if (grow < en.M && col < en.N) {
-              const double v = stg[rr * SPITCH + cl];
-              if (en.mode == 3) {   // the 8 bytes already hold the pair (hi, lo)
-                reinterpret_cast<double *>(en.C)[(long long)grow * en.ldc + col] = v;
-              } else {
-                double *p = en.mode == 0 ? en.C + (long long)grow * en.ldc + col
-                                         : en.C + 2 * ((long long)(grow >> 1) * en.ldc + col) + (grow & 1);
-                *p = en.beta == 0.0 ? v : v + en.beta * *p;
+          } else {
+            // lanes along the columns: two rows of 16 columns per store
+            const int cl = lane & 15, col = col0 + cl;
+            const int e_b = col < eN ? eb[col] : 0;
+#pragma unroll 2
+            for (int r2 = 0; r2 < 32; r2 += 2) {
+              const int rr = r2 + (lane >> 4), grow = m0 + 32 * quad + rr;
+              const int e_a = __shfl_sync(0xffffffffu, ea, rr);
+              if (grow < eM && col < eN) {
+                const long long a = stg[rr * (SC + 1) + cl];
+                if (mode == 3) {
+                  float2 pr;
+                  if (pow2 && e_a <= 1024 && e_b <= 1024) {
+                    pr = i64_to_f32x2(aneg ? -a : a, e_a + e_b + ash);
+                  } else {
+                    const double v = value(0, a, e_a, e_b);
+                    pr.x = __double2float_rn(v);
+                    pr.y = __double2float_rn(v - (double)pr.x);
+                  }
+                  reinterpret_cast<float2 *>(C)[(long long)grow * ldc + col] = pr;
+                } else {
+                  store(grow, col, value(0, a, e_a, e_b));
+                }
               }
             }
           }
@@ -823,7 +895,6 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, TMEM_COLS);
 }
-
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 
@@ -842,17 +913,23 @@ CUtensorMap make_map(const Sliced &o, int box_rows) {
   return m;
 }
 
+// dynamic shared memory of k_ozgemm<S>: the pipeline's stages and the epilogue's staging area, overlapping
+// when every CTA has one tile (the shared memory, and so the CTAs an SM holds at once, stay those
+// of the stages alone)
+constexpr int ring_bytes(int S) { return ring_stages(S) * planes(S) * (BM + BN) * 64; }
+constexpr int gemm_smem(int S, bool in_ring) {
+  return (in_ring ? (ring_bytes(S) > stage_bytes(S) ? ring_bytes(S) : stage_bytes(S)) : ring_bytes(S) + stage_bytes(S)) + 1024;
+}
+
 template <int S>
 void launch(const MapPair *mp, const Entry *e, const Tile *t, const int *c, int ntiles, int grid, int *err,
             uint64_t stall_ns, cudaStream_t s) {
-  // the pipeline's stages and the epilogue's staging area (32 rows x 17 doubles per epilogue warp),
-  // overlapping when every CTA has one tile (the shared memory, and so the CTAs an SM holds at
-  // once, stay those of the stages alone)
-  const int ring = NST * planes(S) * (BM + BN) * 64, staging = epi_warps(S) * 32 * 17 * 8;
-  const int in_ring = grid >= ntiles ? 1 : 0;
-  const int smem = (in_ring ? std::max(ring, staging) : ring + staging) + 1024;
-  LR_CUDA(cudaFuncSetAttribute(k_ozgemm<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  k_ozgemm<S><<<grid, 32 * (epi_warps(S) + 2), smem, s>>>(mp, e, t, c, ntiles, err, stall_ns, in_ring);
+  static_assert(gemm_smem(S, false) <= 226 * 1024, "k_ozgemm: shared memory");
+  const bool in_ring = grid >= ntiles;
+  // one limit for every launch: host threads set it concurrently, and a launch's own size could
+  // undercut another thread's launch
+  LR_CUDA(cudaFuncSetAttribute(k_ozgemm<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem(S, false)));
+  k_ozgemm<S><<<grid, 32 * (epi_warps(S) + 2), gemm_smem(S, in_ring), s>>>(mp, e, t, c, ntiles, err, stall_ns, in_ring);
 }
 
 }  // namespace
@@ -925,12 +1002,12 @@ long long gemm_multi(const std::vector<std::pair<const Sliced *, const Sliced *>
   if (ops.empty()) return 0;
   const int S = ops[0].first->S;
   for (const auto &o : ops)
-    if (o.first->S != S || o.second->S != S || S < 0 || (S > SMAX && S != S_TF32 && S != S_TF32X3))
+    if (o.first->S != S || o.second->S != S || S < 0 || S > S_WIDE)
       throw Error{LIBRPA_E_ARG, "oz::gemm: operand mismatch"};
   init();
   // tiles with their K range in stages; MMA flops issued: per tile BM x BN x (K rounded up to the
   // K step) per digit-plane product
-  const double prods = (S == 0 || S == S_TF32) ? 1.0 : S == S_TF32X3 ? 3.0 : S * (S + 1) / 2.0;
+  const double prods = is_digits(S) ? S * (S + 1) / 2.0 : S == S_TF32X3 ? 3.0 : 1.0;
   const int ks = elem_bytes(S) == 4 ? PBK / 2 : PBK;   // K elements per pipeline stage
   std::vector<std::pair<int, Tile>> tk;
   std::vector<int> chunks, cl;
@@ -1008,13 +1085,12 @@ long long gemm_multi(const std::vector<std::pair<const Sliced *, const Sliced *>
   // forms), one CTA per tile, so that several CTAs per SM hide each other's TMA waits and
   // epilogues; with 4 or 5 planes only one CTA fits, and a persistent grid of one CTA per SM, its
   // ring running on across tiles, was measured faster on GB300 (3.5 % on the chi0 GEMMs).
-  const int ring = NST * planes(S) * (BM + BN) * 64;
   int nsm = 0;
   LR_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h.opts.device));
-  const int nt = (int)tk.size(), grid = 2 * (ring + 1024) > 227 * 1024 ? std::min(nt, nsm) : nt;
+  const int nt = (int)tk.size(), grid = 2 * (ring_bytes(S) + 1024) > 227 * 1024 ? std::min(nt, nsm) : nt;
   // testing only: the handle's first opts.test_stall_gemms launches take the failure path
   uint64_t stall = 0;
-  if (h.stalls_left > 0) {
+  if (h.stalls_left > 0 && S != S_WIDE) {
     --h.stalls_left;
     stall = 100000;   // 100 us per CTA
   }
@@ -1024,6 +1100,7 @@ long long gemm_multi(const std::vector<std::pair<const Sliced *, const Sliced *>
     case 2: launch<2>(dm, de, dt, dc, nt, grid, err, stall, s); break;
     case 3: launch<3>(dm, de, dt, dc, nt, grid, err, stall, s); break;
     case 4: launch<4>(dm, de, dt, dc, nt, grid, err, stall, s); break;
+    case S_WIDE: launch<S_WIDE>(dm, de, dt, dc, nt, grid, err, stall, s); break;
     case S_TF32: launch<S_TF32>(dm, de, dt, dc, nt, grid, err, stall, s); break;
     case S_TF32X3: launch<S_TF32X3>(dm, de, dt, dc, nt, grid, err, stall, s); break;
     default: launch<5>(dm, de, dt, dc, nt, grid, err, stall, s); break;

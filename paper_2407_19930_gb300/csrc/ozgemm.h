@@ -6,7 +6,9 @@
 // diagonal accumulates in its own FP32 TMEM accumulator, which is exact while |sum| < 2^24
 // (<= 1024 / (pairs of the diagonal) products of K).  Accumulators are flushed into exact int64
 // register sums and scaled to FP64 once at the end.  S = 5 keeps 39 bits per operand (relative
-// product error ~1e-12); S = 1..3 give the BF16 / split-precision ladder.  Two plain forms
+// product error ~1e-12); S = 1..3 give the BF16 / split-precision ladder; S = 8 keeps 63 bits (every
+// bit of an FP64 element within 2^-10 of its row's largest), the products of the FP64 mode.  A row
+// holding an infinity or a NaN makes its outputs NaN.  Two plain forms
 // take one plane of values rounded per element and accumulate in FP32 over all K: S = 0 (BF16,
 // kind::f16) and S = S_TF32 (TF32 in FP32 containers, kind::tf32).
 #pragma once
@@ -26,8 +28,11 @@ namespace oz {
 
 // S_TF32: one plane of TF32 values; S_TF32X3: two planes hi = tf32(x), lo = tf32(x - hi) and the
 // three products hi hi + hi lo + lo hi summed in one FP32 accumulator (the "3xTF32" split)
-constexpr int BM = 128, BN = 64, BK = 64, SMAX = 5, S_TF32 = 6, S_TF32X3 = 7;
-inline int planes(int S) { return S >= 1 && S <= SMAX ? S : S == S_TF32X3 ? 2 : 1; }
+// S_WIDE: 8 digit planes (63 bits per operand, below the rounding of FP64), whose diagonal sums are
+// carried in two int64 words: the products of the FP64 mode
+constexpr int BM = 128, BN = 64, BK = 64, SMAX = 5, S_TF32 = 6, S_TF32X3 = 7, S_WIDE = 8;
+__host__ __device__ constexpr bool is_digits(int S) { return (S >= 1 && S <= SMAX) || S == S_WIDE; }
+__host__ __device__ constexpr int planes(int S) { return is_digits(S) ? S : S == S_TF32X3 ? 2 : 1; }
 inline int elem_bytes(int S) { return S == S_TF32 || S == S_TF32X3 ? 4 : 2; }
 
 // K-major sliced operand: digit planes [S][rows][kpad] (BF16; FP32 for S_TF32) and row exponents
@@ -38,7 +43,7 @@ struct Sliced {
   int rows = 0;     // total rows
   int K = 0;        // logical K (columns beyond K and up to kpad hold zero digits)
   int kpad = 0;     // row pitch in elements (K rounded up to a multiple of 8)
-  int S = 0;        // digit planes 1..SMAX; 0 = one plane of plain BF16 values, S_TF32 = one plane
+  int S = 0;        // digit planes 1..SMAX or S_WIDE; 0 = one plane of plain BF16 values, S_TF32 = one plane
                     // of plain TF32 values (own exponent per element, rounded to nearest)
 };
 size_t sliced_bytes(int rows, int K, int S);   // bytes for digits + exponents (256-byte aligned parts)
