@@ -857,6 +857,10 @@ double dgemm_batched(Handle &h, const std::vector<DGemm> &batch, cudaStream_t s,
 
 }  // namespace
 
+// FP64 mode: requests whose contraction takes this many flops or more run on 8 digit planes on the
+// tensor cores, smaller ones on the FP64 pipes.
+constexpr double kWideMinFlops = 5e8;
+
 void chi0_shape(const Handle &h, Chi0Plan &P) {
   const int nat = h.natoms;
   P.natoms = nat;
@@ -940,7 +944,9 @@ void chi0_shape(const Handle &h, Chi0Plan &P) {
     P.cpnx_off[a + 1] = P.cpnx_off[a] + h.n_aux[a] * h.n_ao[a];
   }
   P.cpnx_rows = P.cpnx_off[nat];
-  P.tc_S = h.chi0_S;
+  // the FP64 mode: 8 digit planes, but for the smallest requests the FP64 pipes (see kWideMinFlops)
+  const double total = fl * h.ntau * (double)chi0_r_list(h.mesh).size();
+  P.tc_S = h.chi0_S >= 0 ? h.chi0_S : total >= kWideMinFlops ? oz::S_WIDE : -1;
 }
 
 void chi0_plan(Handle &h) {
@@ -1078,7 +1084,7 @@ bool run_oassemble(Handle &h, const Point *dpts, int np, double *Nw, double *Xw,
   }
   // arithmetic: FP64 pipes for the FP64 mode, FP32 for the mixed modes, FP32 pairs (~48 bits)
   // for the FP64-accurate tensor-core mode
-  const int ar = h.chi0_S < 0 ? 0 : (h.chi0_S >= 4 && h.chi0_S <= oz::SMAX) ? 2 : 1;
+  const int ar = P.tc_S < 0 || P.tc_S == oz::S_WIDE ? 0 : (P.tc_S >= 4 && P.tc_S <= oz::SMAX) ? 2 : 1;
   const size_t esz = ar == 1 ? sizeof(float) : 8;
   int NL = 4;
   auto smem_for = [&](int nl) { return (size_t)(maxn * 2 * maxn + 2 * maxn * 64 + nl * maxn * 2 * maxn) * esz; };
@@ -1616,7 +1622,7 @@ struct TcWs {
 };
 
 TcWs tc_ws(const Handle &h, const Chi0Plan &P) {
-  const int nat = h.natoms, S = h.chi0_S;
+  const int nat = h.natoms, S = P.tc_S;
   const int rows_bg = 2 * nat * P.m_all, rows_ag = 2 * nat * h.nao, rows_o = nat * h.naux;
   const size_t fp = 8 * (size_t)(2 * P.n_sz + 2 * P.x_sz + P.o_sz);
   const size_t per_point = fp + oz::sliced_bytes(rows_bg, P.max_m, S) + oz::sliced_bytes(rows_ag, P.max_m, S) +
@@ -1681,8 +1687,8 @@ TcRound tc_views(Handle &h, long long *npb) {
   r.wod = r.wag + al(tw.b_ag);
   r.err = (int *)(r.wod + al(tw.b_od));
   LR_CUDA(cudaMemsetAsync(r.err, 0, 4, h.stream));
-  oz::sliced_bind(r.cpnx, P.cp_nx.p, P.cpnx_rows, P.max_m, h.chi0_S);
-  oz::sliced_bind(r.cpf, P.cp_f.p, h.naux, P.max_nm, h.chi0_S);
+  oz::sliced_bind(r.cpnx, P.cp_nx.p, P.cpnx_rows, P.max_m, P.tc_S);
+  oz::sliced_bind(r.cpf, P.cp_f.p, h.naux, P.max_nm, P.tc_S);
   return r;
 }
 
@@ -1690,7 +1696,7 @@ TcRound tc_views(Handle &h, long long *npb) {
 // build the N- and X-step entries
 void tc_gather(Handle &h, TcRound &r) {
   Chi0Plan &P = h.plan;
-  const int nat = h.natoms, nR = h.mesh.size(), nao = h.nao, S = h.chi0_S;
+  const int nat = h.natoms, nR = h.mesh.size(), nao = h.nao, S = P.tc_S;
   const int np = r.np = (int)r.pts.size();
   cudaStream_t s = h.stream;
   h.upload_async(P.t_pts, r.pts.data(), np * sizeof(Point));
@@ -1718,10 +1724,9 @@ void tc_gather(Handle &h, TcRound &r) {
   gs.kind = 1;
   gs.rows_per_entry = nao;
   oz::split_gather(gs, np * rows_ag, P.max_m, r.sag, s);
-  // N-step: N_V = Cpack_V Bg_V^T;  X-step: X_V = Ag_V Cpack_V^T, both as FP32 pairs (hi, lo): the O
-  // assembly reads the pair (FP32-pair arithmetic) or its hi part (FP32 arithmetic)
-  const bool pairs = true;
-  (void)S;
+  // N-step: N_V = Cpack_V Bg_V^T;  X-step: X_V = Ag_V Cpack_V^T, as FP32 pairs (hi, lo) of which the O
+  // assembly reads both or the hi part, or as FP64 numbers (FP64 mode)
+  const bool pairs = S != oz::S_WIDE;
   r.en.clear();
   r.ex.clear();
   for (int q = 0; q < np; ++q)
@@ -1760,7 +1765,7 @@ void tc_assemble(Handle &h, TcRound &r, const unsigned char *zero) {
   const int nat = h.natoms, nR = h.mesh.size(), naux = h.naux, np = r.np;
   // the 3-plane kernel builds the row exponents when O is split into at most 3 digit planes (the
   // plain BF16 / TF32 operands have none)
-  int *rexp = h.chi0_S >= 1 && h.chi0_S <= 3 ? r.sod.expo : nullptr;
+  int *rexp = P.tc_S >= 1 && P.tc_S <= 3 ? r.sod.expo : nullptr;
   if (rexp) oz::expo_init(r.sod, np * nat * naux, h.stream);
   const bool expo_given = run_oassemble(h, (const Point *)P.t_pts.p, np, r.Nw, r.Xw, r.Ow, zero, rexp);
   std::vector<long long> off(np * nat);
@@ -1932,7 +1937,7 @@ void tc_merged(std::vector<Handle *> &hs) {
 
 void chi0_run(Handle &h, double *ms_gemm) {
   if (ms_gemm) *ms_gemm = 0;
-  if (h.chi0_S >= 0) {
+  if (h.plan.tc_S >= 0) {
     chi0_run_tc(h);
     return;
   }
@@ -2009,7 +2014,12 @@ void chi0_run(Handle &h, double *ms_gemm) {
   if (ms_gemm) *ms_gemm = 0;
 }
 
-bool chi0_run_merged(std::vector<Handle *> &hs, MergedChi0 &m) {
+bool chi0_run_merged(std::vector<Handle *> &all, MergedChi0 &m) {
+  // the handles on digit planes share their launches as the tensor-core modes' do, the small ones on the
+  // FP64 pipes share theirs, replayed from a graph
+  std::vector<Handle *> hs, wide;
+  for (Handle *h : all) (h->plan.tc_S >= 0 ? wide : hs).push_back(h);
+  if (!wide.empty()) tc_merged(wide);
   if (hs.empty()) return false;
   Handle &h0 = *hs[0];
   cudaStream_t s = h0.stream;
@@ -2157,9 +2167,9 @@ void MergedChi0::reset() {
 size_t chi0_device_bytes(const Handle &h, const Chi0Plan &P) {
   size_t b = (size_t)P.cp_total * 8;                                    // packed C
   b += (size_t)h.ntau * h.mesh.size() * h.naux * h.naux * 8;            // chi0(R, tau)
-  b += h.chi0_S >= 0 ? tc_ws(h, P).total : dp_ws(h, P).total;           // batch workspace
-  if (h.chi0_S >= 0)                                                    // digit planes of C
-    b += oz::sliced_bytes(P.cpnx_rows, P.max_m, h.chi0_S) + oz::sliced_bytes(h.naux, P.max_nm, h.chi0_S);
+  b += P.tc_S >= 0 ? tc_ws(h, P).total : dp_ws(h, P).total;             // batch workspace
+  if (P.tc_S >= 0)                                                      // digit planes of C
+    b += oz::sliced_bytes(P.cpnx_rows, P.max_m, P.tc_S) + oz::sliced_bytes(h.naux, P.max_nm, P.tc_S);
   // column tables and per-atom tables
   size_t cols = 0;
   for (int a = 0; a < h.natoms; ++a) cols += P.m[a];

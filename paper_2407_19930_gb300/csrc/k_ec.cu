@@ -643,6 +643,11 @@ void potrf_batched_r(Handle &h, double *const *d_mats, const std::vector<double 
   LR_CUDA(cudaGetLastError());
 }
 
+// digit planes of the ln det GEMMs: those of the mode, and 8 in the FP64 mode for matrices of order
+// kWideMinN or more (-1: the FP64 pipes)
+constexpr int kWideMinN = 96;
+int ec_planes(const Handle &h) { return h.ec_S >= 0 ? h.ec_S : h.naux >= kWideMinN ? oz::S_WIDE : -1; }
+
 size_t al256(size_t b) { return (b + 255) / 256 * 256; }
 
 // Workspace of the ln det stage: L[nq], W[nw], A[nw] (complex n x n), pointer tables,
@@ -662,7 +667,7 @@ int ec_chunk(const Handle &h) {
 }
 
 EcLayout ec_layout(const Handle &h) {
-  const int n = h.naux, nq = h.mesh.size(), nw = h.ntau, S = h.ec_S, nc = ec_chunk(h);
+  const int n = h.naux, nq = h.mesh.size(), nw = h.ntau, S = ec_planes(h), nc = ec_chunk(h);
   const size_t n2 = (size_t)n * n, mat = n2 * sizeof(double2);
   const int bmax = std::max(nq, nc * nw);
   EcLayout l;
@@ -700,7 +705,7 @@ EcLayout ec_layout(const Handle &h) {
 size_t ec_work_bytes(const Handle &h) { return ec_layout(h).total; }
 
 int ec_run(Handle &h, double *ec, double *ec_q, double *ec_w) {
-  const int n = h.naux, nq = h.mesh.size(), nw = h.ntau, S = h.ec_S;
+  const int n = h.naux, nq = h.mesh.size(), nw = h.ntau, S = ec_planes(h);
   const size_t n2 = (size_t)n * n;
   cudaStream_t s = h.stream;
   const size_t mat = n2 * sizeof(double2);

@@ -18,8 +18,10 @@
 namespace librpa {
 namespace {
 
-// digit planes of the G build in the tensor-core modes (FP64-accurate products)
-constexpr int kGreenS = 5;
+// digit planes of the G build: 5 in the tensor-core modes (FP64-accurate products), 8 in the FP64 mode
+// from kWideMinAo NAOs on (-1: the FP64 pipes)
+constexpr int kWideMinAo = 64;
+int green_planes(const Handle &h) { return h.chi0_S >= 0 ? 5 : h.nao >= kWideMinAo ? oz::S_WIDE : -1; }
 
 // Y[g][k][n][i] = sqrt(w[g][k][n]) c_in(k) (the weights are >= 0), so that P^g_k = Y^T conj(Y)
 __global__ void k_scale_bands(const double2 *wfc, const double *w, int nk, int nb, int nao, double2 *Y) {
@@ -143,9 +145,10 @@ size_t green_work_bytes(const Handle &h) {
   const size_t b_e = nk * nb * 8, b_w = 2 * b_e, b_p = 2 * nk * n2 * 16, b_t = nk * nR * 16;
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
   size_t b = al(b_w) + al(b_p) + al(b_t) + 256;
-  if (h.chi0_S >= 0)   // tensor-core modes: Y and the digit planes of both GEMM roles
-    b += al(b_p) + oz::sliced_bytes((int)(2 * nk * 2 * h.nao), (int)(2 * nb), kGreenS) +
-         oz::sliced_bytes((int)(2 * nk * h.nao), (int)(2 * nb), kGreenS) + 256;
+  const int S = green_planes(h);
+  if (S >= 0)   // digit planes: Y and the digit planes of both GEMM roles
+    b += al(b_p) + oz::sliced_bytes((int)(2 * nk * 2 * h.nao), (int)(2 * nb), S) +
+         oz::sliced_bytes((int)(2 * nk * h.nao), (int)(2 * nb), S) + 256;
   return b;
 }
 
@@ -160,19 +163,20 @@ double green_build(Handle &h) {
                b_t = (size_t)nk * nR * 16;
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
   const size_t o_w = 0, o_p = o_w + al(b_w), o_t = o_p + al(b_p), o_m = o_t + al(b_t);
-  // tensor-core modes: P^g_k = Y^T conj(Y) as one batched digit-plane GEMM per tau (FP64-accurate)
-  const bool tc = h.chi0_S >= 0;
+  // digit planes: P^g_k = Y^T conj(Y) as one batched digit-plane GEMM per tau (FP64-accurate)
+  const int S = green_planes(h);
+  const bool tc = S >= 0;
   const size_t o_y = o_m + 256, o_sa = o_y + al(b_p),
-               o_sb = o_sa + oz::sliced_bytes(2 * nk * 2 * nao, 2 * nb, kGreenS),
-               o_err = o_sb + oz::sliced_bytes(2 * nk * nao, 2 * nb, kGreenS);
+               o_sb = o_sa + oz::sliced_bytes(2 * nk * 2 * nao, 2 * nb, S),
+               o_err = o_sb + oz::sliced_bytes(2 * nk * nao, 2 * nb, S);
   h.ensure(h.work, green_work_bytes(h));
   char *wk = (char *)h.work.p;
   double2 *d_Y = tc ? (double2 *)(wk + o_y) : nullptr;
   int *d_err = tc ? (int *)(wk + o_err) : nullptr;
   oz::Sliced sa, sb;
   if (tc) {
-    oz::sliced_bind(sa, wk + o_sa, 2 * nk * 2 * nao, 2 * nb, kGreenS);
-    oz::sliced_bind(sb, wk + o_sb, 2 * nk * nao, 2 * nb, kGreenS);
+    oz::sliced_bind(sa, wk + o_sa, 2 * nk * 2 * nao, 2 * nb, S);
+    oz::sliced_bind(sb, wk + o_sb, 2 * nk * nao, 2 * nb, S);
     LR_CUDA(cudaMemsetAsync(d_err, 0, 4, s));
   }
   const double2 *d_wfc0 = (const double2 *)h.d_wfc.p;

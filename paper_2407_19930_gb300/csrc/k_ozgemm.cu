@@ -355,77 +355,55 @@ struct Tile {
 
 // ------------------------------------------------------------------ epilogue conversions
 // The FP64 pipe of GB300 runs at about 1/64 of its FP32 rate, so the epilogue builds its FP64 (and
-// FP32-pair) outputs from the exact int64 digit sums with integer instructions: normalise by the
+// FP32-pair) outputs from the exact integer digit sums with integer instructions: normalise by the
 // leading-one position, round to nearest even, and put the scale 2^sh into the exponent field.
-// Results outside the normal range take the FP64 route (rare).
+// Straight-line but for results outside the normal range (rare), so that a thread's sums interleave.
+
+// mant (53 bits, or 2^53 after rounding up) 2^(e - 1075) with e the biased exponent; neg: sign bit
+__device__ __forceinline__ double make_f64(unsigned long long neg, unsigned long long mant, int e) {
+  double v = __longlong_as_double((long long)(((unsigned long long)(e - 1) << 52) + mant));
+  if (e <= 0 || e >= 2046) {   // subnormal, overflow or next to it: scale [1, 2) in two exact steps
+    const int k = min(1100, max(-1080, e - 1023)), k1 = k / 2, k2 = k - k1;
+    v = __longlong_as_double((long long)((1022ull << 52) + mant));
+    v = v * __longlong_as_double((long long)(k1 + 1023) << 52) * __longlong_as_double((long long)(k2 + 1023) << 52);
+  }
+  return __longlong_as_double(__double_as_longlong(v) | (long long)neg);
+}
 
 // a 2^sh as FP64, rounded to nearest even
 __device__ __forceinline__ double i64_to_f64(long long a, int sh) {
-  if (a == 0) return 0.0;
-  const unsigned long long neg = a < 0 ? 0x8000000000000000ull : 0ull;
-  unsigned long long m = a < 0 ? 0ull - (unsigned long long)a : (unsigned long long)a;
-  const int lz = __clzll((long long)m);
-  m <<= lz;                                    // leading one at bit 63
-  unsigned long long mant = m >> 11;           // 53 significant bits
-  const unsigned rem = (unsigned)(m & 0x7FFull);
-  int e = 1086 - lz + sh;                      // biased exponent: 1023 + (63 - lz) + sh
-  if (rem > 0x400u || (rem == 0x400u && (mant & 1ull))) {
-    ++mant;
-    if (mant >> 53) {
-      mant >>= 1;
-      ++e;
-    }
-  }
-  if (e <= 0 || e >= 2047) return ldexp((double)a, sh);
-  return __longlong_as_double((long long)(neg | ((unsigned long long)e << 52) | (mant & 0xFFFFFFFFFFFFFull)));
-}
-
-// u 2^sh as FP32 (u < 2^63), rounded to nearest even; *ok = false outside the normal range
-__device__ __forceinline__ float u64_to_f32(unsigned long long u, int sh, bool *ok) {
-  if (u == 0) return 0.f;
+  const unsigned long long neg = (unsigned long long)a & 0x8000000000000000ull;
+  const unsigned long long u = (unsigned long long)(a < 0 ? -a : a);
   const int lz = __clzll((long long)u);
-  u <<= lz;
-  unsigned mant = (unsigned)(u >> 40);         // 24 significant bits
-  const unsigned long long rem = u & 0xFFFFFFFFFFull;
-  int e = 190 - lz + sh;                       // biased exponent: 127 + (63 - lz) + sh
-  if (rem > 0x8000000000ull || (rem == 0x8000000000ull && (mant & 1u))) {
-    ++mant;
-    if (mant >> 24) {
-      mant >>= 1;
-      ++e;
-    }
-  }
-  if (e <= 0 || e >= 255) {
-    *ok = false;
-    return 0.f;
-  }
-  return __uint_as_float(((unsigned)e << 23) | (mant & 0x7FFFFFu));
+  const unsigned long long m = u << (lz & 63);                         // leading one at bit 63
+  unsigned long long mant = m >> 11;                                   // 53 significant bits
+  mant += ((unsigned)(m & 0x7FFull) + 0x3FFu + (unsigned)(mant & 1ull)) >> 11;
+  const double v = make_f64(neg, mant, 1086 - lz + sh);                // biased exponent: 1023 + (63 - lz) + sh
+  return a == 0 ? 0.0 : v;
 }
 
 // a 2^sh as an unevaluated pair of FP32 numbers (hi, lo): hi = the value rounded to 24 bits, lo =
 // the remainder rounded to 24 bits (about 48 significant bits)
 __device__ __forceinline__ float2 i64_to_f32x2(long long a, int sh) {
-  if (a == 0) return make_float2(0.f, 0.f);
-  const bool neg = a < 0;
-  unsigned long long m = neg ? 0ull - (unsigned long long)a : (unsigned long long)a;
-  const int lz = __clzll((long long)m);
-  m <<= lz;                                    // leading one at bit 63; value = m 2^(sh - lz)
-  unsigned long long hm = m >> 40;
+  const unsigned neg = a < 0 ? 0x80000000u : 0u;
+  const unsigned long long u = (unsigned long long)(a < 0 ? -a : a);
+  const int lz = __clzll((long long)u);
+  const unsigned long long m = u << (lz & 63);                         // value = m 2^(sh - lz)
+  const unsigned hm = (unsigned)(m >> 40);                             // 24 significant bits
   long long r = (long long)(m & 0xFFFFFFFFFFull);
-  if (r > 0x8000000000ll || (r == 0x8000000000ll && (hm & 1ull))) {
-    ++hm;
-    r -= 0x10000000000ll;                      // the remainder of the rounded-up hi is negative
+  const unsigned up = (r > 0x8000000000ll || (r == 0x8000000000ll && (hm & 1u))) ? 1u : 0u;
+  r -= (long long)up << 40;                                            // the remainder of a rounded-up hi is negative
+  const int e = sh - lz;
+  float hi = __uint_as_float(((unsigned)(e + 189) << 23) + hm + up);   // biased exponent 127 + 63 + e, less the leading one
+  // r = rh 2^20 + rl, both exact in FP32: one rounding
+  float lo = fmaf((float)(int)(r >> 20), 1048576.f, (float)(int)(r & 0xFFFFFll)) * __uint_as_float((unsigned)(e + 127) << 23);
+  if (e < -126 || e > 63) {   // outside the FP32 range of a direct scaling: through FP64
+    const double v = i64_to_f64(a < 0 ? -a : a, sh);
+    hi = __double2float_rn(v);
+    lo = __double2float_rn(v - (double)hi);
   }
-  bool ok = true;
-  float hi = u64_to_f32(hm, sh - lz + 40, &ok);   // hm <= 2^24: exact
-  float lo = u64_to_f32((unsigned long long)(r < 0 ? -r : r), sh - lz, &ok);
-  if (!ok) {   // outside the FP32 normal range: through FP64
-    const double v = ldexp((double)a, sh);
-    const float h = __double2float_rn(v);
-    return make_float2(h, __double2float_rn(v - (double)h));
-  }
-  if (r < 0) lo = -lo;
-  return neg ? make_float2(-hi, -lo) : make_float2(hi, lo);
+  if (a == 0) hi = lo = 0.f;
+  return make_float2(__uint_as_float(__float_as_uint(hi) ^ neg), __uint_as_float(__float_as_uint(lo) ^ neg));
 }
 
 // (hi 2^32 + lo) 2^sh as FP64, rounded to nearest even (|hi|, |lo| < 2^62): the two words are carried
@@ -433,60 +411,46 @@ __device__ __forceinline__ float2 i64_to_f32x2(long long a, int sh) {
 __device__ __forceinline__ double i96_to_f64(long long hi, long long lo, int sh) {
   hi += lo >> 32;
   unsigned l = (unsigned)(unsigned long long)lo;
-  const bool neg = hi < 0;
+  const unsigned long long neg = (unsigned long long)hi & 0x8000000000000000ull;
   if (neg) {
     l = 0u - l;
     hi = l ? ~hi : -hi;
   }
+  // the leading one of the 96 bits: in hi, or (hi = 0) in l
   const unsigned long long h = (unsigned long long)hi;
-  if (h == 0) {
-    const double v = i64_to_f64((long long)l, sh);
-    return neg ? -v : v;
-  }
-  const int lz = __clzll((long long)h);
-  unsigned long long m = h << lz;   // leading one at bit 63 of the upper 64 of 96 bits
-  unsigned rest = 0;
-  if (lz <= 32) {
-    m |= (unsigned long long)l >> (32 - lz);
-    rest = lz < 32 ? l << lz : 0u;
-  } else {
-    m |= (unsigned long long)l << (lz - 32);
-  }
+  const int lz = h ? __clzll((long long)h) : 64 + __clz((int)l);
+  // x = the bits of (h : l : 0) below the first min(lz, 64) ones
+  unsigned long long m = h << (lz & 63);
+  const unsigned long long l64 = (unsigned long long)l << 32;
+  if (lz >= 64)
+    m = l64 << (lz - 64 & 63);
+  else
+    m |= lz ? l64 >> (64 - lz) : 0ull;
+  const unsigned rest = lz < 32 ? l << lz : 0u;   // bits of l below the leading 64
   unsigned long long mant = m >> 11;
-  const unsigned rem = (unsigned)(m & 0x7FFull);
-  int e = 1086 - lz + 32 + sh;
-  if (rem > 0x400u || (rem == 0x400u && (rest != 0u || (mant & 1ull)))) {
-    ++mant;
-    if (mant >> 53) {
-      mant >>= 1;
-      ++e;
-    }
-  }
-  if (e <= 0 || e >= 2047) {   // outside the normal range (rare)
-    const double v = ldexp((double)m, sh + 32 - lz);
-    return neg ? -v : v;
-  }
-  return __longlong_as_double(
-      (long long)((neg ? 0x8000000000000000ull : 0ull) | ((unsigned long long)e << 52) | (mant & 0xFFFFFFFFFFFFFull)));
+  mant += ((unsigned)(m & 0x7FFull) + 0x3FFu + ((unsigned)(mant & 1ull) | (rest ? 1u : 0u))) >> 11;
+  const double v = make_f64(neg, mant, 1086 + 32 - lz + sh);
+  return h == 0 && l == 0 ? 0.0 : v;
 }
 
-template <int S>
-__host__ __device__ constexpr uint32_t tmem_cols() {
-  return S * BN <= 64 ? 64 : S * BN <= 128 ? 128 : S * BN <= 256 ? 256 : 512;
-}
+__host__ __device__ constexpr uint32_t tmem_cols(int cols) { return cols <= 128 ? 128 : cols <= 256 ? 256 : 512; }
 constexpr uint64_t WAIT_NS = 2000000000ull;   // 2 s
 
 constexpr int PBK = 32;   // K per stage: one 64-byte swizzle row of BF16 (16 TF32 values)
-// pipeline depth: 3 stages (180 KB with 5 planes); 2 with more planes (8 planes: 96 KB a stage)
-__host__ __device__ constexpr int ring_stages(int S) { return S == S_WIDE ? 2 : 3; }
-// epilogue warps of the S variant
-__host__ __device__ constexpr int epi_warps(int S) { return is_digits(S) ? 8 : 4; }
-// columns the epilogue stages at a time, and bytes of its staging area: 16 columns of int64 sums, pitch
-// 17 (conflict-free by rows and by columns), or 4 columns of two-word sums, pitch 5
-__host__ __device__ constexpr int stage_cols(int S) { return S == S_WIDE ? 4 : 16; }
-__host__ __device__ constexpr int stage_bytes(int S) {
-  return is_digits(S) ? epi_warps(S) * 32 * (stage_cols(S) + 1) * (S == S_WIDE ? 16 : 8) : 0;
+// pipeline depth: what fits in the shared memory beside the staging area (180 KB with 3 or 5 planes, 192 KB
+// with 8)
+__host__ __device__ constexpr int ring_stages(int S) {
+  return S == S_WIDE ? 2 : S == 5 ? 3 : S == 4 ? 3 : S == 3 ? 5 : planes(S) == 2 ? 6 : 8;
 }
+// accumulator sets in TMEM: two where they fit (up to 4 planes), so that one is drained while the other fills
+__host__ __device__ constexpr int acc_sets(int S) { return !is_digits(S) || S <= 4 ? 2 : 1; }
+__host__ __device__ constexpr int acc_cols(int S) { return (is_digits(S) ? S : 1) * BN; }
+// epilogue warps of the S variant
+__host__ __device__ constexpr int epi_warps(int S) { return is_digits(S) ? 16 : 4; }
+// columns the epilogue stages at a time (what the shared memory beside the ring holds), pitch + 1, and the
+// bytes of its staging area
+__host__ __device__ constexpr int stage_cols(int S) { return S == S_WIDE ? 4 : 8; }
+__host__ __device__ constexpr int stage_bytes(int S) { return is_digits(S) ? epi_warps(S) * 32 * (stage_cols(S) + 1) * 8 : 0; }
 // digit planes of B multiplied by one MMA: at most 256 columns
 constexpr int kStack = 256 / BN;
 
@@ -514,25 +478,24 @@ struct alignas(128) MapPair {
 
 // Pipelined, warp-specialised kernel: CTA c takes tiles c, c + gridDim.x, ... (128 x 64 output
 // tiles of the launch's entries, sorted by decreasing K range on the host), keeping its barriers and
-// TMEM across them (one CTA per tile, or a persistent grid of one CTA per SM: see gemm_multi).
+// TMEM across them (a persistent grid of one CTA per SM).
 //   warp EW (one lane): TMA producer over a ring of NST shared-memory stages (each the NP digit
 //     planes of a 128 x 32 A slice and a 64 x 32 B slice, SWIZZLE_64B, K-major); the ring runs on
 //     across tiles, so the next tile's loads overlap this tile's MMAs and epilogue;
 //   warp EW + 1 (one lane): tcgen05.mma issuer; commits free a stage when its MMAs complete and, at
-//     the end of a flush group, signal the epilogue; the next group (of this or the next tile)
-//     starts once the epilogue has drained the accumulators.  The B planes lie one after the other in a
+//     the end of a flush group, signal the epilogue; the next group (of this or the next tile) uses the
+//     other accumulator set (up to 4 planes), or starts once the epilogue has drained the only one.  The B planes lie one after the other in a
 //     stage and the accumulators of consecutive diagonals in consecutive columns, so plane s of A
 //     meets up to four planes of B in one MMA of N = 256: 6 MMAs per K step of 16 with 5 planes in place of 15
 //     of N = 64, and A read from shared memory 6 times instead of 15 (54 KB a step, below what the
 //     MMAs' 480 cycles can take; at N = 64 the 90 KB held the tensor pipe at two thirds);
-//   warps 0..EW-1: epilogue; warp w owns TMEM lanes 32 (w % 4) .. + 31 (= tile rows).  With EW = 8
-//     (digit planes) warp w takes columns 32 (w / 4) .. + 31 and after each flush group moves the
-//     diagonal accumulators into exact int64 register sums (32 per thread, two words each with 8
+//   warps 0..EW-1: epilogue; warp w owns TMEM lanes 32 (w % 4) .. + 31 (= tile rows).  With EW = 16
+//     (digit planes) warp w takes columns 16 (w / 4) .. + 15 and after each flush group moves the
+//     diagonal accumulators into exact int64 register sums (16 per thread, of two words each with 8
 //     planes); with EW = 4 (plain BF16 / TF32, one group) each warp takes all 64 columns into
 //     registers.  The TMEM columns go back to the issuer before the values are converted and stored, so
-//     conversion and stores overlap the next tile's MMAs.  The sums go through a per-warp staging area into
-//     short rolled loops that convert and store: the conversion is ~50 instructions, and unrolled over
-//     a thread's 32 sums it ran from outside the instruction cache.
+//     conversion and stores overlap the next tile's MMAs.  The conversion (~30 integer instructions) is
+//     bound by its latency: four warps per scheduler, 16 independent sums each.
 // stall_ns > 0 (testing only): the MMA issuer first waits that long on an mbarrier nothing arrives
 // at, so the CTA takes the bounded-wait failure path.  On any failure the CTA sets *err, stops
 // issuing, waits (with the full limit) for the TMA copies and MMAs it has already issued, frees its
@@ -553,9 +516,11 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
   // forms accumulate over the whole K in FP32
   constexpr int G = PLAIN ? (1 << 30) : 32 / NP;
   constexpr int EPI_WARPS = epi_warps(S), HALF = BN * 4 / EPI_WARPS;   // HALF: columns per epilogue warp
-  constexpr uint32_t TMEM_COLS = tmem_cols<PLAIN ? 1 : NP>();
+  constexpr int SETS = acc_sets(S);                    // accumulator sets, one flush group each
+  constexpr uint32_t SET_COLS = acc_cols(S), TMEM_COLS = tmem_cols(SETS * acc_cols(S));
+  static_assert(SETS * acc_cols(S) <= 512, "k_ozgemm: TMEM");
   extern __shared__ uint8_t smem_raw[];
-  __shared__ uint64_t full[NST], empty[NST], tfull, tempty, mdone, never;
+  __shared__ uint64_t full[NST], empty[NST], tfull[SETS], tempty[SETS], mdone, never;
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -569,8 +534,11 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
-    mbar_init(&tfull, 1);
-    mbar_init(&tempty, EPI_WARPS);
+#pragma unroll
+    for (int b = 0; b < SETS; ++b) {
+      mbar_init(&tfull[b], 1);
+      mbar_init(&tempty[b], EPI_WARPS);
+    }
     mbar_init(&mdone, 1);
     mbar_init(&never, 1);
     abort_flag = 0;
@@ -633,8 +601,9 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
         const int nsteps = steps_of(entries[tl.e], tl, kbeg);
         for (int i = 0; i < nsteps; ++i, ++it) {
           const int st = (int)(it % NST), c = i % G;
-          // a new group needs the accumulators drained by the epilogue (previous group, any tile)
-          if (c == 0 && g > 0 && (abort_flag || !mbar_wait(&tempty, (uint32_t)((g - 1) & 1), WAIT_NS, &abort_flag))) {
+          // a new group needs its accumulators drained by the epilogue (group g - SETS, any tile)
+          if (c == 0 && g >= SETS &&
+              (abort_flag || !mbar_wait(&tempty[g % SETS], (uint32_t)((g / SETS - 1) & 1), WAIT_NS, &abort_flag))) {
             abort_flag = 1;
             break;
           }
@@ -644,6 +613,7 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
           }
           tc_fence_after();
           const uint32_t sa = smem_u32(smem + st * STAGE), sb = sa + NP * A_BYTES;
+          const uint32_t tacc = tmem + (uint32_t)(g % SETS) * SET_COLS;
           if constexpr (PLAIN) {
             // one accumulator for all products: hi hi (and hi lo, lo hi of the 3xTF32 split)
 #pragma unroll
@@ -656,9 +626,9 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
                   const uint64_t db = smem_desc64(sb + (u - 1) * B_BYTES + 32 * j);
                   const uint32_t accum = (c == 0 && j == 0 && s == 1 && u == 1) ? 0u : 1u;
                   if constexpr (TF)
-                    umma_tf32(tmem, da, db, idesc(BN, true), accum);
+                    umma_tf32(tacc, da, db, idesc(BN, true), accum);
                   else
-                    umma(tmem, da, db, idesc(BN, false), accum);
+                    umma(tacc, da, db, idesc(BN, false), accum);
                 }
           } else {
             // plane s of A by planes u .. u + w - 1 of B (N = 64 w), into the diagonals s + u ..
@@ -671,12 +641,12 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
                   const int w = NP + 2 - s - u < kStack ? NP + 2 - s - u : kStack;
                   const uint64_t da = smem_desc64(sa + (s - 1) * A_BYTES + 32 * j);
                   const uint64_t db = smem_desc64(sb + (u - 1) * B_BYTES + 32 * j);
-                  umma(tmem + (uint32_t)(s + u - 2) * BN, da, db, idesc(BN * w, false), (c == 0 && j == 0 && s == 1) ? 0u : 1u);
+                  umma(tacc + (uint32_t)(s + u - 2) * BN, da, db, idesc(BN * w, false), (c == 0 && j == 0 && s == 1) ? 0u : 1u);
                 }
           }
           umma_commit(&empty[st]);
           if (c == G - 1 || i == nsteps - 1) {
-            umma_commit(&tfull);
+            umma_commit(&tfull[g % SETS]);
             ++g;
           }
         }
@@ -690,7 +660,7 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
     }
   } else {
     const int quad = warp & 3, half = warp >> 2;   // TMEM lane quadrant, column half
-    const uint32_t tbase = tmem + ((uint32_t)(32 * quad) << 16) + half * HALF;
+    const uint32_t tbase0 = tmem + ((uint32_t)(32 * quad) << 16) + half * HALF;
     long long g = 0;   // flush groups drained (all tiles)
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
       const Tile tl = tiles[t];
@@ -703,6 +673,11 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
       // diagonals in acch, in units of the fourth's, the last four in acc)
       long long acc[PLAIN ? 1 : HALF], acch[WIDE ? HALF : 1];
       uint32_t fa[PLAIN ? HALF : 1];   // plain forms: the FP32 accumulators
+      // FP32-pair outputs of a tile with a single flush group (the short-K GEMMs of the chi0 steps): the
+      // diagonal sums, integers below 2^24 times their powers of two, are summed into an unevaluated FP32
+      // pair by exact two-sums, held in the halves of acc -- FP32 arithmetic instead of the integer
+      // conversions
+      const bool fpath = !PLAIN && !WIDE && ngroups == 1 && en.mode == 3 && en.alpha_shift != kNoShift;
       if constexpr (!PLAIN) {
 #pragma unroll
         for (int j = 0; j < HALF; ++j) acc[j] = 0;
@@ -713,7 +688,8 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
       }
       bool ok_all = true;
       for (int gi = 0; gi < ngroups; ++gi, ++g) {
-        bool ok = !abort_flag && mbar_wait(&tfull, (uint32_t)(g & 1), WAIT_NS, &abort_flag);
+        bool ok = !abort_flag && mbar_wait(&tfull[g % SETS], (uint32_t)((g / SETS) & 1), WAIT_NS, &abort_flag);
+        const uint32_t tbase = tbase0 + (uint32_t)(g % SETS) * SET_COLS;
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) {
           abort_flag = 1;
@@ -722,30 +698,41 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
         }
         tc_fence_after();
         if constexpr (!PLAIN) {
-          // 16 columns of one diagonal at a time, the next load in flight while these are added
-          // (registers for one load only with the two-word sums)
-          constexpr int CB = HALF / 16, NL = S * CB, RB = WIDE ? 1 : 2;
+          // one diagonal at a time, the next load in flight while this one is added
+          constexpr int CB = HALF / 16, RB = WIDE ? 1 : 2;
           uint32_t r[RB][16];
           if (!WIDE) tmem_ld16(tbase, r[0]);
 #pragma unroll
-          for (int l = 0; l < NL; ++l) {
-            const int d = l / CB, cb = l % CB;
-            if (WIDE) tmem_ld16(tbase + (uint32_t)d * BN + cb * 16, r[0]);
+          for (int l = 0; l < S * CB; ++l) {
+            const int d = l / CB, cb = l % CB * 16;
+            if (WIDE) tmem_ld16(tbase + (uint32_t)d * BN + cb, r[0]);
             tmem_ld_wait(r[l % RB]);
-            if (!WIDE && l + 1 < NL)
-              tmem_ld16(tbase + (uint32_t)((l + 1) / CB) * BN + ((l + 1) % CB) * 16, r[(l + 1) % RB]);
+            if (!WIDE && l + 1 < S * CB)
+              tmem_ld16(tbase + (uint32_t)((l + 1) / CB) * BN + (l + 1) % CB * 16, r[(l + 1) % RB]);
+            if (!WIDE && fpath) {
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const float t = __uint_as_float(r[l % RB][j]) * (float)(1ull << (8 * (S - 1 - d)));   // exact
+                const float hi = __int_as_float((int)(acc[cb + j] & 0xFFFFFFFFll));
+                float lo = __int_as_float((int)(acc[cb + j] >> 32));
+                const float sm = hi + t, bb = sm - hi;
+                lo += (hi - (sm - bb)) + (t - bb);
+                acc[cb + j] = ((long long)__float_as_int(lo) << 32) | (long long)(uint32_t)__float_as_int(sm);
+              }
+              continue;
+            }
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
               const int v = __float2int_rn(__uint_as_float(r[l % RB][j]));
               if constexpr (WIDE) {
                 if (d < 4)
-                  acch[cb * 16 + j] += (long long)v * (1 << (8 * (3 - d)));
+                  acch[cb + j] += (long long)v * (1 << (8 * (3 - d)));
                 else
-                  acc[cb * 16 + j] += (long long)v * (1 << (8 * (7 - d)));
+                  acc[cb + j] += (long long)v * (1 << (8 * (7 - d)));
               } else if (S == 5 && d == 0) {
-                acc[cb * 16 + j] += (long long)((unsigned long long)(unsigned)v << 32);   // 2^32 v (mod 2^64)
+                acc[cb + j] += (long long)((unsigned long long)(unsigned)v << 32);   // 2^32 v (mod 2^64)
               } else {
-                acc[cb * 16 + j] += (long long)v * (1 << (8 * (S - 1 - d) % 32));
+                acc[cb + j] += (long long)v * (1 << (8 * (S - 1 - d) % 32));
               }
             }
           }
@@ -761,7 +748,7 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&tempty);   // the accumulators may be overwritten now
+        if (lane == 0) mbar_arrive(&tempty[g % SETS]);   // the accumulators may be overwritten now
       }
       if (!ok_all) break;
       const int eM = en.M, eN = en.N, mode = en.mode;
@@ -771,13 +758,11 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
       const bool pow2 = en.alpha_shift != kNoShift;   // alpha = +-2^alpha_shift: folded into the exponent
       const int row = m0 + 32 * quad + lane;          // thread = tile row (the TMEM lane layout)
       const bool row_ok = row < eM;
-      // one output element (modes 0, 1, 2, 4)
-      auto store = [&](int r_, int c_, double v) {
-        double *p = mode == 0   ? C + (long long)r_ * ldc + c_
-                    : mode == 1 ? C + 2 * ((long long)(r_ >> 1) * ldc + c_) + (r_ & 1)
-                    : mode == 4 ? C + (long long)c_ * ldc + r_
-                                : C + 2 * ((long long)c_ * ldc + (r_ >> 1)) + (r_ & 1);
-        *p = beta == 0.0 ? v : v + beta * *p;
+      auto at = [&](int r_, int c_) {   // one output element (modes 0, 1, 2, 4)
+        return mode == 0   ? C + (long long)r_ * ldc + c_
+               : mode == 1 ? C + 2 * ((long long)(r_ >> 1) * ldc + c_) + (r_ & 1)
+               : mode == 4 ? C + (long long)c_ * ldc + r_
+                           : C + 2 * ((long long)c_ * ldc + (r_ >> 1)) + (r_ & 1);
       };
       if constexpr (PLAIN) {
         // plain forms: one FP32 sum per element, scaled in FP64 and stored from the registers,
@@ -799,90 +784,112 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
                   make_float2(hi, __double2float_rn(v - (double)hi));
               continue;
             }
-            store(row, col, v);
+            double *p = at(row, col);
+            *p = beta == 0.0 ? v : v + beta * *p;
           }
         }
       } else {
         constexpr int SC = stage_cols(S);
+        const int cbase = n0 + half * HALF, nc = min(HALF, eN - cbase);   // nc: live columns of the warp
+        if (nc <= 0) continue;
         const MapPair &mp = maps[en.pair];
-        const int ea = row_ok ? mp.ea[en.a_row0 + row] : 0;
-        const int *eb = mp.eb + en.b_row0;
         const int ash = (pow2 ? en.alpha_shift : 0) - 14 - 8 * (S - 1);
+        const int ea = (row_ok ? mp.ea[en.a_row0 + row] : 0) + ash;
+        const int *eb = mp.eb + en.b_row0 + cbase;
         const bool aneg = pow2 && alpha < 0.0;
-        const int cbase = n0 + half * HALF;
-        // value of a sum: its scale from the row's and the column's exponents; a row or column with an
-        // infinity or a NaN (exponent 1025) gives NaN
-        auto value = [&](long long hi, long long lo, int e_a, int e_b) {
-          const int sh = e_a + e_b + ash;
-          double v;
-          if constexpr (WIDE)
-            v = i96_to_f64(aneg ? -hi : hi, aneg ? -lo : lo, sh);
-          else
-            v = i64_to_f64(aneg ? -lo : lo, sh);
-          if (!pow2) v *= alpha;
-          return e_a > 1024 || e_b > 1024 ? __longlong_as_double(0x7FF8000000000000ll) : v;
-        };
-        long long *stg = reinterpret_cast<long long *>(stage_out + (size_t)warp * (stage_bytes(S) / EPI_WARPS));
+        // a row or column with an infinity or a NaN has the exponent 1025 (finite ones at most 1024)
+        const bool row_nan = ea - ash > 1024;
+        // the values in place of the sums: FP64 bits, or (mode 3) the pair (hi, lo)
+#pragma unroll
+        for (int j = 0; j < HALF; ++j) {
+          const int e_b = j < nc ? eb[j] : 0, sh = ea + e_b;
+          float2 pr;
+          if (fpath) {
+            // renormalise the pair, then scale it by 2^sh (exact in the normal range)
+            float hi = __int_as_float((int)(acc[j] & 0xFFFFFFFFll)), lo = __int_as_float((int)(acc[j] >> 32));
+            const float sm = hi + lo;
+            lo = lo - (sm - hi);
+            hi = sm;
+            const int eh = (int)((__float_as_uint(hi) >> 23) & 0xFF);
+            const float sc = __uint_as_float((uint32_t)(sh + 127) << 23);
+            pr = make_float2(hi * sc, lo * sc);
+            if (!(sh >= -126 && sh <= 127 && (hi == 0.f || (eh + sh >= 1 && eh + sh <= 254)))) {
+              const double dv = ldexp((double)hi + (double)lo, sh);   // outside the FP32 range: through FP64
+              pr.x = __double2float_rn(dv);
+              pr.y = __double2float_rn(dv - (double)pr.x);
+            }
+            if (aneg) pr = make_float2(-pr.x, -pr.y);
+          } else if (!WIDE && mode == 3 && pow2) {
+            pr = i64_to_f32x2(aneg ? -acc[j] : acc[j], sh);
+          } else {
+            double v;
+            if constexpr (WIDE)
+              v = i96_to_f64(acch[j], acc[j], sh);
+            else
+              v = i64_to_f64(acc[j], sh);
+            if (!pow2)
+              v *= alpha;
+            else if (aneg)
+              v = -v;
+            if (row_nan || e_b > 1024) v = __longlong_as_double(0x7FF8000000000000ll);
+            acc[j] = __double_as_longlong(v);
+            if (mode == 3) {
+              pr.x = __double2float_rn(v);
+              pr.y = __double2float_rn(v - (double)pr.x);
+            }
+          }
+          if (mode == 3) {
+            if (row_nan || e_b > 1024) pr = make_float2(__uint_as_float(0x7FC00000u), 0.f);
+            acc[j] = (long long)(((unsigned long long)__float_as_uint(pr.y) << 32) | __float_as_uint(pr.x));
+          }
+        }
+        if (mode == 2 || mode == 4) {
+          // transposed outputs: consecutive along the lanes (tile rows)
+          if (row_ok) {
+#pragma unroll
+            for (int j0 = 0; j0 < HALF; j0 += 8) {
+              double old[8];
+              if (beta != 0.0) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                  if (j0 + j < nc) old[j] = *at(row, cbase + j0 + j);
+              }
+#pragma unroll
+              for (int j = 0; j < 8; ++j)
+                if (j0 + j < nc) {
+                  const double v = __longlong_as_double(acc[j0 + j]);
+                  *at(row, cbase + j0 + j) = beta == 0.0 ? v : v + beta * old[j];
+                }
+            }
+          }
+          continue;
+        }
+        // row-major outputs: through the staging area, lanes along SC columns of 32 / SC rows
+        long long *stg = reinterpret_cast<long long *>(stage_out) + warp * 32 * (SC + 1);
+        const int cl = lane % SC, rl = lane / SC, rbase = m0 + 32 * quad + rl;
 #pragma unroll
         for (int cb = 0; cb < HALF / SC; ++cb) {
-          const int col0 = cbase + cb * SC;
-          if (col0 >= eN) break;   // the same for the whole warp
+          if (cb * SC >= nc) break;   // the same for the whole warp
+          const int col = cbase + cb * SC + cl;
+          const bool col_ok = cb * SC + cl < nc;
+          double old[SC];
+          if (beta != 0.0) {
 #pragma unroll
-          for (int j = 0; j < SC; ++j) {
-            if constexpr (WIDE)
-              reinterpret_cast<longlong2 *>(stg)[lane * (SC + 1) + j] = make_longlong2(acch[cb * SC + j], acc[cb * SC + j]);
-            else
-              stg[lane * (SC + 1) + j] = acc[cb * SC + j];
+            for (int i = 0; i < SC; ++i)
+              if (col_ok && rbase + i * (32 / SC) < eM) old[i] = *at(rbase + i * (32 / SC), col);
           }
+#pragma unroll
+          for (int j = 0; j < SC; ++j) stg[lane * (SC + 1) + j] = acc[cb * SC + j];
           __syncwarp();
-          if (WIDE || mode == 2 || mode == 4) {
-            // thread = tile row: the transposed outputs are consecutive along the lanes; with the two-word sums
-            // a lane writes 4 columns, one 32-byte sector of a row-major output
-            const int nc = min(SC, eN - col0);
-            if (row_ok) {
-#pragma unroll 1
-              for (int j = 0; j < nc; ++j) {
-                double v;
-                if constexpr (WIDE) {
-                  const longlong2 a = reinterpret_cast<const longlong2 *>(stg)[lane * (SC + 1) + j];
-                  v = value(a.x, a.y, ea, eb[col0 + j]);
-                } else {
-                  v = value(0, stg[lane * (SC + 1) + j], ea, eb[col0 + j]);
-                }
-                if (WIDE && mode == 3) {
-                  const float h = __double2float_rn(v);
-                  reinterpret_cast<float2 *>(C)[(long long)row * ldc + col0 + j] =
-                      make_float2(h, __double2float_rn(v - (double)h));
-                } else {
-                  store(row, col0 + j, v);
-                }
-              }
-            }
-          } else {
-            // lanes along the columns: two rows of 16 columns per store
-            const int cl = lane & 15, col = col0 + cl;
-            const int e_b = col < eN ? eb[col] : 0;
-#pragma unroll 2
-            for (int r2 = 0; r2 < 32; r2 += 2) {
-              const int rr = r2 + (lane >> 4), grow = m0 + 32 * quad + rr;
-              const int e_a = __shfl_sync(0xffffffffu, ea, rr);
-              if (grow < eM && col < eN) {
-                const long long a = stg[rr * (SC + 1) + cl];
-                if (mode == 3) {
-                  float2 pr;
-                  if (pow2 && e_a <= 1024 && e_b <= 1024) {
-                    pr = i64_to_f32x2(aneg ? -a : a, e_a + e_b + ash);
-                  } else {
-                    const double v = value(0, a, e_a, e_b);
-                    pr.x = __double2float_rn(v);
-                    pr.y = __double2float_rn(v - (double)pr.x);
-                  }
-                  reinterpret_cast<float2 *>(C)[(long long)grow * ldc + col] = pr;
-                } else {
-                  store(grow, col, value(0, a, e_a, e_b));
-                }
-              }
-            }
+#pragma unroll
+          for (int i = 0; i < SC; ++i) {
+            const int rr = rl + i * (32 / SC), grow = rbase + i * (32 / SC);
+            if (!col_ok || grow >= eM) continue;
+            const double v = __longlong_as_double(stg[rr * (SC + 1) + cl]);
+            if (mode == 3)   // the 8 bytes hold the pair (hi, lo)
+              C[(long long)grow * ldc + col] = v;
+            else
+              *at(grow, col) = beta == 0.0 ? v : v + beta * old[i];
           }
           __syncwarp();
         }
@@ -1081,13 +1088,11 @@ long long gemm_multi(const std::vector<std::pair<const Sliced *, const Sliced *>
   const Entry *de = (const Entry *)((const char *)args.p + off1);
   const Tile *dt = (const Tile *)((const char *)args.p + off2);
   const int *dc = (const int *)((const char *)args.p + off3);
-  // Grid: when two CTAs' stages fit in an SM's shared memory (fewer than 4 digit planes, the plain
-  // forms), one CTA per tile, so that several CTAs per SM hide each other's TMA waits and
-  // epilogues; with 4 or 5 planes only one CTA fits, and a persistent grid of one CTA per SM, its
-  // ring running on across tiles, was measured faster on GB300 (3.5 % on the chi0 GEMMs).
+  // a persistent grid of one CTA per SM (its shared memory and registers fill the SM): the ring and the
+  // accumulators run on across its tiles
   int nsm = 0;
   LR_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h.opts.device));
-  const int nt = (int)tk.size(), grid = 2 * (ring_bytes(S) + 1024) > 227 * 1024 ? std::min(nt, nsm) : nt;
+  const int nt = (int)tk.size(), grid = std::min(nt, nsm);
   // testing only: the handle's first opts.test_stall_gemms launches take the failure path
   uint64_t stall = 0;
   if (h.stalls_left > 0 && S != S_WIDE) {
