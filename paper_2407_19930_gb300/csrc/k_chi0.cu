@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "oasm.h"
 #include "ozgemm.h"
 
 namespace librpa {
@@ -141,10 +142,6 @@ using ChunkFn = std::function<bool(int, int, int, int, int, int, int, std::vecto
 
 // ---------------------------------------------------------------------------------------
 // gathers.  Column tables hold 6 ints per column: {atom, R0, R1, R2, orbital, ao(atom)+orbital}.
-struct Point {
-  int iR, itau;
-  int R[3];
-};
 
 // G of the spin channel being contracted ([spin][g][tau][R][i][j]) and the spin factor of chi0 per
 // channel: 2 for the single unpolarised channel, 1 per channel when nspins = 2 (chi0 = sum over
@@ -199,32 +196,8 @@ __global__ void k_gather_ag(const double *__restrict__ G, size_t g_gstride, cons
 }
 
 // ---------------------------------------------------------------------------------------
-// O assembly: O^nu_{ik}(K R1) for every (point, U, V), written as O_U[nu][(i, kap)].
-struct OArgs {
-  const double *G;       // [2][ntau][nR][nao][nao]
-  size_t g_gstride;
-  int nR_stride, nao, natoms, naux, n1, n2, n3;
-  const Point *pts;
-  const int *n_ao, *n_aux, *ao_off, *aux_off, *m;
-  const int *kap;            // per-U column table {K, R0, R1, R2, ao(K)+k, union column}
-  const long long *kap_off;
-  const double *N;           // [P][2][sum_V n_aux_V n_V M_all]
-  const long long *n_off;
-  long long n_sz_g, n_sz_p;
-  int m_all;
-  const double *X;           // [P][2][sum_V nao n_aux_V n_V]
-  const long long *x_off;
-  long long x_sz_g, x_sz_p;
-  double *O;                 // [P][sum_U naux n_U m_U]
-  const long long *o_off;
-  long long o_sz_p;
-  // under screening: 1 where the CTA's O block is exactly zero ([P][U][V][64-column chunk]), else NULL
-  const unsigned char *zero;
-  // 3-plane tensor-core kernel: the row exponents of O's digit planes (rows (p, U, nu); atomicMax
-  // of the largest biased FP64 exponent minus 1022), or NULL
-  int *rexp;
-};
-
+// O assembly (oasm.h) on the FP64 and FP32 pipes: requests below the digit-plane threshold of the FP64 mode,
+// and atoms with more NAOs than the tensor-core kernel takes.
 // Arithmetic of the O assembly.  ArD: FP64 (FP64 modes).  ArF: FP32, for the mixed modes whose
 // contraction GEMMs keep at most ~23 bits.  ArDF: unevaluated sums of two FP32 numbers (about 48
 // significant bits; the product of the high parts split exactly with an FMA, sums by Knuth's
@@ -379,361 +352,6 @@ __global__ void __launch_bounds__(256, 2) k_oassemble(OArgs a, int NL, const int
       for (int r = 0; r < ROWS; ++r)
         if (i0 + r < nU) orow[(size_t)(i0 + r) * mU + kc] = Ar::to(acc[r]);
     }
-  }
-}
-
-// ------------------------------------------------------------ O assembly on the tensor cores
-// The same O = M + M* + Z + Z* for the tensor-core modes, as exact digit-plane products on the
-// BF16 tensor cores (mma.sync m16n8k16, FP32 accumulators).  Per nu of V, O_nu[i][kc] is the sum
-// of two products over K = 2 n_V:
-//   term 1:  Lm[i][t] . Nt_nu[t][kc]   Lm = [A_UV(R) | B_UV(R)],  Nt = [N[G^occ]; N[G^vir]] at ucol(kc)
-//   term 2:  LX_nu[i][t] . RG[t][kc]   LX = [X^A_nu | X^B_nu] (rows of U),  RG = [B_{V,kap}; A_{V,kap}]
-// Each row of an A operand (i, over t) and each column of a B operand (kc, over t) is scaled by a
-// power of two 2^-E (E: its largest |value| < 2^E) and cut into S balanced base-256 digits
-// x = sum_s d_s 2^{-7-8(s-1)}, |d_s| <= 128 (exact in BF16); the digit products of one diagonal
-// s + t are summed exactly on the tensor cores (|sum| <= 5 * 32 * 2^14 < 2^22 for K <= 32), the
-// diagonals folded into one int64 per term, the two terms aligned to the larger scale and
-// converted to FP64 once.  Inputs: N and X as (hi, lo) FP32 pairs, G as FP64 turned into pairs;
-// the low part joins the digits after the second (error below 2^-39 of the row or column
-// maximum).  One CTA of 4 warps per (point, U, V, 64-column chunk of U); warp w owns columns
-// c0 + 16 w .. + 16 (two n8 tiles) and runs over every nu.  Needs n_U, n_V <= 16.
-constexpr int kTcKP = 40;   // row pitch of a digit plane in BF16 elements (80 bytes: ldmatrix rows
-                            // of 8 consecutive planes rows fall in distinct 16-byte bank groups)
-constexpr float kRintMagic = 12582912.0f;   // 1.5 * 2^23: (x + M) - M rounds |x| < 2^22 to an integer
-
-__host__ __device__ constexpr int oasm_tc_smem(int S) {
-  // Lm, LX [S][16][KP]; RG [S][64][KP]; N [4][S][16][KP] (BF16); exponents: e1[16], e2[16], f2[64], f1[4][16]
-  return (S * 16 * kTcKP * 2 + S * 64 * kTcKP + 4 * S * 16 * kTcKP) * 2 + (16 + 16 + 64 + 64) * 4;
-}
-
-// E with max |value| < 2^E from the largest |hi| (0 for an all-zero row), kept in [-100, 100]
-__device__ __forceinline__ int tc_expo(float m) {
-  if (!(m > 0.f)) return 0;
-  const int be = (__float_as_int(m) >> 23) & 0xff;
-  return min(100, max(-100, be - 126));
-}
-__device__ __forceinline__ float tc_pow2(int k) { return __int_as_float((k + 127) << 23); }   // |k| <= 126
-
-// S digits of (h + l) 2^-E into d[] (sc7 = 2^{7-E}, sc15 = 2^{15-E})
-template <int S>
-__device__ __forceinline__ void tc_digits(float h, float l, float sc7, float sc15, float *d) {
-  float t = h * sc7;
-  float dd = (t + kRintMagic) - kRintMagic;
-  float r = t - dd;
-  d[0] = dd;
-#pragma unroll
-  for (int s = 1; s < S; ++s) {
-    if (s == 2) r = fmaf(l, sc15, r);   // the low part, in units of the third digit
-    t = r * 256.f;
-    dd = (t + kRintMagic) - kRintMagic;
-    r = t - dd;
-    d[s] = dd;
-  }
-}
-
-__device__ __forceinline__ unsigned pack_bf16(float a, float b) {
-  __nv_bfloat162 v = __floats2bfloat162_rn(a, b);   // small integers: exact
-  return *reinterpret_cast<unsigned *>(&v);
-}
-__device__ __forceinline__ float2 g_pair(double v) {
-  const float h = __double2float_rn(v);
-  return make_float2(h, __double2float_rn(v - (double)h));
-}
-__device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void ldsm_x4(unsigned addr, unsigned &r0, unsigned &r1, unsigned &r2, unsigned &r3) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-               : "r"(addr));
-}
-__device__ __forceinline__ void mma_bf16(float *c, const unsigned *a, unsigned b0, unsigned b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-               "{%0,%1,%2,%3};\n"
-               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// Digit products of one term for the warp's two n8 tiles: A planes [S][16][KP] (rows i), B planes
-// [S][..][KP] (rows kc, from brow0), ks_n k-steps of 16; acc[d][nt][4] for the diagonals d = sa + sb.
-template <int S>
-__device__ __forceinline__ void tc_term(const __nv_bfloat16 *A, const __nv_bfloat16 *B, int bplane, int brow0,
-                                        int ks_n, int lane, float (*acc)[2][4]) {
-#pragma unroll
-  for (int d = 0; d < S; ++d)
-#pragma unroll
-    for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-      for (int r = 0; r < 4; ++r) acc[d][nt][r] = 0.f;
-  const int arow = lane & 15, acol = (lane >> 4) * 8;
-  const int brow = brow0 + (lane & 7) + ((lane >> 4) << 3), bcol = ((lane >> 3) & 1) * 8;
-  for (int ks = 0; ks < ks_n; ++ks) {
-    unsigned a[S][4], b[S][4];
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      ldsm_x4(smem_u32(A + (s * 16 + arow) * kTcKP + ks * 16 + acol), a[s][0], a[s][1], a[s][2], a[s][3]);
-      ldsm_x4(smem_u32(B + s * bplane + brow * kTcKP + ks * 16 + bcol), b[s][0], b[s][1], b[s][2], b[s][3]);
-    }
-#pragma unroll
-    for (int sa = 0; sa < S; ++sa)
-#pragma unroll
-      for (int sb = 0; sb < S - sa; ++sb) {
-        mma_bf16(acc[sa + sb][0], a[sa], b[sb][0], b[sb][1]);
-        mma_bf16(acc[sa + sb][1], a[sa], b[sb][2], b[sb][3]);
-      }
-  }
-}
-
-// sum_d A_d 2^{8(S-1-d)} of exact integer-valued FP32 diagonal sums (|A_d| < 2^22)
-template <int S>
-__device__ __forceinline__ long long tc_fold(const float *a) {
-  int v[S];
-#pragma unroll
-  for (int d = 0; d < S; ++d) v[d] = (int)((unsigned)__float_as_int(a[d] + kRintMagic) - 0x4B400000u);
-  if constexpr (S == 5) {   // v0 2^8 + v1 and v3 2^8 + v4 stay below 2^31
-    return ((long long)(v[0] * 256 + v[1]) << 24) + ((long long)v[2] << 16) + (long long)(v[3] * 256 + v[4]);
-  } else if constexpr (S == 3) {
-    return ((long long)v[0] << 16) + (long long)(v[1] * 256 + v[2]);
-  } else {
-    long long T = 0;
-#pragma unroll
-    for (int d = 0; d < S; ++d) T = T * 256 + v[d];
-    return T;
-  }
-}
-
-template <int S>
-__global__ void __launch_bounds__(128) k_oassemble_tc(OArgs a) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  __nv_bfloat16 *sLm = reinterpret_cast<__nv_bfloat16 *>(smraw);   // [S][16][KP]
-  __nv_bfloat16 *sLX = sLm + S * 16 * kTcKP;                        // [S][16][KP]
-  __nv_bfloat16 *sRG = sLX + S * 16 * kTcKP;                        // [S][64][KP]
-  __nv_bfloat16 *sN = sRG + S * 64 * kTcKP;                         // [4][S][16][KP]
-  int *sE1 = reinterpret_cast<int *>(sN + 4 * S * 16 * kTcKP);      // [16]
-  int *sE2 = sE1 + 16;                                              // [16]
-  int *sF2 = sE2 + 16;                                              // [64]
-  int *sF1 = sF2 + 64;                                              // [4][16]
-  const int V = blockIdx.y % a.natoms;
-  const int U = (blockIdx.y / a.natoms) % a.natoms;
-  const int p = blockIdx.y / (a.natoms * a.natoms);
-  const int mU = a.m[U];
-  const int c0 = blockIdx.x * 64;
-  if (c0 >= mU) return;
-  const int nU = a.n_ao[U], nV = a.n_ao[V], two = 2 * nV, nauxV = a.n_aux[V];
-  double *Ob = a.O + p * a.o_sz_p + a.o_off[U];
-  const int ldo = nU * mU;
-  if (a.zero && a.zero[((size_t)(p * a.natoms + U) * a.natoms + V) * gridDim.x + blockIdx.x]) {
-    const int w = min(64, mU - c0);
-    for (long long e = threadIdx.x; e < (long long)nauxV * nU * 64; e += blockDim.x) {
-      const int col = (int)(e % 64);
-      if (col >= w) continue;
-      const long long r = e / 64;
-      Ob[(size_t)(a.aux_off[V] + r / nU) * ldo + (size_t)(r % nU) * mU + c0 + col] = 0.0;
-    }
-    return;
-  }
-  const Point pt = a.pts[p];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const size_t n2 = (size_t)a.nao * a.nao;
-  const double *GB = a.G + ((size_t)pt.itau * a.nR_stride) * n2;                 // G^occ(tau)
-  const double *GA = a.G + a.g_gstride + ((size_t)pt.itau * a.nR_stride) * n2;   // G^vir(tau)
-  const int aoU = a.ao_off[U], aoV = a.ao_off[V];
-  const int ks_n = (two + 15) / 16;
-  // Lm digits (A of term 1): thread = (row i, 4 t); row exponent over the 8 lanes of the row
-  {
-    const int i = tid >> 3, t0 = (tid & 7) * 4;
-    float2 v[4];
-    float m = 0.f;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int t = t0 + q;
-      v[q] = make_float2(0.f, 0.f);
-      if (i < nU && t < two) {
-        const double *Gs = t < nV ? GA : GB;
-        v[q] = g_pair(Gs[((size_t)pt.iR) * n2 + (size_t)(aoU + i) * a.nao + aoV + (t < nV ? t : t - nV)]);
-      }
-      m = fmaxf(m, fabsf(v[q].x));
-    }
-    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
-    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
-    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 4));
-    const int E = tc_expo(m);
-    if ((tid & 7) == 0) sE1[i] = E;
-    const float sc7 = tc_pow2(7 - E), sc15 = tc_pow2(15 - E);
-    float d[4][S];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) tc_digits<S>(v[q].x, v[q].y, sc7, sc15, d[q]);
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      uint2 w2 = make_uint2(pack_bf16(d[0][s], d[1][s]), pack_bf16(d[2][s], d[3][s]));
-      *reinterpret_cast<uint2 *>(sLm + (s * 16 + i) * kTcKP + t0) = w2;
-    }
-  }
-  // RG digits (B of term 2, stored [kc][t]): thread = (column, 16 t); column exponent over 2 lanes
-  {
-    const int col = tid >> 1, t0 = (tid & 1) * 16;
-    const int kc = c0 + col;
-    const bool live = kc < mU;
-    const int *kp = a.kap + 6 * (a.kap_off[U] + (live ? kc : 0));
-    auto fold = [](int x, int nn) { int r = x % nn; return r < 0 ? r + nn : r; };
-    const int iR = (fold(kp[1] - pt.R[0], a.n1) * a.n2 + fold(kp[2] - pt.R[1], a.n2)) * a.n3 +
-                   fold(kp[3] - pt.R[2], a.n3);
-    float2 v[16];
-    float m = 0.f;
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const int t = t0 + q;
-      v[q] = make_float2(0.f, 0.f);
-      if (live && t < two) {
-        const double *Gs = t < nV ? GB : GA;
-        v[q] = g_pair(Gs[(size_t)iR * n2 + (size_t)(aoV + (t < nV ? t : t - nV)) * a.nao + kp[4]]);
-      }
-      m = fmaxf(m, fabsf(v[q].x));
-    }
-    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
-    const int E = tc_expo(m);
-    if ((tid & 1) == 0) sF2[col] = E;
-    const float sc7 = tc_pow2(7 - E), sc15 = tc_pow2(15 - E);
-#pragma unroll
-    for (int q0 = 0; q0 < 16; q0 += 8) {
-      float d[8][S];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) tc_digits<S>(v[q0 + q].x, v[q0 + q].y, sc7, sc15, d[q]);
-#pragma unroll
-      for (int s = 0; s < S; ++s) {
-        uint4 w4 = make_uint4(pack_bf16(d[0][s], d[1][s]), pack_bf16(d[2][s], d[3][s]), pack_bf16(d[4][s], d[5][s]),
-                              pack_bf16(d[6][s], d[7][s]));
-        *reinterpret_cast<uint4 *>(sRG + (s * 64 + col) * kTcKP + t0 + q0) = w4;
-      }
-    }
-  }
-  // this lane's column of the N operand: (column = lane & 15 of the warp's 16, t half = lane >> 4)
-  const int ncol = lane & 15, nt0 = (lane >> 4) * 16;
-  const int nkc = c0 + warp * 16 + ncol;
-  const bool nlive = nkc < mU;
-  const int ucol = a.kap[6 * (a.kap_off[U] + (nlive ? nkc : 0)) + 5];
-  const double *NB = a.N + p * a.n_sz_p + a.n_off[V];                 // N[G^occ]: g = 0
-  const double *NA = a.N + p * a.n_sz_p + a.n_sz_g + a.n_off[V];      // N[G^vir]: g = 1
-  const double *XB = a.X + p * a.x_sz_p + a.x_off[V];                 // X[G^occ]
-  const double *XA = a.X + p * a.x_sz_p + a.x_sz_g + a.x_off[V];      // X[G^vir]
-  const int ldx = nauxV * nV;
-  __nv_bfloat16 *sNw = sN + warp * S * 16 * kTcKP;
-  const int g = lane >> 2, tig = lane & 3;
-  for (int nu = 0; nu < nauxV; ++nu) {
-    // LX digits (A of term 2), shared by the 4 warps
-    {
-      const int i = tid >> 3, t0 = (tid & 7) * 4;
-      float2 v[4];
-      float m = 0.f;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int t = t0 + q;
-        v[q] = make_float2(0.f, 0.f);
-        if (i < nU && t < two)
-          v[q] = *reinterpret_cast<const float2 *>(t < nV ? XA + (size_t)(aoU + i) * ldx + nu * nV + t
-                                                          : XB + (size_t)(aoU + i) * ldx + nu * nV + (t - nV));
-        m = fmaxf(m, fabsf(v[q].x));
-      }
-      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
-      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
-      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 4));
-      const int E = tc_expo(m);
-      if ((tid & 7) == 0) sE2[i] = E;
-      const float sc7 = tc_pow2(7 - E), sc15 = tc_pow2(15 - E);
-      float d[4][S];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) tc_digits<S>(v[q].x, v[q].y, sc7, sc15, d[q]);
-#pragma unroll
-      for (int s = 0; s < S; ++s) {
-        uint2 w2 = make_uint2(pack_bf16(d[0][s], d[1][s]), pack_bf16(d[2][s], d[3][s]));
-        *reinterpret_cast<uint2 *>(sLX + (s * 16 + i) * kTcKP + t0) = w2;
-      }
-    }
-    // N digits (B of term 1) of the warp's 16 columns, stored [kc][t]
-    {
-      const double *Nn = NB + (size_t)nu * nV * a.m_all + ucol;
-      const double *Na = NA + (size_t)nu * nV * a.m_all + ucol;
-      float2 v[16];
-      float m = 0.f;
-#pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        const int t = nt0 + q;
-        v[q] = make_float2(0.f, 0.f);
-        if (nlive && t < two)
-          v[q] = *reinterpret_cast<const float2 *>(t < nV ? Nn + (size_t)t * a.m_all : Na + (size_t)(t - nV) * a.m_all);
-        m = fmaxf(m, fabsf(v[q].x));
-      }
-      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
-      const int E = tc_expo(m);
-      if (lane < 16) sF1[warp * 16 + ncol] = E;
-      const float sc7 = tc_pow2(7 - E), sc15 = tc_pow2(15 - E);
-#pragma unroll
-      for (int q0 = 0; q0 < 16; q0 += 8) {
-        float d[8][S];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) tc_digits<S>(v[q0 + q].x, v[q0 + q].y, sc7, sc15, d[q]);
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-          uint4 w4 = make_uint4(pack_bf16(d[0][s], d[1][s]), pack_bf16(d[2][s], d[3][s]),
-                                pack_bf16(d[4][s], d[5][s]), pack_bf16(d[6][s], d[7][s]));
-          *reinterpret_cast<uint4 *>(sNw + (s * 16 + ncol) * kTcKP + nt0 + q0) = w4;
-        }
-      }
-    }
-    __syncthreads();   // LX, N and (first pass) Lm, RG digits and exponents written
-    float acc[S][2][4];
-    long long T1[2][4];
-    tc_term<S>(sLm, sNw, 16 * kTcKP, 0, ks_n, lane, acc);
-#pragma unroll
-    for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        float av[S];
-#pragma unroll
-        for (int d = 0; d < S; ++d) av[d] = acc[d][nt][r];
-        T1[nt][r] = tc_fold<S>(av);
-      }
-    tc_term<S>(sLX, sRG, 64 * kTcKP, warp * 16, ks_n, lane, acc);
-    double *orow = Ob + (size_t)(a.aux_off[V] + nu) * ldo;
-    int emax = 0;   // largest biased exponent among this lane's stored outputs
-#pragma unroll
-    for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int i = g + (r >> 1) * 8, cw = nt * 8 + 2 * tig + (r & 1), kc = c0 + warp * 16 + cw;
-        float av[S];
-#pragma unroll
-        for (int d = 0; d < S; ++d) av[d] = acc[d][nt][r];
-        const long long T2 = tc_fold<S>(av);
-        const int E1 = sE1[i] + sF1[warp * 16 + cw], E2 = sE2[i] + sF2[warp * 16 + cw];
-        long long T;
-        int E;
-        if (E1 >= E2) {
-          const int sh = E1 - E2;
-          T = T1[nt][r] + (sh == 0 ? T2 : sh >= 62 ? 0 : (T2 + (1LL << (sh - 1))) >> sh);
-          E = E1;
-        } else {
-          const int sh = E2 - E1;
-          T = T2 + (sh >= 62 ? 0 : (T1[nt][r] + (1LL << (sh - 1))) >> sh);
-          E = E2;
-        }
-        double o = (double)T;
-        if (T != 0) {
-          const long long bits = __double_as_longlong(o);
-          const int k = E - 14 - 8 * (S - 1);
-          const int ex = (int)((bits >> 52) & 0x7ff) + k;
-          o = ex <= 0 ? 0.0 : __longlong_as_double(bits + ((long long)k << 52));
-        }
-        if (i < nU && kc < mU) {
-          orow[(size_t)i * mU + kc] = o;
-          emax = max(emax, (int)((__double_as_longlong(o) >> 52) & 0x7FF));
-        }
-      }
-    if (S < 4 && a.rexp) {   // the row (p, U, nu) of the final contraction's O operand
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, off));
-      if (lane == 0 && emax > 0)
-        atomicMax(a.rexp + ((size_t)p * a.natoms + U) * a.naux + a.aux_off[V] + nu, emax - 1022);
-    }
-    __syncthreads();   // every warp done with LX and the exponents before the next nu
   }
 }
 
@@ -949,6 +567,15 @@ void chi0_shape(const Handle &h, Chi0Plan &P) {
   P.tc_S = h.chi0_S >= 0 ? h.chi0_S : total >= kWideMinFlops ? oz::S_WIDE : -1;
 }
 
+// Digit planes of the O assembly on the tensor cores: 5 (~39 bits) for the FP64-accurate mode, 3 (~23 bits, as
+// FP32) for the mixed modes, 8 for the FP64 mode; 0 = the FP64 / FP32 pipes
+int oasm_planes(const Handle &h, const Chi0Plan &P) {
+  for (int n : h.n_ao)
+    if (n > oasm::kMaxAo) return 0;
+  if (P.tc_S < 0) return 0;
+  return P.tc_S == oz::S_WIDE ? oz::S_WIDE : P.tc_S == 4 || P.tc_S == 5 ? 5 : 3;
+}
+
 void chi0_plan(Handle &h) {
   Chi0Plan &P = h.plan;
   chi0_shape(h, P);
@@ -1019,6 +646,31 @@ void chi0_plan(Handle &h) {
     P.ugroup_off[4] = (int)ug.size();
     upload(h, P.t_ugroups, ug);
   }
+  if (oasm_planes(h, P) > 0) {
+    // O assembly on the tensor cores: U's packed columns in groups of up to 8 consecutive union columns,
+    // 16 groups to a tile
+    std::vector<oasm::Group> groups;
+    std::vector<int> toff(nat + 1, 0), aux_atom, ao_row;
+    P.oasm_max_tiles = 0;
+    for (int U = 0; U < nat; ++U) {
+      const size_t nb = P.nb[U].size();
+      for (size_t b = 0; b < nb;) {
+        const int u0 = P.nb[U][b].ucol, k0 = P.nb[U][b].col;
+        int len = 0;   // the run of neighbour blocks that are consecutive in the union as well
+        for (; b < nb && P.nb[U][b].ucol == u0 + len; ++b) len += h.n_ao[P.nb[U][b].K];
+        for (int x = 0; x < len; x += 8) groups.push_back({u0 + x, k0 + x, std::min(8, len - x)});
+      }
+      while (groups.size() % oasm::kTileGroups) groups.push_back({0, 0, 0});
+      toff[U + 1] = (int)groups.size() / oasm::kTileGroups;
+      P.oasm_max_tiles = std::max(P.oasm_max_tiles, toff[U + 1] - toff[U]);
+      for (int x = 0; x < h.n_aux[U]; ++x) aux_atom.push_back(U);
+      for (int i = 0; i < h.n_ao[U]; ++i) ao_row.push_back(U * oasm::kMaxAo + i);
+    }
+    upload(h, P.t_ogroups, groups);
+    upload(h, P.t_otiles, toff);
+    upload(h, P.t_aux_atom, aux_atom);
+    upload(h, P.t_ao_row, ao_row);
+  }
   // tensor-core route: digit planes of the packed coefficients, split once per plan
   if (P.tc_S >= 0) {
     const int S = P.tc_S;
@@ -1070,11 +722,16 @@ int oasm_chunks(const Handle &h) {
   return c;
 }
 
-// rexp (may be NULL): row exponents of the O operand's digit planes, built by atomicMax (initialised
-// to -1022) in the 3-plane tensor-core kernel only: in the 5-plane kernel the atomics cost more
-// than the exponent pass they save.  Returns true when the kernel that builds them ran.
+// Operands of the tensor-core O assembly: the digit planes of N and X (built by it), the row exponents of O's
+// own digit planes (built by atomicMax, initialised to -1022) and the error flag.
+struct OasmTc {
+  oz::Sliced *nd, *xd;
+  int *rexp, *err;
+};
+
+// Returns true when the row exponents of O's digit planes were built (tc given and the tensor-core kernel ran).
 bool run_oassemble(Handle &h, const Point *dpts, int np, double *Nw, double *Xw, double *Ow,
-                   const unsigned char *zero = nullptr, int *rexp = nullptr) {
+                   const unsigned char *zero = nullptr, const OasmTc *tc = nullptr) {
   Chi0Plan &P = h.plan;
   const int nat = h.natoms;
   int maxn = 0, max_chunks = 0;
@@ -1082,22 +739,6 @@ bool run_oassemble(Handle &h, const Point *dpts, int np, double *Nw, double *Xw,
     maxn = std::max(maxn, h.n_ao[a]);
     max_chunks = std::max(max_chunks, (P.m[a] + 63) / 64);
   }
-  // arithmetic: FP64 pipes for the FP64 mode, FP32 for the mixed modes, FP32 pairs (~48 bits)
-  // for the FP64-accurate tensor-core mode
-  const int ar = P.tc_S < 0 || P.tc_S == oz::S_WIDE ? 0 : (P.tc_S >= 4 && P.tc_S <= oz::SMAX) ? 2 : 1;
-  const size_t esz = ar == 1 ? sizeof(float) : 8;
-  int NL = 4;
-  auto smem_for = [&](int nl) { return (size_t)(maxn * 2 * maxn + 2 * maxn * 64 + nl * maxn * 2 * maxn) * esz; };
-  while (NL > 1 && smem_for(NL) > 200 * 1024) NL /= 2;
-  const size_t osmem = smem_for(NL);
-  // the limit is the same fixed bound for every handle: handles on other host threads (batched
-  // and serving workers) set it concurrently, and a per-handle value could undercut a launch
-  // in flight on another thread
-  constexpr int kOasmSmemLimit = 200 * 1024;
-  if (osmem > (size_t)kOasmSmemLimit) throw Error{LIBRPA_E_ARG, "O assembly: atoms with too many NAOs"};
-  set_oasm_smem_limits<ArD>(kOasmSmemLimit);
-  set_oasm_smem_limits<ArF>(kOasmSmemLimit);
-  set_oasm_smem_limits<ArDF>(kOasmSmemLimit);
   OArgs oa;
   oa.G = g_spin(h);
   oa.g_gstride = (size_t)h.ntau * h.mesh.size() * h.nao * h.nao;
@@ -1129,26 +770,34 @@ bool run_oassemble(Handle &h, const Point *dpts, int np, double *Nw, double *Xw,
   oa.o_off = (const long long *)P.t_o_off.p;
   oa.o_sz_p = P.o_sz;
   oa.zero = zero;
-  oa.rexp = nullptr;
-  if (ar != 0 && maxn <= 16) {
-    oa.rexp = ar == 1 ? rexp : nullptr;
-    // tensor-core modes: digit-plane products on the tensor cores, one launch over every (U, V);
-    // 5 planes (~39 bits) for the FP64-accurate mode, 3 (~23 bits, as FP32) for the mixed modes
-    dim3 og((unsigned)max_chunks, (unsigned)(np * nat * nat));
-    if (ar == 2) {
-      constexpr int kSmem = oasm_tc_smem(5);
-      static_assert(kSmem <= kOasmSmemLimit, "O assembly (tensor cores): shared memory");
-      LR_CUDA(cudaFuncSetAttribute(k_oassemble_tc<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
-      k_oassemble_tc<5><<<og, 128, kSmem, h.stream>>>(oa);
-    } else {
-      constexpr int kSmem = oasm_tc_smem(3);
-      LR_CUDA(cudaFuncSetAttribute(k_oassemble_tc<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
-      k_oassemble_tc<3><<<og, 128, kSmem, h.stream>>>(oa);
-    }
-    ++launch_counter();
-    LR_CUDA(cudaGetLastError());
-    return oa.rexp != nullptr;
+  oa.zero_chunks = max_chunks;
+  const int otc = tc ? oasm_planes(h, P) : 0;
+  if (otc) {
+    oasm::Tables t;
+    t.groups = (const oasm::Group *)P.t_ogroups.p;
+    t.tile_off = (const int *)P.t_otiles.p;
+    t.aux_atom = (const int *)P.t_aux_atom.p;
+    t.ao_row = (const int *)P.t_ao_row.p;
+    t.max_tiles = P.oasm_max_tiles;
+    oasm::run(otc, oa, t, np, *tc->nd, *tc->xd, tc->rexp, tc->err, h.stream);
+    return true;
   }
+  // arithmetic: FP64 pipes for the FP64 mode, FP32 for the mixed modes, FP32 pairs (~48 bits)
+  // for the FP64-accurate tensor-core mode
+  const int ar = P.tc_S < 0 || P.tc_S == oz::S_WIDE ? 0 : (P.tc_S >= 4 && P.tc_S <= oz::SMAX) ? 2 : 1;
+  const size_t esz = ar == 1 ? sizeof(float) : 8;
+  int NL = 4;
+  auto smem_for = [&](int nl) { return (size_t)(maxn * 2 * maxn + 2 * maxn * 64 + nl * maxn * 2 * maxn) * esz; };
+  while (NL > 1 && smem_for(NL) > 200 * 1024) NL /= 2;
+  const size_t osmem = smem_for(NL);
+  // the limit is the same fixed bound for every handle: handles on other host threads (batched
+  // and serving workers) set it concurrently, and a per-handle value could undercut a launch
+  // in flight on another thread
+  constexpr int kOasmSmemLimit = 200 * 1024;
+  if (osmem > (size_t)kOasmSmemLimit) throw Error{LIBRPA_E_ARG, "O assembly: atoms with too many NAOs"};
+  set_oasm_smem_limits<ArD>(kOasmSmemLimit);
+  set_oasm_smem_limits<ArF>(kOasmSmemLimit);
+  set_oasm_smem_limits<ArDF>(kOasmSmemLimit);
   // one launch per row-block size: the atoms U of each group (listed in the plan's table).  The
   // FP64 arithmetic is bound by the FP64 pipe, where rows beyond n_U cost nothing: one launch over
   // every atom with 16-row blocks (no tail of a second, small launch).
@@ -1618,15 +1267,18 @@ void fp64_final(Handle &h, const std::vector<Point> &pts, const Fp64Ws &w, std::
 // of Bg, Ag and O (bounded by 2 GiB, at least one point).
 struct TcWs {
   long long npb;
-  size_t b_n, b_x, b_o, b_bg, b_ag, b_od, total;
+  size_t b_n, b_x, b_o, b_bg, b_ag, b_od, b_nd = 0, b_xd = 0, total;   // nd, xd: O assembly on the tensor cores
 };
 
 TcWs tc_ws(const Handle &h, const Chi0Plan &P) {
   const int nat = h.natoms, S = P.tc_S;
   const int rows_bg = 2 * nat * P.m_all, rows_ag = 2 * nat * h.nao, rows_o = nat * h.naux;
   const size_t fp = 8 * (size_t)(2 * P.n_sz + 2 * P.x_sz + P.o_sz);
-  const size_t per_point = fp + oz::sliced_bytes(rows_bg, P.max_m, S) + oz::sliced_bytes(rows_ag, P.max_m, S) +
+  size_t per_point = fp + oz::sliced_bytes(rows_bg, P.max_m, S) + oz::sliced_bytes(rows_ag, P.max_m, S) +
                            oz::sliced_bytes(rows_o, P.max_nm, S) + 4096;
+  const int So = oasm_planes(h, P);
+  const long long rows_nd = oasm::n_rows(h.naux, P.m_all), rows_xd = oasm::x_rows(h.naux, nat);
+  if (So) per_point += oz::sliced_bytes((int)rows_nd, 32, So) + oz::sliced_bytes((int)rows_xd, 32, So);
   const long long total_pts = (long long)h.ntau * chi0_r_list(h.mesh).size();
   TcWs w;
   w.npb = std::min(std::max<long long>(1, (2LL << 30) / (long long)per_point), total_pts);
@@ -1637,7 +1289,11 @@ TcWs tc_ws(const Handle &h, const Chi0Plan &P) {
   w.b_ag = oz::sliced_bytes((int)w.npb * rows_ag, P.max_m, S);
   w.b_od = oz::sliced_bytes((int)w.npb * rows_o, P.max_nm, S);
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-  w.total = al(w.b_n) + al(w.b_x) + al(w.b_o) + al(w.b_bg) + al(w.b_ag) + al(w.b_od) + 256;
+  if (So) {
+    w.b_nd = oz::sliced_bytes((int)(w.npb * rows_nd), 32, So);
+    w.b_xd = oz::sliced_bytes((int)(w.npb * rows_xd), 32, So);
+  }
+  w.total = al(w.b_n) + al(w.b_x) + al(w.b_o) + al(w.b_bg) + al(w.b_ag) + al(w.b_od) + al(w.b_nd) + al(w.b_xd) + 256;
   return w;
 }
 
@@ -1663,7 +1319,7 @@ struct TcRound {
   std::vector<Point> pts;
   int np = 0;
   double *Nw = nullptr, *Xw = nullptr, *Ow = nullptr;
-  char *wbg = nullptr, *wag = nullptr, *wod = nullptr;
+  char *wbg = nullptr, *wag = nullptr, *wod = nullptr, *wnd = nullptr, *wxd = nullptr;
   int *err = nullptr;
   oz::Sliced cpnx, cpf, sbg, sag, sod;
   std::vector<oz::Entry> en, ex, ef;
@@ -1685,7 +1341,9 @@ TcRound tc_views(Handle &h, long long *npb) {
   r.wbg = w + al(tw.b_n) + al(tw.b_x) + al(tw.b_o);
   r.wag = r.wbg + al(tw.b_bg);
   r.wod = r.wag + al(tw.b_ag);
-  r.err = (int *)(r.wod + al(tw.b_od));
+  r.wnd = r.wod + al(tw.b_od);
+  r.wxd = r.wnd + al(tw.b_nd);
+  r.err = (int *)(r.wxd + al(tw.b_xd));
   LR_CUDA(cudaMemsetAsync(r.err, 0, 4, h.stream));
   oz::sliced_bind(r.cpnx, P.cp_nx.p, P.cpnx_rows, P.max_m, P.tc_S);
   oz::sliced_bind(r.cpf, P.cp_f.p, h.naux, P.max_nm, P.tc_S);
@@ -1763,11 +1421,18 @@ void tc_gather(Handle &h, TcRound &r) {
 void tc_assemble(Handle &h, TcRound &r, const unsigned char *zero) {
   Chi0Plan &P = h.plan;
   const int nat = h.natoms, nR = h.mesh.size(), naux = h.naux, np = r.np;
-  // the 3-plane kernel builds the row exponents when O is split into at most 3 digit planes (the
-  // plain BF16 / TF32 operands have none)
-  int *rexp = P.tc_S >= 1 && P.tc_S <= 3 ? r.sod.expo : nullptr;
-  if (rexp) oz::expo_init(r.sod, np * nat * naux, h.stream);
-  const bool expo_given = run_oassemble(h, (const Point *)P.t_pts.p, np, r.Nw, r.Xw, r.Ow, zero, rexp);
+  // the tensor-core kernel builds the row exponents of O's digit planes (the plain BF16 / TF32 operands have none
+  // of their own: sod.expo is then scratch)
+  const int So = oasm_planes(h, P);
+  oz::Sliced nd, xd;
+  OasmTc tc{&nd, &xd, r.sod.expo, r.err};
+  if (So) {
+    oz::sliced_bind(nd, r.wnd, (int)(np * oasm::n_rows(naux, P.m_all)), 32, So);
+    oz::sliced_bind(xd, r.wxd, (int)(np * oasm::x_rows(naux, nat)), 32, So);
+    oz::expo_init(r.sod, np * nat * naux, h.stream);
+  }
+  const bool expo_given =
+      run_oassemble(h, (const Point *)P.t_pts.p, np, r.Nw, r.Xw, r.Ow, zero, So ? &tc : nullptr);
   std::vector<long long> off(np * nat);
   std::vector<int> ke(np * nat);
   for (int q = 0; q < np; ++q)

@@ -1,0 +1,522 @@
+// O assembly of the chi0 contraction (k_chi0.cu) on the tensor cores.
+//
+// Per nu of V, O_nu[i][kap] is the sum of two products over K = 2 n_V:
+//   term 1:  Lm[i][t] . Nt_nu[t][kap]   Lm = [A_UV(R) | B_UV(R)],  Nt = [N[G^occ]; N[G^vir]] at the union
+//                                       column of kap
+//   term 2:  LX_nu[i][t] . RG[t][kap]   LX = [X^A_nu | X^B_nu] (rows of U),  RG = [B_{V,kap}; A_{V,kap}](R1 - R)
+// Every row of an operand (i or kap, over t) is scaled by a power of two 2^-E (E: its largest |value| < 2^E) and cut
+// into S balanced base-256 digits x = sum_s d_s 2^{-7-8(s-1)}, |d_s| <= 128 (exact in BF16); the digit products
+// of one diagonal s + t are summed exactly in FP32 (|sum| <= S * 32 * 2^14 <= 2^22), the diagonals folded into an
+// integer per term, the two terms aligned to the larger scale and converted to FP64 once (8 planes: each
+// term converted, then added).
+//
+// Two steps:
+//   k_split_n, k_split_x: the digit planes of N and X, once per point (N serves every U that holds the union
+//     column, X every tile of U).  HBM-bound.
+//   k_oasm<S>: one CTA per (point, V, U, tile of 128 rows kap).  tcgen05.mma with the kap rows as M = 128, the
+//     i of U as N (16 per plane, the planes stacked: plane s of A meets all S + 1 - s planes of B in one MMA of
+//     N = 16 (S + 1 - s)), K = 32.  RG and Lm stay in shared memory; a TMA warp streams N and X planes per nu (one
+//     box of 8 rows x S planes per row group, so a tile gathers U's columns from the union), one lane issues the
+//     MMAs, 16 warps fold and store.
+// The kernel is bound by the folding of the diagonal sums (integer and FP32 instructions) and by the
+// L2 -> shared-memory traffic of the N planes, not by the MMAs.
+#include <algorithm>
+#include <cstring>
+
+#include "internal.h"
+#include "oasm.h"
+#include "tc.h"
+
+namespace librpa {
+namespace oasm {
+namespace {
+
+constexpr float kRintMagic = 12582912.0f;   // 1.5 * 2^23: (x + M) - M rounds |x| < 2^22 to an integer
+
+// E with max |value| < 2^E from the largest |hi| (0 for an all-zero row), kept in [-100, 100]
+__device__ __forceinline__ int tc_expo(float m) {
+  if (!(m > 0.f)) return 0;
+  const int be = (__float_as_int(m) >> 23) & 0xff;
+  return min(100, max(-100, be - 126));
+}
+__device__ __forceinline__ float tc_pow2(int k) { return __int_as_float((k + 127) << 23); }   // |k| <= 126
+
+// S digits of (h + l) 2^-E into d[] (sc7 = 2^{7-E}, sc15 = 2^{15-E})
+template <int S>
+__device__ __forceinline__ void tc_digits(float h, float l, float sc7, float sc15, float *d) {
+  float t = h * sc7;
+  float dd = (t + kRintMagic) - kRintMagic;
+  float r = t - dd;
+  d[0] = dd;
+#pragma unroll
+  for (int s = 1; s < S; ++s) {
+    if (s == 2) r = fmaf(l, sc15, r);   // the low part, in units of the third digit
+    t = r * 256.f;
+    dd = (t + kRintMagic) - kRintMagic;
+    r = t - dd;
+    d[s] = dd;
+  }
+}
+
+__device__ __forceinline__ unsigned pack_bf16(float a, float b) {
+  __nv_bfloat162 v = __floats2bfloat162_rn(a, b);   // small integers: exact
+  return *reinterpret_cast<unsigned *>(&v);
+}
+
+// The element type of the operands: (hi, lo) FP32 pairs with up to 5 planes (N and X arrive so from their GEMMs, G as
+// FP64 turned into pairs; the low part joins the digits after the second, error below 2^-39 of the row
+// maximum), FP64 numbers with 8 planes.
+template <int S>
+struct Elem {
+  using T = float2;
+  __device__ static T zero() { return make_float2(0.f, 0.f); }
+  __device__ static T load(const double *p) { return *reinterpret_cast<const float2 *>(p); }
+  __device__ static T from_g(double v) {
+    const float h = __double2float_rn(v);
+    return make_float2(h, __double2float_rn(v - (double)h));
+  }
+  using M = float;   // running maximum
+  __device__ static M m0() { return 0.f; }
+  __device__ static M mx(M m, T v) { return fmaxf(m, fabsf(v.x)); }
+  __device__ static M both(M m, int o) { return fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o)); }
+  __device__ static int expo(M m) { return tc_expo(m); }
+  // digits of 8 elements, 16 bytes per plane
+  __device__ static void digits8(const T *v, int E, uint4 *w) {
+    const float sc7 = tc_pow2(7 - E), sc15 = tc_pow2(15 - E);
+    float d[8][S];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) tc_digits<S>(v[q].x, v[q].y, sc7, sc15, d[q]);
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+      w[s] = make_uint4(pack_bf16(d[0][s], d[1][s]), pack_bf16(d[2][s], d[3][s]), pack_bf16(d[4][s], d[5][s]),
+                        pack_bf16(d[6][s], d[7][s]));
+  }
+};
+template <>
+struct Elem<oz::S_WIDE> {
+  using T = double;
+  __device__ static T zero() { return 0.0; }
+  __device__ static T load(const double *p) { return *p; }
+  __device__ static T from_g(double v) { return v; }
+  using M = int;
+  __device__ static M m0() { return 0; }
+  __device__ static M mx(M m, T v) { return max(m, biased_exp(v)); }
+  __device__ static M both(M m, int o) { return max(m, __shfl_xor_sync(0xffffffffu, m, o)); }
+  __device__ static int expo(M m) { return m - 1022; }   // 1025: the row holds an infinity or a NaN
+  __device__ static void digits8(const T *v, int E, uint4 *w) {
+    constexpr int S = oz::S_WIDE;
+    unsigned *u = reinterpret_cast<unsigned *>(w);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      int d0[S], d1[S];
+      make_digits<S>(v[2 * q], E, d0);
+      make_digits<S>(v[2 * q + 1], E, d1);
+#pragma unroll
+      for (int s = 0; s < S; ++s) u[4 * s + q] = pack_bf16((float)d0[s], (float)d1[s]);
+    }
+  }
+};
+
+// Digit planes of N: rows (p, nu, union column), columns t = (g, j).  Two lanes per row (16 t each), 16 consecutive
+// columns per warp; block = 128 columns of one (p, nu).
+template <int S>
+__global__ void __launch_bounds__(256) k_split_n(OArgs a, const int *__restrict__ aux_atom, __nv_bfloat16 *dig,
+                                                 int *expo, long long plane) {
+  using E_ = Elem<S>;
+  const int p = blockIdx.x / a.naux, nug = blockIdx.x % a.naux, V = aux_atom[nug], nu = nug - a.aux_off[V];
+  const int lane = threadIdx.x & 31, h = lane >> 4;
+  const int col = blockIdx.y * 128 + (threadIdx.x >> 5) * 16 + (lane & 15);
+  const int nV = a.n_ao[V], two = 2 * nV;
+  const double *N0 = a.N + p * a.n_sz_p + a.n_off[V] + (size_t)nu * nV * a.m_all + col, *N1 = N0 + a.n_sz_g;
+  const bool live = col < a.m_all;
+  typename E_::T v[16];
+  typename E_::M m = E_::m0();
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const int t = 16 * h + q;
+    v[q] = E_::zero();
+    if (live && t < two) v[q] = E_::load(t < nV ? N0 + (size_t)t * a.m_all : N1 + (size_t)(t - nV) * a.m_all);
+    m = E_::mx(m, v[q]);
+  }
+  m = E_::both(m, 16);
+  if (!live) return;
+  const int E = E_::expo(m);
+  const long long row = ((long long)p * a.naux + nug) * a.m_all + col;
+  if (h == 0) expo[row] = E;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    uint4 w[S];
+    E_::digits8(v + 8 * c, E, w);
+#pragma unroll
+    for (int s = 0; s < S; ++s) *reinterpret_cast<uint4 *>(dig + s * plane + row * 32 + 16 * h + 8 * c) = w[s];
+  }
+}
+
+// Digit planes of X: rows (p, nu, 16 U + i), columns t; two lanes per row.  Rows i >= n_U are left as they are (the MMA
+// columns they give are not read).
+template <int S>
+__global__ void __launch_bounds__(256) k_split_x(OArgs a, const int *__restrict__ aux_atom,
+                                                 const int *__restrict__ ao_row, __nv_bfloat16 *dig, int *expo,
+                                                 long long plane) {
+  using E_ = Elem<S>;
+  const int p = blockIdx.x / a.naux, nug = blockIdx.x % a.naux, V = aux_atom[nug], nu = nug - a.aux_off[V];
+  const int lane = threadIdx.x & 31, h = lane >> 4;
+  const int ao = blockIdx.y * 128 + (threadIdx.x >> 5) * 16 + (lane & 15);
+  const int nV = a.n_ao[V], two = 2 * nV;
+  const size_t ldx = (size_t)a.n_aux[V] * nV;
+  const double *XB = a.X + p * a.x_sz_p + a.x_off[V] + ao * ldx + (size_t)nu * nV, *XA = XB + a.x_sz_g;
+  const bool live = ao < a.nao;
+  typename E_::T v[16];
+  typename E_::M m = E_::m0();
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const int t = 16 * h + q;
+    v[q] = E_::zero();
+    if (live && t < two) v[q] = E_::load(t < nV ? XA + t : XB + (t - nV));
+    m = E_::mx(m, v[q]);
+  }
+  m = E_::both(m, 16);
+  if (!live) return;
+  const int E = E_::expo(m);
+  const long long row = ((long long)p * a.naux + nug) * (a.natoms * kMaxAo) + ao_row[ao];
+  if (h == 0) expo[row] = E;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    uint4 w[S];
+    E_::digits8(v + 8 * c, E, w);
+#pragma unroll
+    for (int s = 0; s < S; ++s) *reinterpret_cast<uint4 *>(dig + s * plane + row * 32 + 16 * h + 8 * c) = w[s];
+  }
+}
+
+// ------------------------------------------------------------------ the products
+constexpr int kEpi = 16, kThreads = 32 * (kEpi + 2);
+__host__ __device__ constexpr int op_bytes(int S) { return kTileGroups * S * 512; }   // 128 rows: groups of 8 rows x S planes x 64 bytes
+__host__ __device__ constexpr int x_bytes(int S) { return S * kMaxAo * 64; }          // S planes of 16 rows x 64 bytes
+__host__ __device__ constexpr int stage_size(int S) { return op_bytes(S) + x_bytes(S); }
+__host__ __device__ constexpr int ring(int S) { return S == oz::S_WIDE ? 2 : S == 5 ? 3 : 5; }
+__host__ __device__ constexpr int smem_size(int S) { return (1 + ring(S)) * stage_size(S) + 1024; }
+__host__ __device__ constexpr int slot_cols(int S) { return 2 * S * kMaxAo; }         // TMEM columns of one nu: two terms, S diagonals, 16 i
+__host__ __device__ constexpr int slots(int S) { return 512 / slot_cols(S); }
+
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t *r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait4(uint32_t *r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3])::"memory");
+}
+
+__device__ __forceinline__ int rint_sum(uint32_t f) {   // an integer-valued FP32 sum, |f| <= 2^22
+  return (int)((unsigned)__float_as_int(__uint_as_float(f) + kRintMagic) - 0x4B400000u);
+}
+
+// element (x) of the two terms' sums r1, r2 ([diagonal][4] registers), scales 2^E1, 2^E2
+template <int S>
+__device__ __forceinline__ double combine(const uint32_t (&r1)[S][4], const uint32_t (&r2)[S][4], int x, int E1, int E2) {
+  if constexpr (S == oz::S_WIDE) {
+    long long h1 = 0, l1 = 0, h2 = 0, l2 = 0;
+#pragma unroll
+    for (int d = 0; d < 4; ++d) {
+      h1 += (long long)rint_sum(r1[d][x]) * (1 << (8 * (3 - d)));
+      l1 += (long long)rint_sum(r1[d + 4][x]) * (1 << (8 * (3 - d)));
+      h2 += (long long)rint_sum(r2[d][x]) * (1 << (8 * (3 - d)));
+      l2 += (long long)rint_sum(r2[d + 4][x]) * (1 << (8 * (3 - d)));
+    }
+    return i96_to_f64(h1, l1, E1 - 14 - 56) + i96_to_f64(h2, l2, E2 - 14 - 56);
+  } else {
+    long long T1 = rint_sum(r1[S - 1][x]), T2 = rint_sum(r2[S - 1][x]);
+#pragma unroll
+    for (int d = 0; d < S - 1; ++d) {
+      if (S == 5 && d == 0) {
+        T1 += (long long)((unsigned long long)(unsigned)rint_sum(r1[d][x]) << 32);
+        T2 += (long long)((unsigned long long)(unsigned)rint_sum(r2[d][x]) << 32);
+      } else {
+        T1 += (long long)rint_sum(r1[d][x]) * (1 << (8 * (S - 1 - d) % 32));
+        T2 += (long long)rint_sum(r2[d][x]) * (1 << (8 * (S - 1 - d) % 32));
+      }
+    }
+    // the smaller scale's sum rounded to the larger scale
+    const bool one = E1 >= E2;
+    const long long big = one ? T1 : T2, small = one ? T2 : T1;
+    const int sh = min(one ? E1 - E2 : E2 - E1, 62);
+    const long long T = big + ((small + (long long)((1ull << sh) >> 1)) >> sh);
+    return i64_to_f64(T, (one ? E1 : E2) - 14 - 8 * (S - 1));
+  }
+}
+
+template <int S>
+__global__ void __launch_bounds__(kThreads, 1)
+    k_oasm(OArgs a, Tables tb, const __grid_constant__ CUtensorMap nmap, const __grid_constant__ CUtensorMap xmap,
+           const int *__restrict__ nexp, const int *__restrict__ xexp, int *rexp, int *err) {
+  using E_ = Elem<S>;
+  constexpr int NST = ring(S), NSL = slots(S), SL = slot_cols(S);
+  constexpr uint32_t OPB = op_bytes(S), XB_ = x_bytes(S), STAGE = stage_size(S);
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ uint64_t full[NST], empty[NST], tfull[NSL], tempty[NSL], mdone;
+  __shared__ uint32_t tmem_slot;
+  __shared__ volatile int abort_flag;
+  __shared__ int s_e1[kMaxAo], s_f2[128], s_kap[128], s_urow[128], s_box[kTileGroups];
+  __shared__ int s_groups;
+  // U and its tiles run fastest: the CTAs in flight share the N planes of a few V in the L2
+  const int uv = blockIdx.x / tb.max_tiles;
+  const int U = uv % a.natoms, V = (uv / a.natoms) % a.natoms, p = uv / (a.natoms * a.natoms);
+  const int tile = tb.tile_off[U] + (int)(blockIdx.x % tb.max_tiles);
+  if (tile >= tb.tile_off[U + 1]) return;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nU = a.n_ao[U], nV = a.n_ao[V], two = 2 * nV, nauxV = a.n_aux[V], mU = a.m[U];
+  double *Ob = a.O + p * a.o_sz_p + a.o_off[U];
+  const int ldo = nU * mU;
+  if (a.zero) {   // under screening: a tile whose 64-column chunks are all exactly zero
+    const Group g0 = tb.groups[(size_t)tile * kTileGroups];
+    int k1 = g0.kap;
+    for (int g = 0; g < kTileGroups; ++g) {
+      const Group gg = tb.groups[(size_t)tile * kTileGroups + g];
+      if (gg.live) k1 = gg.kap + gg.live;
+    }
+    const unsigned char *z = a.zero + ((size_t)(p * a.natoms + U) * a.natoms + V) * a.zero_chunks;
+    bool all = true;
+    for (int c = g0.kap / 64; c * 64 < k1; ++c) all = all && z[c];
+    if (all) {
+      const int w = k1 - g0.kap;
+      for (long long e = tid; e < (long long)nauxV * nU * w; e += kThreads) {
+        const int col = (int)(e % w);
+        const long long r = e / w;
+        Ob[(size_t)(a.aux_off[V] + r / nU) * ldo + (size_t)(r % nU) * mU + g0.kap + col] = 0.0;
+      }
+      return;
+    }
+  }
+  uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint8_t *sRG = smem, *sLm = smem + OPB;   // static operands, then the ring
+  if (tid == 0) {
+    for (int s = 0; s < NST; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int s = 0; s < NSL; ++s) {
+      mbar_init(&tfull[s], 1);
+      mbar_init(&tempty[s], 8);
+    }
+    mbar_init(&mdone, 1);
+    abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == kEpi) tmem_alloc(&tmem_slot, 512);
+  if (warp == kEpi + 1 && lane < kTileGroups) {   // the tile's row groups
+    const Group g = tb.groups[(size_t)tile * kTileGroups + lane];
+    s_box[lane] = g.live ? g.urow : -1;
+    const unsigned m = __ballot_sync(0xffffu, g.live > 0);
+    if (lane == 0) s_groups = __popc(m);
+  }
+  const Point pt = a.pts[p];
+  const size_t n2 = (size_t)a.nao * a.nao;
+  const double *GB = a.G + ((size_t)pt.itau * a.nR_stride) * n2;                 // G^occ(tau)
+  const double *GA = a.G + a.g_gstride + ((size_t)pt.itau * a.nR_stride) * n2;   // G^vir(tau)
+  const int aoU = a.ao_off[U], aoV = a.ao_off[V];
+  // RG digits: four threads per row kap, 8 columns t each; 16-byte pieces swizzled as TMA would
+  if (tid < 512) {
+    const int r = tid >> 2, c = tid & 3;
+    const Group g = tb.groups[(size_t)tile * kTileGroups + (r >> 3)];
+    const bool live = (r & 7) < g.live;
+    const int kc = g.kap + (r & 7);
+    const int *kp = a.kap + 6 * (a.kap_off[U] + (live ? kc : 0));
+    auto fold = [](int x, int nn) { int q = x % nn; return q < 0 ? q + nn : q; };
+    const int iR = (fold(kp[1] - pt.R[0], a.n1) * a.n2 + fold(kp[2] - pt.R[1], a.n2)) * a.n3 + fold(kp[3] - pt.R[2], a.n3);
+    typename E_::T v[8];
+    typename E_::M m = E_::m0();
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int t = 8 * c + q;
+      v[q] = E_::zero();
+      if (live && t < two)
+        v[q] = E_::from_g((t < nV ? GB : GA)[(size_t)iR * n2 + (size_t)(aoV + (t < nV ? t : t - nV)) * a.nao + kp[4]]);
+      m = E_::mx(m, v[q]);
+    }
+    m = E_::both(E_::both(m, 1), 2);
+    const int E = E_::expo(m);
+    if (c == 0) {
+      s_f2[r] = E;
+      s_kap[r] = live ? kc : -1;
+      s_urow[r] = g.urow + (r & 7);
+    }
+    uint4 w[S];
+    E_::digits8(v, E, w);
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+      *reinterpret_cast<uint4 *>(sRG + (r >> 3) * (S * 512) + s * 512 + (r & 7) * 64 + ((c ^ ((r >> 1) & 3)) << 4)) = w[s];
+  }
+  if (tid < 64) {   // Lm digits: rows i, planes of 16 rows one after the other
+    const int i = tid >> 2, c = tid & 3;
+    typename E_::T v[8];
+    typename E_::M m = E_::m0();
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int t = 8 * c + q;
+      v[q] = E_::zero();
+      if (i < nU && t < two)
+        v[q] = E_::from_g((t < nV ? GA : GB)[(size_t)pt.iR * n2 + (size_t)(aoU + i) * a.nao + aoV + (t < nV ? t : t - nV)]);
+      m = E_::mx(m, v[q]);
+    }
+    m = E_::both(E_::both(m, 1), 2);
+    const int E = E_::expo(m);
+    if (c == 0) s_e1[i] = E;
+    uint4 w[S];
+    E_::digits8(v, E, w);
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+      *reinterpret_cast<uint4 *>(sLm + s * 1024 + i * 64 + ((c ^ ((i >> 1) & 3)) << 4)) = w[s];
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the MMAs read what was stored here
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  const long long nu0 = (long long)p * a.naux + a.aux_off[V];
+  if (warp == kEpi) {
+    if (lane == 0) {   // TMA producer: N rows of the tile's groups and the 16 X rows of U, per nu
+      const int ng = s_groups;
+      int it = 0;
+      for (; it < nauxV; ++it) {
+        const int st = it % NST;
+        if (abort_flag || !mbar_wait(&empty[st], (uint32_t)(((it / NST) & 1) ^ 1), WAIT_NS, &abort_flag)) {
+          abort_flag = 1;
+          break;
+        }
+        uint8_t *sn = smem + STAGE + st * STAGE, *sx = sn + OPB;
+        mbar_expect_tx(&full[st], (uint32_t)ng * S * 512 + XB_);
+        const int row = (int)((nu0 + it) * a.m_all);
+        for (int g = 0; g < ng; ++g) tma_load_3d(sn + g * (S * 512), &nmap, &full[st], 0, row + s_box[g], 0);
+        tma_load_3d(sx, &xmap, &full[st], 0, (int)((nu0 + it) * a.natoms + U) * kMaxAo, 0);
+      }
+      // after a failure: wait for the copies still in flight (the last NST issued stages)
+      if (abort_flag)
+        for (int i = it > NST ? it - NST : 0; i < it; ++i) mbar_wait(&full[i % NST], (uint32_t)((i / NST) & 1), WAIT_NS);
+    }
+  } else if (warp == kEpi + 1) {
+    if (lane == 0) {   // MMA issuer
+      const int ks = (two + 15) / 16;
+      const uint32_t rg = smem_u32(sRG), lm = smem_u32(sLm);
+      for (int it = 0; it < nauxV; ++it) {
+        const int st = it % NST, sl = it % NSL;
+        if (it >= NSL && (abort_flag || !mbar_wait(&tempty[sl], (uint32_t)((it / NSL - 1) & 1), WAIT_NS, &abort_flag))) {
+          abort_flag = 1;
+          break;
+        }
+        if (abort_flag || !mbar_wait(&full[st], (uint32_t)((it / NST) & 1), WAIT_NS, &abort_flag)) {
+          abort_flag = 1;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t sn = smem_u32(smem + STAGE + st * STAGE), sx = sn + OPB, d = tmem + sl * SL;
+        for (int j = 0; j < ks; ++j)
+#pragma unroll
+          for (int s = 0; s < S; ++s) {   // plane s of A by planes 0 .. S - 1 - s of B, into the diagonals s ..
+            const uint32_t ide = idesc(kMaxAo * (S - s), false), acc = (j == 0 && s == 0) ? 0u : 1u;
+            umma(d + s * kMaxAo, smem_desc64(sn + s * 512 + 32 * j, S * 512), smem_desc64(lm + 32 * j), ide, acc);
+            umma(d + (S + s) * kMaxAo, smem_desc64(rg + s * 512 + 32 * j, S * 512), smem_desc64(sx + 32 * j), ide, acc);
+          }
+        umma_commit(&empty[st]);
+        umma_commit(&tfull[sl]);
+      }
+      if (abort_flag) {   // after a failure: wait for the MMAs already issued
+        umma_commit(&mdone);
+        mbar_wait(&mdone, 0, WAIT_NS);
+      }
+    }
+  } else {
+    // epilogue: warps 0-7 the even nu, 8-15 the odd ones; thread = row kap, half of the i each
+    const int grp = warp >> 3, quad = warp & 3, half = (warp >> 2) & 1;
+    const int r = quad * 32 + lane, kap = s_kap[r], f2 = s_f2[r], urow = s_urow[r];
+    const bool any = __any_sync(0xffffffffu, kap >= 0);
+    const int per = (nU + 1) / 2, c0 = half * per, c1 = min(nU, c0 + per);
+    for (int it = grp; it < nauxV; it += 2) {
+      const int sl = it % NSL;
+      const int f1 = kap >= 0 ? nexp[(nu0 + it) * a.m_all + urow] : 0;
+      const int *xe = xexp + ((nu0 + it) * a.natoms + U) * kMaxAo;
+      bool ok = !abort_flag && mbar_wait(&tfull[sl], (uint32_t)((it / NSL) & 1), WAIT_NS, &abort_flag);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) {
+        abort_flag = 1;
+        break;
+      }
+      tc_fence_after();
+      int emax = 0;   // largest biased exponent among this lane's outputs
+      if (any) {
+        const uint32_t tb0 = tmem + ((uint32_t)(32 * quad) << 16) + sl * SL;
+        double *orow = Ob + (size_t)(a.aux_off[V] + it) * ldo + kap;
+#pragma unroll 1
+        for (int c = c0; c < c1; c += 4) {
+          uint32_t r1[S][4], r2[S][4];
+          int e2[4];
+#pragma unroll
+          for (int x = 0; x < 4; ++x) e2[x] = xe[min(c + x, kMaxAo - 1)];
+#pragma unroll
+          for (int d = 0; d < S; ++d) {
+            tmem_ld4(tb0 + d * kMaxAo + c, r1[d]);
+            tmem_ld4(tb0 + (S + d) * kMaxAo + c, r2[d]);
+          }
+#pragma unroll
+          for (int d = 0; d < S; ++d) {
+            tmem_wait4(r1[d]);
+            tmem_wait4(r2[d]);
+          }
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            if (c + x >= c1) break;   // the same for the whole warp
+            const int e1 = s_e1[c + x];
+            double o = combine<S>(r1, r2, x, e1 + f1, e2[x] + f2);
+            if (S == oz::S_WIDE && max(max(e1, f1), max(e2[x], f2)) > 1024) o = __longlong_as_double(0x7FF8000000000000ll);
+            if (kap >= 0) {
+              orow[(size_t)(c + x) * mU] = o;
+              emax = max(emax, biased_exp(o));
+            }
+          }
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&tempty[sl]);
+      // the row (p, U, nu) of the final contraction's O operand
+      emax = __reduce_max_sync(0xffffffffu, emax);
+      if (lane == 0 && emax > 0) atomicMax(rexp + ((size_t)p * a.natoms + U) * a.naux + a.aux_off[V] + it, emax - 1022);
+    }
+  }
+  __syncthreads();
+  if (abort_flag && tid == 0) atomicExch(err, 1);
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kEpi) tmem_dealloc(tmem, 512);
+}
+
+template <int S>
+void launch(const OArgs &a, const Tables &t, int np, oz::Sliced &nd, oz::Sliced &xd, int *expo, int *err, cudaStream_t s) {
+  static_assert(smem_size(S) <= 227 * 1024, "k_oasm: shared memory");
+  const unsigned rows = (unsigned)(np * a.naux);
+  k_split_n<S><<<dim3(rows, (unsigned)((a.m_all + 127) / 128)), 256, 0, s>>>(
+      a, t.aux_atom, (__nv_bfloat16 *)nd.digits, nd.expo, (long long)nd.rows * nd.kpad);
+  k_split_x<S><<<dim3(rows, (unsigned)((a.nao + 127) / 128)), 256, 0, s>>>(
+      a, t.aux_atom, t.ao_row, (__nv_bfloat16 *)xd.digits, xd.expo, (long long)xd.rows * xd.kpad);
+  LR_CUDA(cudaFuncSetAttribute(k_oasm<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_size(S)));
+  k_oasm<S><<<(unsigned)t.max_tiles * (unsigned)(np * a.natoms * a.natoms), kThreads, smem_size(S), s>>>(
+      a, t, oz::make_map(nd, 8, S), oz::make_map(xd, kMaxAo, S), nd.expo, xd.expo, expo, err);
+  launch_counter() += 3;
+  LR_CUDA(cudaGetLastError());
+}
+
+}  // namespace
+
+void run(int S, const OArgs &a, const Tables &t, int np, oz::Sliced &nd, oz::Sliced &xd, int *expo, int *err,
+         cudaStream_t s) {
+  oz::init();
+  if (S == 3)
+    launch<3>(a, t, np, nd, xd, expo, err, s);
+  else if (S == 5)
+    launch<5>(a, t, np, nd, xd, expo, err, s);
+  else
+    launch<oz::S_WIDE>(a, t, np, nd, xd, expo, err, s);
+}
+
+}  // namespace oasm
+}  // namespace librpa

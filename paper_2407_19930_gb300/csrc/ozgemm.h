@@ -13,6 +13,7 @@
 // kind::f16) and S = S_TF32 (TF32 in FP32 containers, kind::tf32).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -136,6 +137,10 @@ long long gemm_multi(const std::vector<std::pair<const Sliced *, const Sliced *>
 // an operand with exactly M (N) rows is shared by all entries.
 long long gemm(const Sliced &a, const Sliced &b, int M, int N, int batch, const Out &out, int km, int kn,
                int lower_div, int *err, cudaStream_t s, Handle &h);
+
+// Tensor map of an operand's planes with boxes of 64 bytes x box_rows rows x box_planes planes (64-byte
+// swizzle); after init().
+CUtensorMap make_map(const Sliced &o, int box_rows, int box_planes = 1);
 
 // One-time host setup (driver entry point for tensor-map encoding).  Throws on failure.
 void init();
