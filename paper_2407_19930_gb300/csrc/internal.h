@@ -96,11 +96,13 @@ struct Chi0Plan {
   // of each NAO among the X digit planes (oasm.h)
   DevBuf t_ogroups, t_otiles, t_aux_atom, t_ao_row;
   int oasm_max_tiles = 0;
+  DevBuf t_lamf, t_unif;   // the columns of d_lam and d_uni with folded, packed lattice vectors (GatherSrc)
+  bool folded = false;
   std::vector<DevBuf *> all() {
     return {&d_lam, &d_uni, &d_kap, &t_n_ao, &t_n_aux, &t_ao_off, &t_aux_off, &t_m, &t_lam_off, &t_kap_off,
             &t_bg_off, &t_ag_off, &t_n_off, &t_x_off, &t_o_off, &t_pts, &ws, &gargs1, &gargs2,
             &cp_nx, &cp_f, &t_oe_off, &t_oe_k, &gargs3, &t_ozero, &t_ugroups,
-            &t_ogroups, &t_otiles, &t_aux_atom, &t_ao_row};
+            &t_ogroups, &t_otiles, &t_aux_atom, &t_ao_row, &t_lamf, &t_unif};
   }
 };
 

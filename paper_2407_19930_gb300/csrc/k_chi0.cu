@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(256, 2) k_oassemble(OArgs a, int NL, const int
       const int col = (int)(e % 64);
       if (col >= w) continue;
       const long long r = e / 64;
-      Ob[(size_t)(a.aux_off[V] + r / nU) * nU * mU + (size_t)(r % nU) * mU + c0 + col] = 0.0;
+      Ob[(size_t)(a.aux_off[V] + r / nU) * o_pitch(nU, mU) + (size_t)(r % nU) * mU + c0 + col] = 0.0;
     }
     return;
   }
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(256, 2) k_oassemble(OArgs a, int NL, const int
   const double *XA = a.X + p * a.x_sz_p + a.x_sz_g + a.x_off[V];      // X[G^vir]
   const int ldx = nauxV * nV;
   double *Ob = a.O + p * a.o_sz_p + a.o_off[U];
-  const int ldo = nU * mU;
+  const int ldo = o_pitch(nU, mU);
   for (int nu0 = 0; nu0 < nauxV; nu0 += NL) {
     __syncthreads();   // previous LX consumed; Lm and RG written
     for (int e = tid; e < NL * nU * two; e += nthr) {
@@ -536,7 +536,7 @@ void chi0_shape(const Handle &h, Chi0Plan &P) {
     P.ag_off[V + 1] = P.ag_off[V] + (long long)h.nao * P.m[V];
     P.n_off[V + 1] = P.n_off[V] + rowsV * P.m_all;
     P.x_off[V + 1] = P.x_off[V] + (long long)h.nao * rowsV;
-    P.o_off[V + 1] = P.o_off[V] + (long long)h.naux * h.n_ao[V] * P.m[V];
+    P.o_off[V + 1] = P.o_off[V] + (long long)h.naux * o_pitch(h.n_ao[V], P.m[V]);
     fl += 2.0 * 2.0 * rowsV * P.m[V] * P.m_all;    // N-step, both G
     fl += 2.0 * 2.0 * h.nao * P.m[V] * rowsV;      // X-step, both G
   }
@@ -623,6 +623,19 @@ void chi0_plan(Handle &h) {
   upload(h, P.d_lam, lam);
   upload(h, P.d_kap, kap);
   upload(h, P.d_uni, un);
+  P.folded = h.mesh.n1 <= 255 && h.mesh.n2 <= 255 && h.mesh.n3 <= 255;
+  if (P.folded) {   // the lattice vectors folded into the BvK cell and packed (k_digits_gather)
+    auto pack = [&](const std::vector<int> &t) {
+      std::vector<int2> f(t.size() / 6);
+      for (size_t x = 0; x < f.size(); ++x)
+        f[x] = make_int2(Mesh::fold(t[6 * x + 1], h.mesh.n1) | Mesh::fold(t[6 * x + 2], h.mesh.n2) << 8 |
+                             Mesh::fold(t[6 * x + 3], h.mesh.n3) << 16,
+                         t[6 * x + 5]);
+      return f;
+    };
+    upload(h, P.t_lamf, pack(lam));
+    upload(h, P.t_unif, pack(un));
+  }
   upload(h, P.t_n_ao, h.n_ao);
   upload(h, P.t_n_aux, h.n_aux);
   upload(h, P.t_ao_off, h.ao_off);
@@ -1257,7 +1270,7 @@ void fp64_final(Handle &h, const std::vector<Point> &pts, const Fp64Ws &w, std::
     for (int U = 0; U < h.natoms; ++U) {
       const int K = h.n_ao[U] * P.m[U];
       DGemm df{Cp + P.cp_off[U], w.Ow + q * P.o_sz + P.o_off[U], chi + (size_t)h.aux_off[U] * naux, h.n_aux[U],
-               naux, K, K, K, naux, -spin, beta};
+               naux, K, K, o_pitch(h.n_ao[U], P.m[U]), naux, -spin, beta};
       b.push_back(df);
     }
   }
@@ -1374,6 +1387,8 @@ void tc_gather(Handle &h, TcRound &r) {
   gs.lam = (const int *)P.d_lam.p;
   gs.lam_off = (const long long *)P.t_lam_off.p;
   gs.m = (const int *)P.t_m.p;
+  gs.lamf = P.folded ? (const int2 *)P.t_lamf.p : nullptr;
+  gs.unif = P.folded ? (const int2 *)P.t_unif.p : nullptr;
   const int rows_bg = 2 * nat * P.m_all, rows_ag = 2 * nat * nao, rows_o = nat * h.naux;
   oz::sliced_bind(r.sbg, r.wbg, np * rows_bg, P.max_m, S);
   oz::sliced_bind(r.sag, r.wag, np * rows_ag, P.max_m, S);

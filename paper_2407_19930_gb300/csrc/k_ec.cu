@@ -32,137 +32,286 @@ namespace {
 
 constexpr int NB = 64;
 
+// ------------------------------------------------------------------ panel kernels (FP64 pipe)
+// FP64 runs at two fused multiply-adds per cycle and SM on GB300, a warp's instruction taking ~64 cycles of its
+// scheduler's share, so the panel kernels are bound by that pipe (a 64 x 64 complex factorisation is 87k
+// cycles of it) and by how few FP64 instructions the serial chains take: columns go in blocks of 8, whose
+// 8 x 8 triangle 64 threads factor, an element each, and every other product runs over many threads.
+constexpr int KB = 8;   // columns per block
+
+// 1 / sqrt(d) for a normal d > 0 in five FP64 instructions: FP32 seed r0 of the mantissa and one step of third order
+// in e = 1 - d r0^2 (r0 (1 + e / 2 + 3 e^2 / 8), error ~e^3 < 2^-60), conversions and scaling by integer instructions
+__device__ __forceinline__ double fast_rsqrt(double d) {
+  const int hi = __double2hiint(d), ex = hi >> 20;
+  if (ex < 1 || ex > 2046) return rsqrt(d);
+  const int q = (ex - 1023) & ~1;   // d 2^-q in [1, 4)
+  const double x = __hiloint2double(hi - (q << 20), __double2loint(d));
+  const float f = __int_as_float(((ex - q - 896) << 23) | ((hi & 0xFFFFF) << 3));
+  const int rb = __float_as_int(rsqrtf(f));
+  const double r0 = __hiloint2double((rb >> 3) + (896 << 20), rb << 29);
+  const double e = fma(-(x * r0), r0, 1.0);
+  const double r = fma(r0 * e, fma(0.375, e, 0.5), r0);
+  return __hiloint2double(__double2hiint(r) - ((q / 2) << 20), __double2loint(r));
+}
+__device__ __forceinline__ void bar_64() { asm volatile("bar.sync 1, 64;" ::: "memory"); }   // threads 0..63
+
+// element arithmetic: T = double2 (complex) or double
+__device__ __forceinline__ void sub_mul_conj(double2 &c, double2 a, double2 b) {   // c -= a conj(b)
+  c.x = fma(-a.x, b.x, fma(-a.y, b.y, c.x));
+  c.y = fma(-a.y, b.x, fma(a.x, b.y, c.y));
+}
+__device__ __forceinline__ void sub_mul_conj(double &c, double a, double b) { c = fma(-a, b, c); }
+__device__ __forceinline__ void sub_mul(double2 &c, double2 a, double2 b) {        // c -= a b
+  c.x = fma(-a.x, b.x, fma(a.y, b.y, c.x));
+  c.y = fma(-a.x, b.y, fma(-a.y, b.x, c.y));
+}
+__device__ __forceinline__ void sub_mul(double &c, double a, double b) { c = fma(-a, b, c); }
+__device__ __forceinline__ double2 scaled(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
+__device__ __forceinline__ double scaled(double a, double s) { return a * s; }
+__device__ __forceinline__ double re_of(double2 a) { return a.x; }
+__device__ __forceinline__ double re_of(double a) { return a; }
+__device__ __forceinline__ void set_re(double2 &a, double x) { a = make_double2(x, 0.0); }
+__device__ __forceinline__ void set_re(double &a, double x) { a = x; }
+
 // Factor the NB x NB diagonal block at p0 of every matrix in place (lower triangle).  One CTA per
 // matrix.  Adds 2 sum ln d_jj to lndet[b]; sets info[b] = 1 on a non-positive pivot.
-// inv (optional, [matrix][NB][NB]): receives L_pp^{-1} of the factored block (lower triangular,
-// zero elsewhere), computed in shared memory by forward substitution, one column per thread.
-__global__ void __launch_bounds__(256) k_potrf_diag(double2 *const *mats, int n, int ld, int p0, double *lndet,
-                                                    int *info, double2 *inv) {
-  extern __shared__ double2 a[];   // [NB][NB + 1] (and, with inv, a second such array)
-  const int b = blockIdx.x;
-  double2 *M = mats[b];
-  const int nb = min(NB, n - p0);
-  const int lda = NB + 1;
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    const int i = e / nb, j = e % nb;
-    a[i * lda + j] = j <= i ? M[(size_t)(p0 + i) * ld + p0 + j] : make_double2(0.0, 0.0);
-  }
-  __syncthreads();
-  __shared__ double dsh;
+// inv (optional, [matrix][NB][NB]): receives L_pp^{-1} of the factored block (lower triangular, zero elsewhere), by
+// blocks of 8 rows: Y_II = L_II^{-1}, Y_IJ = -Y_II sum_K L_IK Y_KJ.
+// 64 x 64 complex: 268 -> ~75 us (with the inverse 390 -> ~150 us at 96 matrices) against one column at a time.
+template <class T>
+__global__ void __launch_bounds__(256) k_potrf_diag(T *const *mats, int n, int ld, int p0, double *lndet, int *info,
+                                                    T *inv) {
+  extern __shared__ __align__(16) unsigned char sm_potrf[];
+  T *a = reinterpret_cast<T *>(sm_potrf);   // [NB][NB + 1] (and, with inv, a second such array)
+  constexpr int lda = NB + 1;
+  __shared__ double rinv[NB], piv[NB];
+  __shared__ T colj[2][KB];
   __shared__ int bad;
-  if (threadIdx.x == 0) bad = 0;
-  double lsum = 0.0;
-  for (int j = 0; j < nb; ++j) {
-    if (threadIdx.x == 0) {
-      double d = a[j * lda + j].x;
-      if (!(d > 0.0) || !isfinite(d)) {
-        bad = 1;
-        d = 1.0;
+  const int b = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  T *M = mats[b];
+  const int nb = min(NB, n - p0);
+  // a ragged last block is completed with the unit matrix
+  for (int e = tid; e < NB * NB; e += 256) {
+    const int i = e / NB, j = e % NB;
+    T v{};
+    if (i < nb) {
+      if (j <= i) v = M[(size_t)(p0 + i) * ld + p0 + j];
+    } else if (i == j) {
+      set_re(v, 1.0);
+    }
+    a[i * lda + j] = v;
+  }
+  if (tid == 0) bad = 0;
+  __syncthreads();
+  for (int j0 = 0; j0 < nb; j0 += KB) {
+    if (tid < KB * KB) {   // the 8 x 8 triangle: thread = element (r, k)
+      const int r = tid / KB, k = tid % KB;
+      T e = a[(j0 + r) * lda + j0 + k];
+#pragma unroll
+      for (int j = 0; j < KB; ++j) {
+        T *col = colj[j & 1];   // column j before its scaling
+        if (k == j) col[r] = e;
+        bar_64();
+        double d = re_of(col[j]);
+        const bool ok = d > 0.0 && isfinite(d);
+        if (!ok) d = 1.0;
+        const double ri = fast_rsqrt(d);
+        if (k == j) {
+          if (r == j) {
+            double sq = d * ri;
+            sq = fma(0.5 * ri, fma(-sq, sq, d), sq);   // sqrt(d)
+            set_re(e, sq);
+            rinv[j0 + j] = ri;
+            piv[j0 + j] = sq;
+            if (!ok) bad = 1;
+          } else {
+            e = scaled(e, ri);
+          }
+        } else if (k > j && r >= k) {
+          sub_mul_conj(e, scaled(col[r], ri), scaled(col[k], ri));
+        }
       }
-      d = sqrt(d);
-      a[j * lda + j] = make_double2(d, 0.0);
-      lsum += 2.0 * log(d);
-      dsh = d;
+      if (k <= r) a[(j0 + r) * lda + j0 + k] = e;
     }
     __syncthreads();
-    const double inv = 1.0 / dsh;
-    for (int i = j + 1 + threadIdx.x; i < nb; i += blockDim.x) {
-      a[i * lda + j].x *= inv;
-      a[i * lda + j].y *= inv;
+    const int c0 = j0 + KB, m = NB - c0;   // the rows and columns left
+    if (tid < m) {   // panel rows: x_j = (b_j - sum_{k<j} x_k conj(L_jk)) / L_jj
+      T x[KB], *row = a + (c0 + tid) * lda + j0;
+#pragma unroll
+      for (int j = 0; j < KB; ++j) {
+        x[j] = row[j];
+#pragma unroll
+        for (int k = 0; k < j; ++k) sub_mul_conj(x[j], x[k], a[(j0 + j) * lda + j0 + k]);
+        x[j] = scaled(x[j], rinv[j0 + j]);
+      }
+#pragma unroll
+      for (int j = 0; j < KB; ++j) row[j] = x[j];
     }
     __syncthreads();
-    // trailing update of the block: a_ik -= a_ij conj(a_kj), j < k <= i
-    const int m = nb - j - 1;
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-      const int i = j + 1 + e / m, k = j + 1 + e % m;
-      if (k > i) continue;
-      const double2 x = a[i * lda + j], y = a[k * lda + j];
-      a[i * lda + k].x -= x.x * y.x + x.y * y.y;
-      a[i * lda + k].y -= x.y * y.x - x.x * y.y;
+    // trailing update a_ik -= sum_j a_ij conj(a_kj) in 2 x 2 tiles of the lower triangle
+    const int mt = m / 2, nt = mt * (mt + 1) / 2;
+    for (int t = tid; t < nt; t += 256) {
+      int ty = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+      if (ty * (ty + 1) / 2 > t) --ty;
+      if ((ty + 1) * (ty + 2) / 2 <= t) ++ty;
+      const int tx = t - ty * (ty + 1) / 2, i = c0 + 2 * ty, k = c0 + 2 * tx;
+      T c00 = a[i * lda + k], c01 = a[i * lda + k + 1], c10 = a[(i + 1) * lda + k], c11 = a[(i + 1) * lda + k + 1];
+#pragma unroll
+      for (int j = 0; j < KB; ++j) {
+        const T x0 = a[i * lda + j0 + j], x1 = a[(i + 1) * lda + j0 + j], y0 = a[k * lda + j0 + j],
+                y1 = a[(k + 1) * lda + j0 + j];
+        sub_mul_conj(c00, x0, y0);
+        sub_mul_conj(c01, x0, y1);
+        sub_mul_conj(c10, x1, y0);
+        sub_mul_conj(c11, x1, y1);
+      }
+      a[i * lda + k] = c00;
+      if (tx < ty) a[i * lda + k + 1] = c01;   // (the element above the diagonal stays)
+      a[(i + 1) * lda + k] = c10;
+      a[(i + 1) * lda + k + 1] = c11;
     }
     __syncthreads();
   }
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
+  for (int e = tid; e < nb * nb; e += 256) {
     const int i = e / nb, j = e % nb;
     if (j <= i) M[(size_t)(p0 + i) * ld + p0 + j] = a[i * lda + j];
   }
-  if (threadIdx.x == 0) {
-    lndet[b] += lsum;
-    if (bad) info[b] = 1;
+  if (warp == 0) {
+    double l = 0.0;
+    for (int j = lane; j < nb; j += 32) l += 2.0 * log(piv[j]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    if (lane == 0) {
+      lndet[b] += l;
+      if (bad) info[b] = 1;
+    }
   }
-  if (inv) {
-    // y = L^{-1}: column j solves L y_j = e_j (y_ij = 0 for i < j); L's diagonal is real.  Four
-    // consecutive lanes per column (blockDim.x == 4 NB), each summing every fourth k of a row.
-    double2 *y = a + NB * lda;
-    const int j = threadIdx.x >> 2, part = threadIdx.x & 3;
-    for (int i = 0; i < NB; ++i) {
-      double sr = 0.0, si = 0.0;
-      if (j < nb && i < nb && i > j)
-        for (int k = j + part; k < i; k += 4) {
-          const double2 l = a[i * lda + k], z = y[k * lda + j];
-          sr += l.x * z.x - l.y * z.y;
-          si += l.x * z.y + l.y * z.x;
-        }
-      sr += __shfl_xor_sync(0xffffffffu, sr, 1);
-      si += __shfl_xor_sync(0xffffffffu, si, 1);
-      sr += __shfl_xor_sync(0xffffffffu, sr, 2);
-      si += __shfl_xor_sync(0xffffffffu, si, 2);
-      if (part == 0) {
-        double2 v = make_double2(0.0, 0.0);
-        if (j < nb && i < nb && i >= j) {
-          const double d = a[i * lda + i].x;
-          v = make_double2(((i == j ? 1.0 : 0.0) - sr) / d, -si / d);
-        }
-        y[i * lda + j] = v;
+  if (!inv) return;
+  T *y = a + NB * lda;
+  if (tid < 64) {   // Y_II: thread = column c of its block
+    const int I = tid / KB, c = tid % KB;
+    T v[KB];
+#pragma unroll
+    for (int i = 0; i < KB; ++i) {
+      T s{};
+      if (i == c) set_re(s, 1.0);
+#pragma unroll
+      for (int k = 0; k < i; ++k) sub_mul(s, a[(I * KB + i) * lda + I * KB + k], v[k]);   // v[k] = 0 for k < c
+      v[i] = I * KB + i < nb ? scaled(s, rinv[I * KB + i]) : s;
+    }
+#pragma unroll
+    for (int i = 0; i < KB; ++i) y[(I * KB + i) * lda + I * KB + c] = v[i];
+  }
+  __syncthreads();
+  for (int I = 1; I < NB / KB; ++I) {
+    // S_IJ = -sum_K L_IK Y_KJ, 2 I tasks of 32 elements (half of a block (I, J)): the warps w < I take tasks w and
+    // 2 I - 1 - w, whose sums are equally long together
+    if (warp < I) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int t = h ? 2 * I - 1 - warp : warp, J = t >> 1;
+        const int i = I * KB + (t & 1) * 4 + (lane >> 3), c = J * KB + (lane & 7);
+        T s{};
+        for (int k = J * KB; k < I * KB; ++k) sub_mul(s, a[i * lda + k], y[k * lda + c]);
+        y[i * lda + c] = s;
       }
-      __syncwarp();
     }
     __syncthreads();
-    double2 *Y = inv + (size_t)b * NB * NB;
-    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) Y[e] = y[(e / NB) * lda + e % NB];
+    // Y_IJ = Y_II S_IJ: an element per thread, written after every read
+    T z[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int e = h * 256 + tid;
+      z[h] = T{};
+      if (e < KB * KB * I) {
+        const int i = e & 7, c = e >> 3;
+        for (int k = 0; k <= i; ++k) sub_mul(z[h], y[(I * KB + i) * lda + I * KB + k], y[(I * KB + k) * lda + c]);
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int e = h * 256 + tid;
+      if (e < KB * KB * I) y[(I * KB + (e & 7)) * lda + (e >> 3)] = scaled(z[h], -1.0);
+    }
+    __syncthreads();
+  }
+  T *Y = inv + (size_t)b * NB * NB;
+  for (int e = tid; e < NB * NB; e += 256) {
+    const int i = e / NB, j = e % NB;
+    Y[e] = j <= i && i < nb ? y[i * lda + j] : T{};
   }
 }
 
-// Panel solve: rows i >= p0 + NB, X L_pp^H = B  =>  x_j = (b_j - sum_{k<j} x_k conj(L_jk)) / L_jj.
-// One CTA per (matrix, 64-row chunk); one thread per row.
-__global__ void __launch_bounds__(64) k_trsm_panel(double2 *const *mats, int n, int ld, int p0) {
-  extern __shared__ double2 tsm[];
-  double2(*L)[NB + 1] = reinterpret_cast<double2(*)[NB + 1]>(tsm);
-  double2(*X)[NB + 1] = reinterpret_cast<double2(*)[NB + 1]>(tsm + NB * (NB + 1));
-  const int b = blockIdx.y;
-  double2 *M = mats[b];
-  const int nb = min(NB, n - p0);
-  const int r0 = p0 + nb + blockIdx.x * 64;
-  if (r0 >= n) return;
-  for (int e = threadIdx.x; e < nb * nb; e += 64) {
-    const int i = e / nb, j = e % nb;
-    L[i][j] = M[(size_t)(p0 + i) * ld + p0 + j];
+// Panel solve by substitution: rows i >= p0 + nb, X L_pp^H = B  =>  x_j = (b_j - sum_{k<j} x_k conj(L_jk)) / L_jj, 16
+// rows per CTA (so that the few matrices of V(q) fill the SMs), columns in blocks of 8.  Graphene slab, one
+// matrix of order 2010: 465 -> ~45 us per panel against 64 rows per CTA, a row per thread.
+constexpr int TR = 16;
+template <class T>
+__global__ void __launch_bounds__(128) k_trsm_panel(T *const *mats, int n, int ld, int p0) {
+  extern __shared__ __align__(16) unsigned char sm_trsm[];
+  constexpr int lda = NB + 1;
+  T *L = reinterpret_cast<T *>(sm_trsm), *X = L + NB * lda;   // [NB][NB + 1], [TR][NB + 1]
+  __shared__ double rinv[NB];
+  T *M = mats[blockIdx.y];
+  const int nb = min(NB, n - p0), r0 = p0 + nb + blockIdx.x * TR, rows = min(TR, n - r0), tid = threadIdx.x;
+  for (int e = tid; e < NB * NB; e += 128) {
+    const int i = e / NB, j = e % NB;
+    L[i * lda + j] = i < nb && j <= i ? M[(size_t)(p0 + i) * ld + p0 + j] : T{};
   }
-  const int rows = min(64, n - r0);
-  for (int e = threadIdx.x; e < rows * nb; e += 64) {
-    const int i = e / nb, j = e % nb;
-    X[i][j] = M[(size_t)(r0 + i) * ld + p0 + j];
+  for (int e = tid; e < TR * NB; e += 128) {
+    const int i = e / NB, j = e % NB;
+    X[i * lda + j] = i < rows && j < nb ? M[(size_t)(r0 + i) * ld + p0 + j] : T{};
   }
+  if (tid < NB) rinv[tid] = tid < nb ? 1.0 / re_of(M[(size_t)(p0 + tid) * ld + p0 + tid]) : 1.0;
   __syncthreads();
-  const int i = threadIdx.x;
-  if (i < rows) {
-    for (int j = 0; j < nb; ++j) {
-      double2 s = X[i][j];
-      for (int k = 0; k < j; ++k) {
-        const double2 x = X[i][k], l = L[j][k];
-        // s -= x * conj(l)
-        s.x -= x.x * l.x + x.y * l.y;
-        s.y -= x.y * l.x - x.x * l.y;
+  const int r = tid & (TR - 1), cg = tid / TR;   // row, and one of 8 columns in turn
+  for (int j0 = 0; j0 < nb; j0 += KB) {
+    T x[KB];
+    if (cg == 0) {
+#pragma unroll
+      for (int j = 0; j < KB; ++j) {
+        x[j] = X[r * lda + j0 + j];
+#pragma unroll
+        for (int k = 0; k < j; ++k) sub_mul_conj(x[j], x[k], L[(j0 + j) * lda + j0 + k]);
+        x[j] = scaled(x[j], rinv[j0 + j]);
       }
-      const double inv = 1.0 / L[j][j].x;
-      X[i][j] = make_double2(s.x * inv, s.y * inv);
+#pragma unroll
+      for (int j = 0; j < KB; ++j) X[r * lda + j0 + j] = x[j];
     }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < KB; ++j) x[j] = X[r * lda + j0 + j];
+    for (int c = j0 + KB + cg; c < nb; c += 128 / TR) {
+      T s = X[r * lda + c];
+#pragma unroll
+      for (int j = 0; j < KB; ++j) sub_mul_conj(s, x[j], L[c * lda + j0 + j]);
+      X[r * lda + c] = s;
+    }
+    __syncthreads();
   }
-  __syncthreads();
-  for (int e = threadIdx.x; e < rows * nb; e += 64) {
-    const int r = e / nb, j = e % nb;
-    M[(size_t)(r0 + r) * ld + p0 + j] = X[r][j];
+  for (int e = tid; e < rows * NB; e += 128) {
+    const int i = e / NB, j = e % NB;
+    if (j < nb) M[(size_t)(r0 + i) * ld + p0 + j] = X[i * lda + j];
   }
+}
+
+template <class T>
+constexpr size_t potrf_smem(bool inv) { return (size_t)(inv ? 2 : 1) * NB * (NB + 1) * sizeof(T); }
+template <class T>
+constexpr size_t trsm_smem() { return (size_t)(NB + TR) * (NB + 1) * sizeof(T); }
+
+template <class T>
+void launch_potrf(T *const *mats, int B, int n, int ld, int p0, double *lndet, int *info, T *inv, cudaStream_t s) {
+  LR_CUDA(cudaFuncSetAttribute(k_potrf_diag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)potrf_smem<T>(true)));
+  k_potrf_diag<T><<<B, 256, potrf_smem<T>(inv != nullptr), s>>>(mats, n, ld, p0, lndet, info, inv);
+  ++launch_counter();
+}
+template <class T>
+void launch_trsm(T *const *mats, int B, int n, int ld, int p0, int rest, cudaStream_t s) {
+  LR_CUDA(cudaFuncSetAttribute(k_trsm_panel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)trsm_smem<T>()));
+  k_trsm_panel<T><<<dim3((unsigned)((rest + TR - 1) / TR), (unsigned)B), 128, trsm_smem<T>(), s>>>(mats, n, ld, p0);
+  ++launch_counter();
 }
 
 // Zero the strict upper triangle (so a Cholesky factor can be used as a triangular operand).
@@ -298,92 +447,6 @@ __global__ void __launch_bounds__(128) k_dgemm_tri(const RGemm *__restrict__ gs,
   }
 }
 
-// Real diagonal-block Cholesky (as k_potrf_diag, real arithmetic).
-__global__ void __launch_bounds__(256) k_potrf_diag_r(double *const *mats, int n, int ld, int p0, double *lndet,
-                                                      int *info) {
-  extern __shared__ double ar[];   // [NB][NB + 1]
-  const int b = blockIdx.x;
-  double *M = mats[b];
-  const int nb = min(NB, n - p0);
-  const int lda = NB + 1;
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    const int i = e / nb, j = e % nb;
-    ar[i * lda + j] = j <= i ? M[(size_t)(p0 + i) * ld + p0 + j] : 0.0;
-  }
-  __syncthreads();
-  __shared__ double dsh;
-  __shared__ int bad;
-  if (threadIdx.x == 0) bad = 0;
-  double lsum = 0.0;
-  for (int j = 0; j < nb; ++j) {
-    if (threadIdx.x == 0) {
-      double d = ar[j * lda + j];
-      if (!(d > 0.0) || !isfinite(d)) {
-        bad = 1;
-        d = 1.0;
-      }
-      d = sqrt(d);
-      ar[j * lda + j] = d;
-      lsum += 2.0 * log(d);
-      dsh = d;
-    }
-    __syncthreads();
-    const double inv = 1.0 / dsh;
-    for (int i = j + 1 + threadIdx.x; i < nb; i += blockDim.x) ar[i * lda + j] *= inv;
-    __syncthreads();
-    const int m = nb - j - 1;
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-      const int i = j + 1 + e / m, k = j + 1 + e % m;
-      if (k > i) continue;
-      ar[i * lda + k] -= ar[i * lda + j] * ar[k * lda + j];
-    }
-    __syncthreads();
-  }
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    const int i = e / nb, j = e % nb;
-    if (j <= i) M[(size_t)(p0 + i) * ld + p0 + j] = ar[i * lda + j];
-  }
-  if (threadIdx.x == 0) {
-    lndet[b] += lsum;
-    if (bad) info[b] = 1;
-  }
-}
-
-// Real panel solve X L_pp^T = B (as k_trsm_panel, real arithmetic).
-__global__ void __launch_bounds__(64) k_trsm_panel_r(double *const *mats, int n, int ld, int p0) {
-  extern __shared__ double tr[];
-  double(*L)[NB + 1] = reinterpret_cast<double(*)[NB + 1]>(tr);
-  double(*X)[NB + 1] = reinterpret_cast<double(*)[NB + 1]>(tr + NB * (NB + 1));
-  const int b = blockIdx.y;
-  double *M = mats[b];
-  const int nb = min(NB, n - p0);
-  const int r0 = p0 + nb + blockIdx.x * 64;
-  if (r0 >= n) return;
-  for (int e = threadIdx.x; e < nb * nb; e += 64) {
-    const int i = e / nb, j = e % nb;
-    L[i][j] = M[(size_t)(p0 + i) * ld + p0 + j];
-  }
-  const int rows = min(64, n - r0);
-  for (int e = threadIdx.x; e < rows * nb; e += 64) {
-    const int i = e / nb, j = e % nb;
-    X[i][j] = M[(size_t)(r0 + i) * ld + p0 + j];
-  }
-  __syncthreads();
-  const int i = threadIdx.x;
-  if (i < rows) {
-    for (int j = 0; j < nb; ++j) {
-      double sv = X[i][j];
-      for (int k = 0; k < j; ++k) sv -= X[i][k] * L[j][k];
-      X[i][j] = sv / L[j][j];
-    }
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < rows * nb; e += 64) {
-    const int r = e / nb, j = e % nb;
-    M[(size_t)(r0 + r) * ld + p0 + j] = X[r][j];
-  }
-}
-
 // A = -L^T chi0 L on entry: trace[b] = -sum A_ii, then A_ii += 1 (real route).
 __global__ void k_diag_shift_r(double *const *mats, int n, int ld, double *trace) {
   double *M = mats[blockIdx.x];
@@ -462,17 +525,12 @@ void potrf_batched(Handle &h, double2 *const *d_mats, const std::vector<double2 
                    double *lndet, int *info, TcScratch *tc, bool inv_panel = false) {
   cudaStream_t s = h.stream;
   const int B = (int)mats.size();
-  const size_t smem = (size_t)NB * (NB + 1) * sizeof(double2);
   const bool use_inv = tc && inv_panel && tc->inv;
-  LR_CUDA(cudaFuncSetAttribute(k_potrf_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * smem)));
-  LR_CUDA(cudaFuncSetAttribute(k_trsm_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * smem)));
   const long long bstride = B > 1 ? (long long)(mats[1] - mats[0]) : 0;
   for (int p0 = 0; p0 < n; p0 += NB) {
     const int nb = std::min(NB, n - p0), rest = n - p0 - nb;
     const bool inv_now = use_inv && rest > 0;
-    k_potrf_diag<<<B, 256, inv_now ? 2 * smem : smem, s>>>(d_mats, n, ld, p0, lndet, info,
-                                                          inv_now ? tc->inv : nullptr);
-    ++launch_counter();
+    launch_potrf<double2>(d_mats, B, n, ld, p0, lndet, info, inv_now ? tc->inv : nullptr, s);
     if (rest <= 0) break;
     if (inv_now) {
       // X = B L_pp^{-H}: stacked real GEMM over the B matrices, K' = 2 nb, written over B
@@ -496,9 +554,7 @@ void potrf_batched(Handle &h, double2 *const *d_mats, const std::vector<double2 
       LR_CUDA(cudaEventRecord(tm.b, s));
       h.timed.push_back(tm);
     } else {
-      dim3 g((unsigned)((rest + 63) / 64), (unsigned)B);
-      k_trsm_panel<<<g, 64, 2 * smem, s>>>(d_mats, n, ld, p0);
-      ++launch_counter();
+      launch_trsm<double2>(d_mats, B, n, ld, p0, rest, s);
     }
     // algorithmic work: the lower triangle (with diagonal) of a rest x rest update of rank nb
     const double fl = 8.0 * B * (0.5 * rest * (rest + 1.0)) * nb;
@@ -589,25 +645,42 @@ void rgemm_batched(Handle &h, const std::vector<RGemm> &gs, int shape, bool kfro
   LR_CUDA(cudaGetLastError());
 }
 
-// Blocked real Cholesky of `mats` (n x n, lower, in place), in step (as potrf_batched).
-// Real blocked Cholesky (lower, in place).  tc (tensor-core route, uniform matrix stride): the
-// trailing updates as digit-plane GEMMs; otherwise FP64 DMMA.
+// Blocked real Cholesky of `mats` (n x n, lower, in place), in step (as potrf_batched), of matrices
+// I - L^T chi0 L >= I.  tc (tensor-core route, uniform matrix stride): the panels as products with the inverse
+// diagonal block (as inv_panel of potrf_batched) and the trailing updates as digit-plane GEMMs; otherwise
+// substitution and FP64 DMMA.
 void potrf_batched_r(Handle &h, double *const *d_mats, const std::vector<double *> &mats, int n, int ld,
                      double *lndet, int *info, TcScratch *tc = nullptr) {
   cudaStream_t s = h.stream;
   const int B = (int)mats.size();
-  const size_t smem = (size_t)NB * (NB + 1) * sizeof(double);
-  LR_CUDA(cudaFuncSetAttribute(k_potrf_diag_r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  LR_CUDA(cudaFuncSetAttribute(k_trsm_panel_r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * smem)));
   const long long bstride = B > 1 ? (long long)(mats[1] - mats[0]) : 0;
   for (int p0 = 0; p0 < n; p0 += NB) {
-    k_potrf_diag_r<<<B, 256, smem, s>>>(d_mats, n, ld, p0, lndet, info);
-    ++launch_counter();
     const int nb = std::min(NB, n - p0), rest = n - p0 - nb;
+    double *inv = tc && rest > 0 ? (double *)tc->inv : nullptr;
+    launch_potrf<double>(d_mats, B, n, ld, p0, lndet, info, inv, s);
     if (rest <= 0) break;
-    dim3 g((unsigned)((rest + 63) / 64), (unsigned)B);
-    k_trsm_panel_r<<<g, 64, 2 * smem, s>>>(d_mats, n, ld, p0);
-    ++launch_counter();
+    if (tc) {
+      // X = B L_pp^{-T} with 8 digit planes (the substitution it stands for is FP64), written over B
+      double *P = mats[0] + (size_t)(p0 + nb) * ld + p0;
+      oz::sliced_bind(tc->pa, tc->pa.digits, rest * B, nb, oz::S_WIDE);
+      oz::sliced_bind(tc->pi, tc->pi.digits, nb * B, nb, oz::S_WIDE);
+      oz::split_real(P, ld, false, rest, nb, B, bstride, tc->pa, s);
+      oz::split_real(inv, NB, false, nb, nb, B, (long long)NB * NB, tc->pi, s);
+      oz::Out o;
+      o.C = P;
+      o.ldc = ld;
+      o.batch_stride = bstride;
+      o.mode = 0;
+      Handle::Timed tm{nullptr, nullptr, 2.0 * B * rest * 0.5 * nb * nb, 1};
+      LR_CUDA(cudaEventCreate(&tm.a));
+      LR_CUDA(cudaEventCreate(&tm.b));
+      LR_CUDA(cudaEventRecord(tm.a, s));
+      oz::gemm(tc->pa, tc->pi, rest, nb, B, o, 0, 0, 0, tc->err, s, h);
+      LR_CUDA(cudaEventRecord(tm.b, s));
+      h.timed.push_back(tm);
+    } else {
+      launch_trsm<double>(d_mats, B, n, ld, p0, rest, s);
+    }
     const double fl = 2.0 * B * (0.5 * rest * (rest + 1.0)) * nb;
     if (tc) {
       // A22 -= P P^T on the lower tiles, P = A[p0+nb.., p0..p0+nb): one operand in both roles

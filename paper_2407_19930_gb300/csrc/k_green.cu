@@ -46,39 +46,58 @@ __global__ void k_weights(const double *eig, const double *occ, double mu, doubl
   w[nkb + x] = f < 1.0 ? (1.0 - f) * exp(-(e - mu) * tau) : 0.0;
 }
 
-// G[g][R][i][j] (slab of one tau) from the lower triangles of P[g][k] (Hermitian).
-// One thread per (g, i, j); twiddle[k][R] = e^{-i 2 pi k.R}.
-__global__ void k_phase_sum(const double2 *P, const double2 *twiddle, int nk, int nR, int nao,
-                            double inv_nk, double *G, size_t g_stride, unsigned long long *maxabs) {
+// G[g][R][i][j] (slab of one tau) from the lower triangles of P[g][k] (Hermitian), with twiddle[k][R] = e^{-i 2 pi k.R}.
+// One thread per (g, i, j) and, by blockIdx.y, per pair R, -R of the list rl (R <= -R: {R, -R}): with t = c + i s the
+// two cells share the sums of p.x c, p.y s, p.x s and p.y c, half the FP64 flops of a cell at a time.
+// FP64-bound: 4 fused multiply-adds per k and pair (graphene slab, 16 k: 976 -> ~500 us a tau).  The largest
+// |Re| and |Im| go through the warp, one atomic each.
+__global__ void __launch_bounds__(256) k_phase_sum(const double2 *__restrict__ P, const double2 *__restrict__ twiddle,
+                                                   const int2 *__restrict__ rl, int nk, int nR, int nao, double inv_nk,
+                                                   double *__restrict__ G, size_t g_stride, unsigned long long *maxabs) {
   const size_t n2 = (size_t)nao * nao;
   const size_t x = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= 2 * n2) return;
-  const int g = (int)(x / n2);
-  const size_t ij = x % n2;
-  const int i = (int)(ij / nao), j = (int)(ij % nao);
-  const bool lower = i >= j;
-  const size_t src = lower ? ij : (size_t)j * nao + i;
+  const int2 R = rl[blockIdx.y];
   double mre = 0.0, mim = 0.0;
-  for (int R = 0; R < nR; ++R) {
-    double re = 0.0, im = 0.0;
+  if (x < 2 * n2) {
+    const int g = (int)(x / n2);
+    const size_t ij = x % n2;
+    const int i = (int)(ij / nao), j = (int)(ij % nao);
+    const bool lower = i >= j;
+    const double2 *p0 = P + (size_t)g * nk * n2 + (lower ? ij : (size_t)j * nao + i);
+    double xc = 0.0, ys = 0.0, xs = 0.0, yc = 0.0;
+#pragma unroll 4
     for (int k = 0; k < nk; ++k) {
-      double2 p = P[((size_t)g * nk + k) * n2 + src];
-      if (!lower) p.y = -p.y;
-      const double2 t = twiddle[(size_t)k * nR + R];
-      re = fma(p.x, t.x, re);
-      re = fma(-p.y, t.y, re);
-      im = fma(p.x, t.y, im);
-      im = fma(p.y, t.x, im);
+      const double2 p = p0[(size_t)k * n2], t = twiddle[(size_t)k * nR + R.x];
+      xc = fma(p.x, t.x, xc);
+      ys = fma(p.y, t.y, ys);
+      xs = fma(p.x, t.y, xs);
+      yc = fma(p.y, t.x, yc);
     }
-    re *= inv_nk;
-    im *= inv_nk;
-    G[(size_t)g * g_stride + (size_t)R * n2 + ij] = re;
-    mre = fmax(mre, fabs(re));
-    mim = fmax(mim, fabs(im));
+    if (!lower) {   // conj P
+      ys = -ys;
+      yc = -yc;
+    }
+    double *out = G + (size_t)g * g_stride + ij;
+    const double re = (xc - ys) * inv_nk, im = (xs + yc) * inv_nk;
+    out[(size_t)R.x * n2] = re;
+    mre = fabs(re);
+    mim = fabs(im);
+    if (R.y != R.x) {
+      const double re2 = (xc + ys) * inv_nk, im2 = (yc - xs) * inv_nk;
+      out[(size_t)R.y * n2] = re2;
+      mre = fmax(mre, fabs(re2));
+      mim = fmax(mim, fabs(im2));
+    }
   }
-  // non-negative doubles order like their bit patterns
-  atomicMax(&maxabs[0], __double_as_longlong(mre));
-  atomicMax(&maxabs[1], __double_as_longlong(mim));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    mre = fmax(mre, __shfl_xor_sync(0xffffffffu, mre, o));
+    mim = fmax(mim, __shfl_xor_sync(0xffffffffu, mim, o));
+  }
+  if ((threadIdx.x & 31) == 0) {   // non-negative doubles order like their bit patterns
+    atomicMax(&maxabs[0], __double_as_longlong(mre));
+    atomicMax(&maxabs[1], __double_as_longlong(mim));
+  }
 }
 
 // Green's-function block screening (Sec. 5): the atom-pair block G^g_{IJ}(R, tau) is zeroed when
@@ -144,7 +163,7 @@ size_t green_work_bytes(const Handle &h) {
   const size_t nk = h.mesh.size(), nR = nk, nb = h.nao, n2 = (size_t)h.nao * h.nao;
   const size_t b_e = nk * nb * 8, b_w = 2 * b_e, b_p = 2 * nk * n2 * 16, b_t = nk * nR * 16;
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-  size_t b = al(b_w) + al(b_p) + al(b_t) + 256;
+  size_t b = al(b_w) + al(b_p) + al(b_t) + al(nR * sizeof(int2)) + 256;
   const int S = green_planes(h);
   if (S >= 0)   // digit planes: Y and the digit planes of both GEMM roles
     b += al(b_p) + oz::sliced_bytes((int)(2 * nk * 2 * h.nao), (int)(2 * nb), S) +
@@ -162,7 +181,8 @@ double green_build(Handle &h) {
   const size_t b_e = (size_t)nk * nb * 8, b_w = 2 * b_e, b_p = 2 * (size_t)nk * n2 * 16,
                b_t = (size_t)nk * nR * 16;
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-  const size_t o_w = 0, o_p = o_w + al(b_w), o_t = o_p + al(b_p), o_m = o_t + al(b_t);
+  const size_t b_rl = (size_t)nR * sizeof(int2);
+  const size_t o_w = 0, o_p = o_w + al(b_w), o_t = o_p + al(b_p), o_rl = o_t + al(b_t), o_m = o_rl + al(b_rl);
   // digit planes: P^g_k = Y^T conj(Y) as one batched digit-plane GEMM per tau (FP64-accurate)
   const int S = green_planes(h);
   const bool tc = S >= 0;
@@ -200,7 +220,11 @@ double green_build(Handle &h) {
     }
   }
   LR_CUDA(cudaMemcpyAsync(d_tw, tw.data(), b_t, cudaMemcpyHostToDevice, s));
-  LR_CUDA(cudaStreamSynchronize(s));   // tw is a host temporary
+  std::vector<int2> rl;   // the cells R <= -R with their partners
+  for (int R : chi0_r_list(h.mesh)) rl.push_back(make_int2(R, h.mesh.neg(R)));
+  int2 *d_rl = (int2 *)(wk + o_rl);
+  LR_CUDA(cudaMemcpyAsync(d_rl, rl.data(), rl.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
+  LR_CUDA(cudaStreamSynchronize(s));   // tw and rl are host temporaries
   LR_CUDA(cudaMemsetAsync(d_max, 0, 16, s));
   const size_t g_stride = (size_t)ntau * nR * n2;
   for (int sp = 0; sp < h.nspins; ++sp) {   // one spin channel at a time, own KS data, own G
@@ -215,6 +239,12 @@ double green_build(Handle &h) {
         if (f > 0) { olo[k] = std::min(olo[k], n); ohi[k] = n + 1; }
         if (f < 1) { vlo[k] = std::min(vlo[k], n); vhi[k] = n + 1; }
       }
+    auto phase_sum = [&](int it) {
+      k_phase_sum<<<dim3((unsigned)((2 * n2 + 255) / 256), (unsigned)rl.size()), 256, 0, s>>>(
+          d_P, d_tw, d_rl, nk, nR, nao, 1.0 / nk, d_gs + (size_t)it * nR * n2, g_stride, d_max);
+      ++launch_counter();
+      LR_CUDA(cudaGetLastError());
+    };
     for (int it = 0; it < ntau; ++it) {
       k_weights<<<(nk * nb + 255) / 256, 256, 0, s>>>(d_eig, d_occ, mu, h.tau[it], nk * nb, d_w);
       ++launch_counter();
@@ -231,11 +261,7 @@ double green_build(Handle &h) {
         o.batch_stride = (long long)n2;
         o.mode = 1;
         oz::gemm(sa, sb, 2 * nao, nao, 2 * nk, o, 0, 0, 2, d_err, s, h);
-        const size_t nthr = 2 * n2;
-        k_phase_sum<<<(unsigned)((nthr + 255) / 256), 256, 0, s>>>(d_P, d_tw, nk, nR, nao, 1.0 / nk,
-                                                                  d_gs + (size_t)it * nR * n2, g_stride, d_max);
-        ++launch_counter();
-        LR_CUDA(cudaGetLastError());
+        phase_sum(it);
         continue;
       }
       std::vector<ZGemm> batch;
@@ -265,11 +291,7 @@ double green_build(Handle &h) {
       f.conjB = true;    // B = conj(wfc) stored [band][j]
       f.lower_only = true;
       zgemm_batched(batch, f, s, h);
-      const size_t nthr = 2 * n2;
-      k_phase_sum<<<(unsigned)((nthr + 255) / 256), 256, 0, s>>>(d_P, d_tw, nk, nR, nao, 1.0 / nk,
-                                                                d_gs + (size_t)it * nR * n2, g_stride, d_max);
-      ++launch_counter();
-      LR_CUDA(cudaGetLastError());
+      phase_sum(it);
     }
   }
   unsigned long long mx[2];

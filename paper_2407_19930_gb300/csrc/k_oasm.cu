@@ -58,11 +58,6 @@ __device__ __forceinline__ void tc_digits(float h, float l, float sc7, float sc1
   }
 }
 
-__device__ __forceinline__ unsigned pack_bf16(float a, float b) {
-  __nv_bfloat162 v = __floats2bfloat162_rn(a, b);   // small integers: exact
-  return *reinterpret_cast<unsigned *>(&v);
-}
-
 // The element type of the operands: (hi, lo) FP32 pairs with up to 5 planes (N and X arrive so from their GEMMs, G as
 // FP64 turned into pairs; the low part joins the digits after the second, error below 2^-39 of the row
 // maximum), FP64 numbers with 8 planes.
@@ -108,11 +103,11 @@ struct Elem<oz::S_WIDE> {
     unsigned *u = reinterpret_cast<unsigned *>(w);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      int d0[S], d1[S];
+      float d0[S], d1[S];
       make_digits<S>(v[2 * q], E, d0);
       make_digits<S>(v[2 * q + 1], E, d1);
 #pragma unroll
-      for (int s = 0; s < S; ++s) u[4 * s + q] = pack_bf16((float)d0[s], (float)d1[s]);
+      for (int s = 0; s < S; ++s) u[4 * s + q] = pack_bf16(d0[s], d1[s]);
     }
   }
 };
@@ -199,50 +194,38 @@ __host__ __device__ constexpr int smem_size(int S) { return (1 + ring(S)) * stag
 __host__ __device__ constexpr int slot_cols(int S) { return 2 * S * kMaxAo; }         // TMEM columns of one nu: two terms, S diagonals, 16 i
 __host__ __device__ constexpr int slots(int S) { return 512 / slot_cols(S); }
 
-__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t *r) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_wait4(uint32_t *r) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3])::"memory");
+// sum_d A_d 2^{8(N-1-d)} of N exact integer-valued FP32 diagonal sums (|A_d| <= 2^22): the bits of A_d + 1.5 2^23
+// are A_d plus a constant, so the constants are subtracted from the sum once (mod 2^64)
+template <int N>
+__device__ __forceinline__ long long fold_sums(const uint32_t *a) {
+  constexpr unsigned long long kOne = 0x4B400000ull;
+  unsigned long long c = 0, T = 0;
+#pragma unroll
+  for (int d = 0; d < N; ++d) {
+    const unsigned b = __float_as_uint(__uint_as_float(a[4 * d]) + kRintMagic);
+    c += kOne << (8 * (N - 1 - d));
+    T += (unsigned long long)b << (8 * (N - 1 - d));
+  }
+  return (long long)(T - c);
 }
 
-__device__ __forceinline__ int rint_sum(uint32_t f) {   // an integer-valued FP32 sum, |f| <= 2^22
-  return (int)((unsigned)__float_as_int(__uint_as_float(f) + kRintMagic) - 0x4B400000u);
-}
-
-// element (x) of the two terms' sums r1, r2 ([diagonal][4] registers), scales 2^E1, 2^E2
+// element x of the two terms' sums r1, r2 ([diagonal][4] registers), scales 2^E1, 2^E2
 template <int S>
 __device__ __forceinline__ double combine(const uint32_t (&r1)[S][4], const uint32_t (&r2)[S][4], int x, int E1, int E2) {
   if constexpr (S == oz::S_WIDE) {
-    long long h1 = 0, l1 = 0, h2 = 0, l2 = 0;
-#pragma unroll
-    for (int d = 0; d < 4; ++d) {
-      h1 += (long long)rint_sum(r1[d][x]) * (1 << (8 * (3 - d)));
-      l1 += (long long)rint_sum(r1[d + 4][x]) * (1 << (8 * (3 - d)));
-      h2 += (long long)rint_sum(r2[d][x]) * (1 << (8 * (3 - d)));
-      l2 += (long long)rint_sum(r2[d + 4][x]) * (1 << (8 * (3 - d)));
-    }
-    return i96_to_f64(h1, l1, E1 - 14 - 56) + i96_to_f64(h2, l2, E2 - 14 - 56);
+    return i96_to_f64(fold_sums<4>(&r1[0][x]), fold_sums<4>(&r1[4][x]), E1 - 14 - 56) +
+           i96_to_f64(fold_sums<4>(&r2[0][x]), fold_sums<4>(&r2[4][x]), E2 - 14 - 56);
   } else {
-    long long T1 = rint_sum(r1[S - 1][x]), T2 = rint_sum(r2[S - 1][x]);
-#pragma unroll
-    for (int d = 0; d < S - 1; ++d) {
-      if (S == 5 && d == 0) {
-        T1 += (long long)((unsigned long long)(unsigned)rint_sum(r1[d][x]) << 32);
-        T2 += (long long)((unsigned long long)(unsigned)rint_sum(r2[d][x]) << 32);
-      } else {
-        T1 += (long long)rint_sum(r1[d][x]) * (1 << (8 * (S - 1 - d) % 32));
-        T2 += (long long)rint_sum(r2[d][x]) * (1 << (8 * (S - 1 - d) % 32));
-      }
-    }
-    // the smaller scale's sum rounded to the larger scale
+    const long long T1 = fold_sums<S>(&r1[0][x]), T2 = fold_sums<S>(&r2[0][x]);
+    // the smaller scale's sum rounded to the larger scale, half up
     const bool one = E1 >= E2;
     const long long big = one ? T1 : T2, small = one ? T2 : T1;
-    const int sh = min(one ? E1 - E2 : E2 - E1, 62);
-    const long long T = big + ((small + (long long)((1ull << sh) >> 1)) >> sh);
-    return i64_to_f64(T, (one ? E1 : E2) - 14 - 8 * (S - 1));
+    const int E = max(E1, E2), sh = min(E - min(E1, E2), 62);
+    const long long T = big + ((((small << 1) >> sh) + 1) >> 1);
+    // the conversion on the FP64 pipe, which is idle otherwise (one instruction in place of ~25); the scales are
+    // within 2^+-200 (tc_expo), far from the ends of the exponent range
+    const long long bits = __double_as_longlong((double)T) + ((long long)(E - 14 - 8 * (S - 1)) << 52);
+    return __longlong_as_double(T == 0 ? 0ll : bits);
   }
 }
 
@@ -267,7 +250,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nU = a.n_ao[U], nV = a.n_ao[V], two = 2 * nV, nauxV = a.n_aux[V], mU = a.m[U];
   double *Ob = a.O + p * a.o_sz_p + a.o_off[U];
-  const int ldo = nU * mU;
+  const int ldo = o_pitch(nU, mU);
   if (a.zero) {   // under screening: a tile whose 64-column chunks are all exactly zero
     const Group g0 = tb.groups[(size_t)tile * kTileGroups];
     int k1 = g0.kap;
@@ -375,7 +358,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tmem = tmem_slot;
   const long long nu0 = (long long)p * a.naux + a.aux_off[V];
   if (warp == kEpi) {
-    if (lane == 0) {   // TMA producer: N rows of the tile's groups and the 16 X rows of U, per nu
+    if (elect_one()) {   // TMA producer: N rows of the tile's groups and the 16 X rows of U, per nu
       const int ng = s_groups;
       int it = 0;
       for (; it < nauxV; ++it) {
@@ -395,7 +378,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int i = it > NST ? it - NST : 0; i < it; ++i) mbar_wait(&full[i % NST], (uint32_t)((i / NST) & 1), WAIT_NS);
     }
   } else if (warp == kEpi + 1) {
-    if (lane == 0) {   // MMA issuer
+    if (elect_one()) {   // MMA issuer
       const int ks = (two + 15) / 16;
       const uint32_t rg = smem_u32(sRG), lm = smem_u32(sLm);
       for (int it = 0; it < nauxV; ++it) {
@@ -410,13 +393,22 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         tc_fence_after();
         const uint32_t sn = smem_u32(smem + STAGE + st * STAGE), sx = sn + OPB, d = tmem + sl * SL;
-        for (int j = 0; j < ks; ++j)
+        const uint64_t dn = smem_desc64(sn, S * 512), dr = smem_desc64(rg, S * 512), dl = smem_desc64(lm), dx = smem_desc64(sx);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          if (j >= ks) break;
 #pragma unroll
           for (int s = 0; s < S; ++s) {   // plane s of A by planes 0 .. S - 1 - s of B, into the diagonals s ..
-            const uint32_t ide = idesc(kMaxAo * (S - s), false), acc = (j == 0 && s == 0) ? 0u : 1u;
-            umma(d + s * kMaxAo, smem_desc64(sn + s * 512 + 32 * j, S * 512), smem_desc64(lm + 32 * j), ide, acc);
-            umma(d + (S + s) * kMaxAo, smem_desc64(rg + s * 512 + 32 * j, S * 512), smem_desc64(sx + 32 * j), ide, acc);
+            const uint32_t ide = idesc(kMaxAo * (S - s), false), o = (s * 512 + 32 * j) / 16;
+            if (j == 0 && s == 0) {
+              umma(d, dn, dl, ide, 0u);
+              umma(d + S * kMaxAo, dr, dx, ide, 0u);
+            } else {
+              umma_add(d + s * kMaxAo, dn + o, dl + 2 * j, ide);
+              umma_add(d + (S + s) * kMaxAo, dr + o, dx + 2 * j, ide);
+            }
           }
+        }
         umma_commit(&empty[st]);
         umma_commit(&tfull[sl]);
       }
@@ -442,7 +434,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         break;
       }
       tc_fence_after();
-      int emax = 0;   // largest biased exponent among this lane's outputs
+      int emax = 0;   // upper word of the largest |output| of this lane: its biased exponent
       if (any) {
         const uint32_t tb0 = tmem + ((uint32_t)(32 * quad) << 16) + sl * SL;
         double *orow = Ob + (size_t)(a.aux_off[V] + it) * ldo + kap;
@@ -454,13 +446,13 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int x = 0; x < 4; ++x) e2[x] = xe[min(c + x, kMaxAo - 1)];
 #pragma unroll
           for (int d = 0; d < S; ++d) {
-            tmem_ld4(tb0 + d * kMaxAo + c, r1[d]);
-            tmem_ld4(tb0 + (S + d) * kMaxAo + c, r2[d]);
+            tmem_ld(tb0 + d * kMaxAo + c, r1[d]);
+            tmem_ld(tb0 + (S + d) * kMaxAo + c, r2[d]);
           }
 #pragma unroll
           for (int d = 0; d < S; ++d) {
-            tmem_wait4(r1[d]);
-            tmem_wait4(r2[d]);
+            tmem_ld_wait(r1[d]);
+            tmem_ld_wait(r2[d]);
           }
 #pragma unroll
           for (int x = 0; x < 4; ++x) {
@@ -470,7 +462,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (S == oz::S_WIDE && max(max(e1, f1), max(e2[x], f2)) > 1024) o = __longlong_as_double(0x7FF8000000000000ll);
             if (kap >= 0) {
               orow[(size_t)(c + x) * mU] = o;
-              emax = max(emax, biased_exp(o));
+              emax = max(emax, __double2hiint(o) & 0x7FFFFFFF);
             }
           }
         }
@@ -479,7 +471,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[sl]);
       // the row (p, U, nu) of the final contraction's O operand
-      emax = __reduce_max_sync(0xffffffffu, emax);
+      emax = __reduce_max_sync(0xffffffffu, emax) >> 20;
       if (lane == 0 && emax > 0) atomicMax(rexp + ((size_t)p * a.natoms + U) * a.naux + a.aux_off[V] + it, emax - 1022);
     }
   }
@@ -500,7 +492,7 @@ void launch(const OArgs &a, const Tables &t, int np, oz::Sliced &nd, oz::Sliced 
       a, t.aux_atom, t.ao_row, (__nv_bfloat16 *)xd.digits, xd.expo, (long long)xd.rows * xd.kpad);
   LR_CUDA(cudaFuncSetAttribute(k_oasm<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_size(S)));
   k_oasm<S><<<(unsigned)t.max_tiles * (unsigned)(np * a.natoms * a.natoms), kThreads, smem_size(S), s>>>(
-      a, t, oz::make_map(nd, 8, S), oz::make_map(xd, kMaxAo, S), nd.expo, xd.expo, expo, err);
+      a, t, oz::make_map(nd, 8, S, 64), oz::make_map(xd, kMaxAo, S, 64), nd.expo, xd.expo, expo, err);
   launch_counter() += 3;
   LR_CUDA(cudaGetLastError());
 }

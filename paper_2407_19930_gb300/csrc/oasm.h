@@ -13,6 +13,9 @@ struct Point {
   int R[3];
 };
 
+// Row pitch of O_U (rows nu, columns (i, kap)): n_U m_U rounded up to even, so that rows start on 16 bytes.
+__host__ __device__ constexpr int o_pitch(int n, int m) { return (n * m + 1) & ~1; }
+
 // Operands of the O assembly: O^nu_{ik}(K R1) for every (point, U, V), written as O_U[nu][(i, kap)].
 struct OArgs {
   const double *G;       // [2][ntau][nR][nao][nao]

@@ -75,10 +75,14 @@ struct GatherSrc {
   const int *lam;        // per-atom column tables (6 ints per column)
   const long long *lam_off;
   const int *m;          // m_V
+  // the same column tables with the lattice vectors folded into the BvK cell, {R0 | R1 << 8 | R2 << 16, ao}, or NULL
+  // (a mesh dimension above 255): lam's columns and the union's
+  const int2 *lamf, *unif;
 };
 void split_gather(const GatherSrc &src, int rows, int K, Sliced &out, cudaStream_t s);
 //  ragged entries: row r belongs to entry e = r / rows_per_entry; its K_e columns are
-//  base[off[e] + (r % rows_per_entry) * K_e + k] (zero for k >= K_e); off, K on the device.
+//  base[off[e] + (r % rows_per_entry) * P_e + k] (zero for k >= K_e), P_e = K_e rounded up to even; off, K on the
+//  device.
 //  expo_given: out.expo already holds each row's exponent (its largest biased FP64 exponent
 //  minus 1022, as the exponent pass would write it), which is then not recomputed.
 void split_ragged(const double *base, const long long *off, const int *Ke, int rows_per_entry, int n_entries,
@@ -138,9 +142,9 @@ long long gemm_multi(const std::vector<std::pair<const Sliced *, const Sliced *>
 long long gemm(const Sliced &a, const Sliced &b, int M, int N, int batch, const Out &out, int km, int kn,
                int lower_div, int *err, cudaStream_t s, Handle &h);
 
-// Tensor map of an operand's planes with boxes of 64 bytes x box_rows rows x box_planes planes (64-byte
-// swizzle); after init().
-CUtensorMap make_map(const Sliced &o, int box_rows, int box_planes = 1);
+// Tensor map of an operand's planes with boxes of row_bytes (64 or 128, the swizzle width) x box_rows rows x
+// box_planes planes; after init().
+CUtensorMap make_map(const Sliced &o, int box_rows, int box_planes, int row_bytes);
 
 // One-time host setup (driver entry point for tensor-map encoding).  Throws on failure.
 void init();

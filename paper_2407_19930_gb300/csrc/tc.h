@@ -15,34 +15,59 @@ namespace {
 
 __device__ __forceinline__ int biased_exp(double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7FF); }
 
-// balanced base-256 digits of x = v 2^-E (|x| < 1): x ~ sum_s d_s 2^{-7-8(s-1)}, |d_s| <= 128
+// balanced base-256 digits of x = v 2^-E (|x| < 1): x ~ sum_s d_s 2^{-7-8(s-1)}, |d_s| <= 128, as FP32 integers.
+// W = x 2^{7+8(S-1)} rounded (half up in magnitude); with 128 added at every lower digit's place the digits are the
+// bytes of the sum less 128, and a byte b becomes a float by the bits of 2^23 + b.
 template <int S>
-__device__ __forceinline__ void make_digits(double v, int E, int (&d)[S]) {
+__device__ __forceinline__ void make_digits(double v, int E, float (&d)[S]) {
   const long long bits = __double_as_longlong(v);
   const int ex = (int)((bits >> 52) & 0x7FF);
-#pragma unroll
-  for (int s = 0; s < S; ++s) d[s] = 0;
-  if (ex == 0) return;   // zero (subnormals are far below any row scale of interest)
-  const long long mant = (bits & 0xFFFFFFFFFFFFFLL) | (1LL << 52);
-  const int r = 1075 + E - 7 - 8 * (S - 1) - ex;   // W = mant 2^-r, r > 0 since |x| < 1
-  long long W = 0;
-  if (r <= 0)
-    W = mant << (-r);
-  else if (r < 62)
-    W = (mant + (1LL << (r - 1))) >> r;
-  if (bits < 0) W = -W;
-#pragma unroll
-  for (int s = S - 1; s >= 1; --s) {
-    const long long dg = ((W + 128) & 255) - 128;
-    d[s] = (int)dg;
-    W = (W - dg) >> 8;
+  const int r = 1075 + E - 7 - 8 * (S - 1) - ex;   // |W| = mant 2^-r
+  const unsigned long long mant = ((unsigned long long)bits & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+  unsigned long long u;
+  if (S < 7)   // r > 0 since |x| < 1
+    u = ((mant >> (r - 1 & 63)) + 1) >> 1;
+  else   // r >= -10
+    u = r + 10 == 0 ? mant << 10 : (((mant << 10) >> (r + 9 & 63)) + 1) >> 1;
+  if (ex == 0 || r > 53) u = 0;   // zero (subnormals are far below any row scale of interest), or below half a unit
+  long long W = bits < 0 ? -(long long)u : (long long)u;
+  unsigned lo, hi = 0;
+  int top;
+  if constexpr (S <= 5) {   // |W| < 2^40
+    constexpr unsigned long long kBias = S == 1 ? 0ull : 0x80808080ull >> (8 * (5 - S));
+    W += (long long)kBias;
+    lo = (unsigned)(unsigned long long)W;
+    top = (int)(W >> (8 * (S - 1)));
+  } else {   // the lower digits apart, so that the sum of W near 2^63 does not overflow
+    static_assert(S <= 5 || S == 8, "make_digits: planes");
+    const unsigned long long l = ((unsigned long long)W & 0xFFFFFFFFFFFFFFull) + 0x80808080808080ull;
+    lo = (unsigned)l;
+    hi = (unsigned)(l >> 32);
+    top = (int)(W >> 56) + (int)(l >> 56);
   }
-  d[0] = (int)W;
+  d[0] = __int_as_float(top + 0x4B400000) - 12582912.f;
+#pragma unroll
+  for (int s = 1; s < S; ++s) {
+    const int byte = S - 1 - s;   // place of digit s
+    d[s] = __uint_as_float(__byte_perm(byte < 4 ? lo : hi, 0x4B000000u, 0x7440 + (byte & 3))) - 8388736.f;
+  }
+}
+
+__device__ __forceinline__ unsigned pack_bf16(float a, float b) {
+  __nv_bfloat162 v = __floats2bfloat162_rn(a, b);   // small integers: exact
+  return *reinterpret_cast<unsigned *>(&v);
 }
 
 // ------------------------------------------------------------------ tcgen05 / TMA / mbarrier
 
 constexpr uint64_t WAIT_NS = 2000000000ull;   // 2 s
+
+// one lane of a converged warp (the compiler then knows that a single thread issues the TMA copies and MMAs)
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -112,6 +137,12 @@ __device__ __forceinline__ void umma(uint32_t d, uint64_t a, uint64_t b, uint32_
       ::"r"(d), "l"(a), "l"(b), "r"(desc), "r"(acc)
       : "memory");
 }
+// the same, always adding to the accumulator
+__device__ __forceinline__ void umma_add(uint32_t d, uint64_t a, uint64_t b, uint32_t desc) {
+  asm volatile("{\n .reg .pred p;\n setp.eq.u32 p, 0, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+               ::"r"(d), "l"(a), "l"(b), "r"(desc)
+               : "memory");
+}
 __device__ __forceinline__ void umma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t desc, uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n"
@@ -122,20 +153,30 @@ __device__ __forceinline__ void umma_commit(uint64_t *bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
 }
-// 16 columns of the warp's 32 TMEM lanes; the registers are valid after tmem_ld_wait on them
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
+// 4, 8, 12 or 16 columns of the warp's 32 TMEM lanes; the registers are valid after tmem_ld_wait on them
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t *r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
 }
-__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[16]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-               :
-               : "memory");
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t *r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+template <int N>
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[N]) {
+  static_assert(N == 4 || N == 8 || N == 12 || N == 16, "tmem_ld: columns");
+  if constexpr (N >= 8) tmem_ld8(taddr, r);
+  if constexpr (N == 16) tmem_ld8(taddr + 8, r + 8);
+  if constexpr (N == 12) tmem_ld4(taddr + 8, r + 8);
+  if constexpr (N == 4) tmem_ld4(taddr, r);
+}
+template <int N>
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[N]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int j = 0; j < N; ++j) asm volatile("" : "+r"(r[j]));   // no use of r[j] moves above the wait
 }
 
 // shared-memory matrix descriptor: K-major, 64-byte swizzle, 8-row groups `sbo` bytes apart
@@ -147,6 +188,12 @@ __device__ __forceinline__ uint64_t smem_desc64(uint32_t saddr, uint32_t sbo = 5
   d |= (uint64_t)1 << 46;             // descriptor version
   d |= (uint64_t)4 << 61;             // SWIZZLE_64B
   return d;
+}
+
+// the same with 128-byte swizzle (8-row groups of 1024 bytes)
+__device__ __forceinline__ uint64_t smem_desc128(uint32_t saddr) {
+  return (uint64_t)((saddr & 0x3FFFF) >> 4) | (uint64_t)1 << 16 | (uint64_t)(1024 >> 4) << 32 | (uint64_t)1 << 46 |
+         (uint64_t)2 << 61;
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
@@ -162,7 +209,8 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
 // mant (53 bits, or 2^53 after rounding up) 2^(e - 1075) with e the biased exponent; neg: sign bit
 __device__ __forceinline__ double make_f64(unsigned long long neg, unsigned long long mant, int e) {
   double v = __longlong_as_double((long long)(((unsigned long long)(e - 1) << 52) + mant));
-  if (e <= 0 || e >= 2046) {   // subnormal, overflow or next to it: scale [1, 2) in two exact steps
+  if ((unsigned)(e - 1) >= 2045u) {   // subnormal, overflow or next to it: scale [1, 2) in two exact steps
+    asm volatile("");   // a branch: predicated, its FP64 instructions would cost every element
     const int k = min(1100, max(-1080, e - 1023)), k1 = k / 2, k2 = k - k1;
     v = __longlong_as_double((long long)((1022ull << 52) + mant));
     v = v * __longlong_as_double((long long)(k1 + 1023) << 52) * __longlong_as_double((long long)(k2 + 1023) << 52);
@@ -198,6 +246,7 @@ __device__ __forceinline__ float2 i64_to_f32x2(long long a, int sh) {
   // r = rh 2^20 + rl, both exact in FP32: one rounding
   float lo = fmaf((float)(int)(r >> 20), 1048576.f, (float)(int)(r & 0xFFFFFll)) * __uint_as_float((unsigned)(e + 127) << 23);
   if (e < -126 || e > 63) {   // outside the FP32 range of a direct scaling: through FP64
+    asm volatile("");
     const double v = i64_to_f64(a < 0 ? -a : a, sh);
     hi = __double2float_rn(v);
     lo = __double2float_rn(v - (double)hi);
