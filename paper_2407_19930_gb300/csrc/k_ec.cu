@@ -764,10 +764,11 @@ EcLayout ec_layout(const Handle &h) {
     l.o_sw = take(oz::sliced_bytes(nw * n, 2 * n, S));
     l.o_sl = take(oz::sliced_bytes(n, 2 * n, S));
     l.o_slh = take(oz::sliced_bytes(2 * n, 2 * n, S));
-    l.o_pa = take(oz::sliced_bytes(bmax * 2 * n, 2 * NB, S));
+    // panels and inverse diagonal blocks: complex ones with S planes, those of the real route with 8
+    l.o_pa = take(std::max(oz::sliced_bytes(bmax * 2 * n, 2 * NB, S), oz::sliced_bytes(bmax * n, NB, oz::S_WIDE)));
     l.o_pb = take(oz::sliced_bytes(bmax * n, 2 * NB, S));
     l.o_inv = take((size_t)bmax * NB * NB * sizeof(double2));
-    l.o_pi = take(oz::sliced_bytes(bmax * NB, 2 * NB, S));
+    l.o_pi = take(std::max(oz::sliced_bytes(bmax * NB, 2 * NB, S), oz::sliced_bytes(bmax * NB, NB, oz::S_WIDE)));
   }
   l.total = off;
   return l;
