@@ -68,13 +68,16 @@ __device__ __forceinline__ void sub_mul(double2 &c, double2 a, double2 b) {     
 __device__ __forceinline__ void sub_mul(double &c, double a, double b) { c = fma(-a, b, c); }
 __device__ __forceinline__ double2 scaled(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
 __device__ __forceinline__ double scaled(double a, double s) { return a * s; }
+__device__ __forceinline__ double2 sum(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double sum(double a, double b) { return a + b; }
 __device__ __forceinline__ double re_of(double2 a) { return a.x; }
 __device__ __forceinline__ double re_of(double a) { return a; }
 __device__ __forceinline__ void set_re(double2 &a, double x) { a = make_double2(x, 0.0); }
 __device__ __forceinline__ void set_re(double &a, double x) { a = x; }
 
 // Factor the NB x NB diagonal block at p0 of every matrix in place (lower triangle).  One CTA per
-// matrix.  Adds 2 sum ln d_jj to lndet[b]; sets info[b] = 1 on a non-positive pivot.
+// matrix.  Adds sum ln d_j of the pivots d_j (= L_jj^2) to lndet[b] (of 2 ln L_jj, the square root's rounding is biased
+// downwards for pivots just above 1, which the ln det adds up); sets info[b] = 1 on a non-positive pivot.
 // inv (optional, [matrix][NB][NB]): receives L_pp^{-1} of the factored block (lower triangular, zero elsewhere), by
 // blocks of 8 rows: Y_II = L_II^{-1}, Y_IJ = -Y_II sum_K L_IK Y_KJ.
 // 64 x 64 complex: 268 -> ~75 us (with the inverse 390 -> ~150 us at 96 matrices) against one column at a time.
@@ -106,11 +109,14 @@ __global__ void __launch_bounds__(256) k_potrf_diag(T *const *mats, int n, int l
   for (int j0 = 0; j0 < nb; j0 += KB) {
     if (tid < KB * KB) {   // the 8 x 8 triangle: thread = element (r, k)
       const int r = tid / KB, k = tid % KB;
-      T e = a[(j0 + r) * lda + j0 + k];
+      T e = a[(j0 + r) * lda + j0 + k], s{};   // s: the updates, added once
 #pragma unroll
       for (int j = 0; j < KB; ++j) {
         T *col = colj[j & 1];   // column j before its scaling
-        if (k == j) col[r] = e;
+        if (k == j) {
+          e = sum(e, s);
+          col[r] = e;
+        }
         bar_64();
         double d = re_of(col[j]);
         const bool ok = d > 0.0 && isfinite(d);
@@ -122,13 +128,13 @@ __global__ void __launch_bounds__(256) k_potrf_diag(T *const *mats, int n, int l
             sq = fma(0.5 * ri, fma(-sq, sq, d), sq);   // sqrt(d)
             set_re(e, sq);
             rinv[j0 + j] = ri;
-            piv[j0 + j] = sq;
+            piv[j0 + j] = d;
             if (!ok) bad = 1;
           } else {
             e = scaled(e, ri);
           }
         } else if (k > j && r >= k) {
-          sub_mul_conj(e, scaled(col[r], ri), scaled(col[k], ri));
+          sub_mul_conj(s, scaled(col[r], ri), scaled(col[k], ri));
         }
       }
       if (k <= r) a[(j0 + r) * lda + j0 + k] = e;
@@ -148,14 +154,15 @@ __global__ void __launch_bounds__(256) k_potrf_diag(T *const *mats, int n, int l
       for (int j = 0; j < KB; ++j) row[j] = x[j];
     }
     __syncthreads();
-    // trailing update a_ik -= sum_j a_ij conj(a_kj) in 2 x 2 tiles of the lower triangle
+    // trailing update a_ik -= sum_j a_ij conj(a_kj) in 2 x 2 tiles of the lower triangle; the sums apart: products
+    // below the last place of a diagonal near 1 (high frequencies) would each be lost, always to the same side
     const int mt = m / 2, nt = mt * (mt + 1) / 2;
     for (int t = tid; t < nt; t += 256) {
       int ty = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
       if (ty * (ty + 1) / 2 > t) --ty;
       if ((ty + 1) * (ty + 2) / 2 <= t) ++ty;
       const int tx = t - ty * (ty + 1) / 2, i = c0 + 2 * ty, k = c0 + 2 * tx;
-      T c00 = a[i * lda + k], c01 = a[i * lda + k + 1], c10 = a[(i + 1) * lda + k], c11 = a[(i + 1) * lda + k + 1];
+      T c00{}, c01{}, c10{}, c11{};
 #pragma unroll
       for (int j = 0; j < KB; ++j) {
         const T x0 = a[i * lda + j0 + j], x1 = a[(i + 1) * lda + j0 + j], y0 = a[k * lda + j0 + j],
@@ -165,10 +172,11 @@ __global__ void __launch_bounds__(256) k_potrf_diag(T *const *mats, int n, int l
         sub_mul_conj(c10, x1, y0);
         sub_mul_conj(c11, x1, y1);
       }
-      a[i * lda + k] = c00;
-      if (tx < ty) a[i * lda + k + 1] = c01;   // (the element above the diagonal stays)
-      a[(i + 1) * lda + k] = c10;
-      a[(i + 1) * lda + k + 1] = c11;
+      T *row0 = a + i * lda + k, *row1 = row0 + lda;
+      row0[0] = sum(row0[0], c00);
+      if (tx < ty) row0[1] = sum(row0[1], c01);   // (the element above the diagonal stays)
+      row1[0] = sum(row1[0], c10);
+      row1[1] = sum(row1[1], c11);
     }
     __syncthreads();
   }
@@ -178,7 +186,7 @@ __global__ void __launch_bounds__(256) k_potrf_diag(T *const *mats, int n, int l
   }
   if (warp == 0) {
     double l = 0.0;
-    for (int j = lane; j < nb; j += 32) l += 2.0 * log(piv[j]);
+    for (int j = lane; j < nb; j += 32) l += log(piv[j]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
     if (lane == 0) {
