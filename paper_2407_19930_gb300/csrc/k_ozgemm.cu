@@ -612,8 +612,10 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
     for (int t = blockIdx.x; t < ntiles; t += stride) {
       const Tile &tl = tiles[t];
       const Entry &en = entries[tl.e];
-      asm volatile("prefetch.global.L1 [%0];" ::"l"(&en));
-      asm volatile("prefetch.global.L1 [%0];" ::"l"(&tiles[t + stride < ntiles ? t + stride : t]));
+      const Tile &tn = tiles[t + stride < ntiles ? t + stride : t];   // the next tile's record and exponents to the L1
+      prefetch_l1(&tiles[t + 2 * stride < ntiles ? t + 2 * stride : t]);
+      prefetch_l1(&entries[tn.e]);
+      prefetch_l1(&maps[tn.pair].ea);
       const int nsteps = tl.nsteps;
       const int ngroups = (nsteps + G - 1) / G;
       const int m0 = tl.m0, n0 = tl.n0;
@@ -624,11 +626,11 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
       const bool pow2 = en.alpha_shift != kNoShift;   // alpha = +-2^alpha_shift: folded into the exponent
       const int row = m0 + 32 * quad + lane;          // thread = tile row (the TMEM lane layout)
       const bool row_ok = row < eM;
-      auto at = [&](int r_, int c_) {   // one output element (modes 0, 1, 2, 4)
-        return mode == 0   ? C + (long long)r_ * ldc + c_
-               : mode == 1 ? C + 2 * ((long long)(r_ >> 1) * ldc + c_) + (r_ & 1)
-               : mode == 4 ? C + (long long)c_ * ldc + r_
-                           : C + 2 * ((long long)c_ * ldc + (r_ >> 1)) + (r_ & 1);
+      // output (row, col) at out_row(row) + col cstep
+      const bool trans = mode == 2 || mode == 4;
+      const long long cstep = mode == 4 ? ldc : mode == 2 ? 2 * ldc : mode == 1 ? 2 : 1;
+      auto out_row = [&](int r_) {
+        return trans ? C + r_ : mode == 1 ? C + 2 * (r_ >> 1) * ldc + (r_ & 1) : C + r_ * ldc;
       };
       // digit planes: exact sums of the diagonals, in units of the last one's scale (WIDE: the first four
       // diagonals in acch, in units of the fourth's, the last four in acc)
@@ -639,7 +641,13 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
       const MapPair &mp = maps[tl.pair];
       const int ash = (pow2 ? en.alpha_shift : 0) - 14 - 8 * (S - 1);
       const int ea = PLAIN || !row_ok ? ash : mp.ea[tl.arow + 32 * quad + lane] + ash;
-      const int *eb = mp.eb + tl.brow + half * HALF;
+      // the exponents of the warp's columns, one per lane
+      int eb_lane = 0;
+      auto load_eb = [&] {
+        if (lane < nc) eb_lane = (maps[tl.pair].eb + tl.brow + half * HALF)[lane];
+      };
+      if constexpr (DIRECT) load_eb();
+      auto eb = [&](int j) { return __shfl_sync(0xffffffffu, eb_lane, j); };
       const bool aneg = pow2 && alpha < 0.0;
       // a row or column with an infinity or a NaN has the exponent 1025 (finite ones at most 1024)
       const bool row_nan = ea - ash > 1024;
@@ -656,10 +664,12 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
             v = i96_to_f64(hi, lo, sh);
           else
             v = i64_to_f64(lo, sh);
-          if (!pow2)
+          if (!pow2) {
+            asm volatile("");   // a branch: FP64 instructions cost their place on the pipe even when predicated off
             v *= alpha;
-          else if (aneg)
+          } else if (aneg) {
             v = -v;
+          }
           if (nan) v = __longlong_as_double(0x7FF8000000000000ll);
           if (mode != 3) return __double_as_longlong(v);
           pr.x = __double2float_rn(v);
@@ -668,32 +678,45 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
         if (nan) pr = make_float2(__uint_as_float(0x7FC00000u), 0.f);
         return (long long)(((unsigned long long)__float_as_uint(pr.y) << 32) | __float_as_uint(pr.x));
       };
-      // row-major outputs go through the staging area, lanes along SC columns, then rows
+      // row-major outputs go through the staging area: SC columns of RPI rows at a time, the components of a
+      // complex element (rows 2 i, 2 i + 1) next to each other, so that every pass stores whole sectors
+      constexpr int RPI = PLAIN ? 2 : 32 / SC, PASSES = 32 / RPI;
+      static_assert(PLAIN || RPI % 2 == 0, "k_ozgemm: staging");
       long long *stg = reinterpret_cast<long long *>(stage_out) + warp * 32 * (SC + 1);
-      auto store_rows = [&](int cb) {   // columns cb .. + SC of the warp, staged
-        const int rbase = m0 + 32 * quad;
-        double old[SC];
-        if (beta != 0.0) {
+      const int lr = mode == 1 ? lane / (2 * SC) * 2 + (lane & 1) : lane / SC;   // the lane's row and column of a pass
+      const int lc = mode == 1 ? lane % (2 * SC) >> 1 : lane % SC;
+      const int rlive = lane < RPI * SC ? eM - (m0 + 32 * quad) - lr : 0;        // passes with RPI i < rlive
+      auto out0 = [&](int cb) { return out_row(m0 + 32 * quad + lr) + (cbase + cb + lc) * cstep; };
+      const long long step = RPI * ldc;
+      auto store_rows = [&](int cb, auto &&old) {   // columns cb .. + SC of the warp, staged; old(i, q): *q before
+        __syncwarp();
+        double *q = out0(cb);
+        const long long *sp = stg + lr * (SC + 1) + lc;
+        if (cb + lc < nc) {
 #pragma unroll
-          for (int i = 0; i < SC; ++i) {
-            const int x = lane + 32 * i, rr = x / SC, cc = cb + x % SC;
-            if (cc < nc && rbase + rr < eM) old[i] = *at(rbase + rr, cbase + cc);
+          for (int i = 0; i < PASSES; ++i, q += step) {
+            if (RPI * i >= rlive) break;
+            double v = __longlong_as_double(sp[i * RPI * (SC + 1)]);
+            if (beta != 0.0) {   // (modes 0 and 1)
+              asm volatile("");
+              v += beta * old(i, q);
+            }
+            *q = v;
           }
         }
         __syncwarp();
-#pragma unroll
-        for (int i = 0; i < SC; ++i) {
-          const int x = lane + 32 * i, rr = x / SC, cc = cb + x % SC;
-          if (cc >= nc || rbase + rr >= eM) continue;
-          const double v = __longlong_as_double(stg[rr * (SC + 1) + x % SC]);
-          if (mode == 3)   // the 8 bytes hold the pair (hi, lo)
-            C[(long long)(rbase + rr) * ldc + cbase + cc] = v;
-          else
-            *at(rbase + rr, cbase + cc) = beta == 0.0 ? v : v + beta * old[i];
-        }
-        __syncwarp();
       };
-      const bool trans = mode == 2 || mode == 4;
+      // updated outputs of a single group are read before its sums are waited for
+      double old0[DIRECT ? PASSES : 1];
+      if constexpr (DIRECT) {
+        if (beta != 0.0 && !trans) {
+          const double *q = out0(0);
+#pragma unroll
+          for (int i = 0; i < PASSES; ++i, q += step) old0[i] = RPI * i < rlive && lc < nc ? *q : 0.0;
+        }
+      }
+      auto read0 = [&](int i, const double *) { return old0[DIRECT ? i : 0]; };
+      auto read_now = [&](int, const double *q) { return *q; };
       if constexpr (!PLAIN && !DIRECT) {
 #pragma unroll
         for (int j = 0; j < HALF; ++j) acc[j] = 0;
@@ -722,7 +745,7 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
 #pragma unroll
               for (int d = 0; d < S; ++d) tmem_ld(tbase + (uint32_t)d * BN + c, r[d]);
 #pragma unroll
-              for (int x = 0; x < 4; ++x) e_b[x] = c + x < nc ? eb[c + x] : 0;
+              for (int x = 0; x < 4; ++x) e_b[x] = eb(c + x);
 #pragma unroll
               for (int d = 0; d < S; ++d) tmem_ld_wait(r[d]);
 #pragma unroll
@@ -770,9 +793,13 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
                 if (!trans) {
                   stg[lane * (SC + 1) + c + x] = o;
                 } else if (row_ok && c + x < nc) {   // consecutive along the lanes
-                  double *q = at(row, cbase + c + x);
-                  const double v = __longlong_as_double(o);
-                  *q = beta == 0.0 ? v : v + beta * *q;
+                  double *q = out_row(row) + (cbase + c + x) * cstep;
+                  double v = __longlong_as_double(o);
+                  if (beta != 0.0) {
+                    asm volatile("");
+                    v += beta * *q;
+                  }
+                  *q = v;
                 }
               }
             }
@@ -780,7 +807,7 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
             __syncwarp();
             if (lane == 0) mbar_arrive(&tempty[rt.slot]);   // the accumulators may be overwritten now
             rt.next();
-            if (!trans && nc > 0) store_rows(0);
+            if (!trans && nc > 0) store_rows(0, read0);
             break;
           }
           if constexpr (!DIRECT) {
@@ -828,13 +855,13 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
         if (nsteps == 0 && nc > 0) {   // nothing to sum: zeros
           if (trans) {
             for (int j = 0; j < nc && row_ok; ++j) {
-              double *q = at(row, cbase + j);
+              double *q = out_row(row) + (cbase + j) * cstep;
               *q = beta == 0.0 ? 0.0 : beta * *q;
             }
           } else {
 #pragma unroll
             for (int j = 0; j < SC; ++j) stg[lane * (SC + 1) + j] = 0;
-            store_rows(0);
+            store_rows(0, read0);
           }
         }
       } else if constexpr (PLAIN) {
@@ -857,28 +884,29 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
                   make_float2(hi, __double2float_rn(v - (double)hi));
               continue;
             }
-            double *p = at(row, col);
+            double *p = out_row(row) + col * cstep;
             *p = beta == 0.0 ? v : v + beta * *p;
           }
         }
       } else {
         if (nc <= 0) continue;
+        load_eb();
         // the values in place of the sums
 #pragma unroll
-        for (int j = 0; j < HALF; ++j) acc[j] = value(WIDE ? acch[WIDE ? j : 0] : 0, acc[j], j < nc ? eb[j] : 0);
+        for (int j = 0; j < HALF; ++j) acc[j] = value(WIDE ? acch[WIDE ? j : 0] : 0, acc[j], eb(j));
         if (trans) {   // consecutive along the lanes (tile rows)
           if (row_ok) {
             double old[HALF];
             if (beta != 0.0) {
 #pragma unroll
               for (int j = 0; j < HALF; ++j)
-                if (j < nc) old[j] = *at(row, cbase + j);
+                if (j < nc) old[j] = out_row(row)[(cbase + j) * cstep];
             }
 #pragma unroll
             for (int j = 0; j < HALF; ++j)
               if (j < nc) {
                 const double v = __longlong_as_double(acc[j]);
-                *at(row, cbase + j) = beta == 0.0 ? v : v + beta * old[j];
+                out_row(row)[(cbase + j) * cstep] = beta == 0.0 ? v : v + beta * old[j];
               }
           }
           continue;
@@ -888,7 +916,7 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
           if (cb >= nc) break;   // the same for the whole warp
 #pragma unroll
           for (int j = 0; j < SC; ++j) stg[lane * (SC + 1) + j] = acc[cb + j];
-          store_rows(cb);
+          store_rows(cb, read_now);
         }
       }
     }
