@@ -22,6 +22,7 @@
 // L2 -> shared-memory traffic of the N planes, not by the MMAs.
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 
 #include "internal.h"
 #include "oasm.h"
@@ -423,10 +424,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int r = quad * 32 + lane, kap = s_kap[r], f2 = s_f2[r], urow = s_urow[r];
     const bool any = __any_sync(0xffffffffu, kap >= 0);
     const int per = (nU + 1) / 2, c0 = half * per, c1 = min(nU, c0 + per);
+    // exponents: of the lane's N row, and of row i = lane of Lm and X; those of the warp's next nu are fetched while
+    // this one is folded
+    const int i16 = lane & (kMaxAo - 1), e1_lane = s_e1[i16];
+    const int *np_ = nexp + nu0 * a.m_all + urow, *xp_ = xexp + (nu0 * a.natoms + U) * kMaxAo + i16;
+    auto next_f1 = [&](int i) { return kap >= 0 && i < nauxV ? np_[(size_t)i * a.m_all] : 0; };
+    auto next_e2 = [&](int i) { return i < nauxV ? xp_[(size_t)i * a.natoms * kMaxAo] : 0; };
+    int f1n = next_f1(grp), e2n = next_e2(grp);
     for (int it = grp; it < nauxV; it += 2) {
-      const int sl = it % NSL;
-      const int f1 = kap >= 0 ? nexp[(nu0 + it) * a.m_all + urow] : 0;
-      const int *xe = xexp + ((nu0 + it) * a.natoms + U) * kMaxAo;
+      const int sl = it % NSL, f1 = f1n;
+      const int e_lane = (int)((unsigned)e1_lane << 16) | (e2n & 0xFFFF);   // both, one shuffle per i (|e| <= 1100)
+      f1n = next_f1(it + 2);
+      e2n = next_e2(it + 2);
       bool ok = !abort_flag && mbar_wait(&tfull[sl], (uint32_t)((it / NSL) & 1), WAIT_NS, &abort_flag);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) {
@@ -441,29 +450,48 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll 1
         for (int c = c0; c < c1; c += 4) {
           uint32_t r1[S][4], r2[S][4];
-          int e2[4];
-#pragma unroll
-          for (int x = 0; x < 4; ++x) e2[x] = xe[min(c + x, kMaxAo - 1)];
+          int e[4];
 #pragma unroll
           for (int d = 0; d < S; ++d) {
             tmem_ld(tb0 + d * kMaxAo + c, r1[d]);
             tmem_ld(tb0 + (S + d) * kMaxAo + c, r2[d]);
           }
 #pragma unroll
+          for (int x = 0; x < 4; ++x) e[x] = __shfl_sync(0xffffffffu, e_lane, c + x & (kMaxAo - 1));
+#pragma unroll
           for (int d = 0; d < S; ++d) {
             tmem_ld_wait(r1[d]);
             tmem_ld_wait(r2[d]);
           }
+          // N elements from x0 on, side by side (a branch per element would fold them one after the other); those
+          // beyond c1 are not stored
+          auto fold = [&](auto x0_, auto n_) {
+            constexpr int x0 = decltype(x0_)::value, N = decltype(n_)::value;
+            double o[N];
 #pragma unroll
-          for (int x = 0; x < 4; ++x) {
-            if (c + x >= c1) break;   // the same for the whole warp
-            const int e1 = s_e1[c + x];
-            double o = combine<S>(r1, r2, x, e1 + f1, e2[x] + f2);
-            if (S == oz::S_WIDE && max(max(e1, f1), max(e2[x], f2)) > 1024) o = __longlong_as_double(0x7FF8000000000000ll);
-            if (kap >= 0) {
-              orow[(size_t)(c + x) * mU] = o;
-              emax = max(emax, __double2hiint(o) & 0x7FFFFFFF);
+            for (int x = x0; x < x0 + N; ++x) {
+              const int e1 = e[x] >> 16, e2 = (int)(short)e[x];
+              o[x - x0] = combine<S>(r1, r2, x, e1 + f1, e2 + f2);
+              if (S == oz::S_WIDE && max(max(e1, f1), max(e2, f2)) > 1024)
+                o[x - x0] = __longlong_as_double(0x7FF8000000000000ll);
             }
+#pragma unroll
+            for (int x = x0; x < x0 + N; ++x)
+              if (kap >= 0 && c + x < c1) {
+                orow[(size_t)(c + x) * mU] = o[x - x0];
+                emax = max(emax, __double2hiint(o[x - x0]) & 0x7FFFFFFF);
+              }
+          };
+          using std::integral_constant;
+          if constexpr (S == oz::S_WIDE) {   // (one at a time: the two-word sums of more do not fit the registers)
+            fold(integral_constant<int, 0>(), integral_constant<int, 1>());
+            if (c + 1 < c1) fold(integral_constant<int, 1>(), integral_constant<int, 1>());
+            if (c + 2 < c1) fold(integral_constant<int, 2>(), integral_constant<int, 1>());
+            if (c + 3 < c1) fold(integral_constant<int, 3>(), integral_constant<int, 1>());
+          } else if (c + 2 < c1) {
+            fold(integral_constant<int, 0>(), integral_constant<int, 4>());
+          } else {
+            fold(integral_constant<int, 0>(), integral_constant<int, 2>());
           }
         }
       }

@@ -623,6 +623,8 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
       const long long ldc = en.ldc;
       double *const C = en.C;
       const double alpha = en.alpha, beta = en.beta;
+      // beta != 0, tested on its bits (a comparison of doubles per store held the FP64 pipe for a third of the N step)
+      const bool upd = (__double_as_longlong(beta) << 1) != 0;
       const bool pow2 = en.alpha_shift != kNoShift;   // alpha = +-2^alpha_shift: folded into the exponent
       const int row = m0 + 32 * quad + lane;          // thread = tile row (the TMEM lane layout)
       const bool row_ok = row < eM;
@@ -642,11 +644,7 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
       const int ash = (pow2 ? en.alpha_shift : 0) - 14 - 8 * (S - 1);
       const int ea = PLAIN || !row_ok ? ash : mp.ea[tl.arow + 32 * quad + lane] + ash;
       // the exponents of the warp's columns, one per lane
-      int eb_lane = 0;
-      auto load_eb = [&] {
-        if (lane < nc) eb_lane = (maps[tl.pair].eb + tl.brow + half * HALF)[lane];
-      };
-      if constexpr (DIRECT) load_eb();
+      const int eb_lane = !PLAIN && lane < nc ? (mp.eb + tl.brow + half * HALF)[lane] : 0;
       auto eb = [&](int j) { return __shfl_sync(0xffffffffu, eb_lane, j); };
       const bool aneg = pow2 && alpha < 0.0;
       // a row or column with an infinity or a NaN has the exponent 1025 (finite ones at most 1024)
@@ -697,7 +695,7 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
           for (int i = 0; i < PASSES; ++i, q += step) {
             if (RPI * i >= rlive) break;
             double v = __longlong_as_double(sp[i * RPI * (SC + 1)]);
-            if (beta != 0.0) {   // (modes 0 and 1)
+            if (upd) {   // (modes 0 and 1)
               asm volatile("");
               v += beta * old(i, q);
             }
@@ -709,7 +707,7 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
       // updated outputs of a single group are read before its sums are waited for
       double old0[DIRECT ? PASSES : 1];
       if constexpr (DIRECT) {
-        if (beta != 0.0 && !trans) {
+        if (upd && !trans) {
           const double *q = out0(0);
 #pragma unroll
           for (int i = 0; i < PASSES; ++i, q += step) old0[i] = RPI * i < rlive && lc < nc ? *q : 0.0;
@@ -795,7 +793,7 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
                 } else if (row_ok && c + x < nc) {   // consecutive along the lanes
                   double *q = out_row(row) + (cbase + c + x) * cstep;
                   double v = __longlong_as_double(o);
-                  if (beta != 0.0) {
+                  if (upd) {
                     asm volatile("");
                     v += beta * *q;
                   }
@@ -856,7 +854,7 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
           if (trans) {
             for (int j = 0; j < nc && row_ok; ++j) {
               double *q = out_row(row) + (cbase + j) * cstep;
-              *q = beta == 0.0 ? 0.0 : beta * *q;
+              *q = !upd ? 0.0 : beta * *q;
             }
           } else {
 #pragma unroll
@@ -885,19 +883,18 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
               continue;
             }
             double *p = out_row(row) + col * cstep;
-            *p = beta == 0.0 ? v : v + beta * *p;
+            *p = !upd ? v : v + beta * *p;
           }
         }
       } else {
         if (nc <= 0) continue;
-        load_eb();
         // the values in place of the sums
 #pragma unroll
         for (int j = 0; j < HALF; ++j) acc[j] = value(WIDE ? acch[WIDE ? j : 0] : 0, acc[j], eb(j));
         if (trans) {   // consecutive along the lanes (tile rows)
           if (row_ok) {
             double old[HALF];
-            if (beta != 0.0) {
+            if (upd) {
 #pragma unroll
               for (int j = 0; j < HALF; ++j)
                 if (j < nc) old[j] = out_row(row)[(cbase + j) * cstep];
@@ -906,7 +903,7 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
             for (int j = 0; j < HALF; ++j)
               if (j < nc) {
                 const double v = __longlong_as_double(acc[j]);
-                out_row(row)[(cbase + j) * cstep] = beta == 0.0 ? v : v + beta * old[j];
+                out_row(row)[(cbase + j) * cstep] = !upd ? v : v + beta * old[j];
               }
           }
           continue;
