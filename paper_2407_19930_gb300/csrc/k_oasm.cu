@@ -15,9 +15,9 @@
 //     column, X every tile of U).  HBM-bound.
 //   k_oasm<S>: one CTA per (point, V, U, tile of 128 rows kap).  tcgen05.mma with the kap rows as M = 128, the
 //     i of U as N (16 per plane, the planes stacked: plane s of A meets all S + 1 - s planes of B in one MMA of
-//     N = 16 (S + 1 - s)), K = 32.  RG and Lm stay in shared memory; a TMA warp streams N and X planes per nu (one
-//     box of 8 rows x S planes per row group, so a tile gathers U's columns from the union), one lane issues the
-//     MMAs, 16 warps fold and store.
+//     N = 16 (S + 1 - s)), K = 32.  RG and Lm stay in shared memory; a TMA warp streams N and X planes of two nu at a
+//     time (one box of 2 nu x S planes x 8 rows per row group, so a tile gathers U's columns from the union), one lane
+//     issues the MMAs, 16 warps fold and store.
 // The kernel is bound by the folding of the diagonal sums (integer and FP32 instructions) and by the
 // L2 -> shared-memory traffic of the N planes, not by the MMAs.
 #include <algorithm>
@@ -113,11 +113,11 @@ struct Elem<oz::S_WIDE> {
   }
 };
 
-// Digit planes of N: rows (p, nu, union column), columns t = (g, j).  Two lanes per row (16 t each), 16 consecutive
+// Digit planes of N: laid out [(p, nu)][plane][union column][t], t = (g, j); row exponents [(p, nu)][union column].  Two lanes per row (16 t each), 16 consecutive
 // columns per warp; block = 128 columns of one (p, nu).
 template <int S>
 __global__ void __launch_bounds__(256) k_split_n(OArgs a, const int *__restrict__ aux_atom, __nv_bfloat16 *dig,
-                                                 int *expo, long long plane) {
+                                                 int *expo) {
   using E_ = Elem<S>;
   const int p = blockIdx.x / a.naux, nug = blockIdx.x % a.naux, V = aux_atom[nug], nu = nug - a.aux_off[V];
   const int lane = threadIdx.x & 31, h = lane >> 4;
@@ -139,21 +139,21 @@ __global__ void __launch_bounds__(256) k_split_n(OArgs a, const int *__restrict_
   const int E = E_::expo(m);
   const long long row = ((long long)p * a.naux + nug) * a.m_all + col;
   if (h == 0) expo[row] = E;
+  __nv_bfloat16 *out = dig + (((size_t)p * a.naux + nug) * S * a.m_all + col) * 32 + 16 * h;
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     uint4 w[S];
     E_::digits8(v + 8 * c, E, w);
 #pragma unroll
-    for (int s = 0; s < S; ++s) *reinterpret_cast<uint4 *>(dig + s * plane + row * 32 + 16 * h + 8 * c) = w[s];
+    for (int s = 0; s < S; ++s) *reinterpret_cast<uint4 *>(out + (size_t)s * a.m_all * 32 + 8 * c) = w[s];
   }
 }
 
-// Digit planes of X: rows (p, nu, 16 U + i), columns t; two lanes per row.  Rows i >= n_U are left as they are (the MMA
+// Digit planes of X: [(p, nu)][plane][16 U + i][t]; two lanes per row.  Rows i >= n_U are left as they are (the MMA
 // columns they give are not read).
 template <int S>
 __global__ void __launch_bounds__(256) k_split_x(OArgs a, const int *__restrict__ aux_atom,
-                                                 const int *__restrict__ ao_row, __nv_bfloat16 *dig, int *expo,
-                                                 long long plane) {
+                                                 const int *__restrict__ ao_row, __nv_bfloat16 *dig, int *expo) {
   using E_ = Elem<S>;
   const int p = blockIdx.x / a.naux, nug = blockIdx.x % a.naux, V = aux_atom[nug], nu = nug - a.aux_off[V];
   const int lane = threadIdx.x & 31, h = lane >> 4;
@@ -176,12 +176,13 @@ __global__ void __launch_bounds__(256) k_split_x(OArgs a, const int *__restrict_
   const int E = E_::expo(m);
   const long long row = ((long long)p * a.naux + nug) * (a.natoms * kMaxAo) + ao_row[ao];
   if (h == 0) expo[row] = E;
+  __nv_bfloat16 *out = dig + (((size_t)p * a.naux + nug) * S * a.natoms * kMaxAo + ao_row[ao]) * 32 + 16 * h;
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     uint4 w[S];
     E_::digits8(v + 8 * c, E, w);
 #pragma unroll
-    for (int s = 0; s < S; ++s) *reinterpret_cast<uint4 *>(dig + s * plane + row * 32 + 16 * h + 8 * c) = w[s];
+    for (int s = 0; s < S; ++s) *reinterpret_cast<uint4 *>(out + (size_t)s * a.natoms * kMaxAo * 32 + 8 * c) = w[s];
   }
 }
 
@@ -189,9 +190,13 @@ __global__ void __launch_bounds__(256) k_split_x(OArgs a, const int *__restrict_
 constexpr int kEpi = 16, kThreads = 32 * (kEpi + 2);
 __host__ __device__ constexpr int op_bytes(int S) { return kTileGroups * S * 512; }   // 128 rows: groups of 8 rows x S planes x 64 bytes
 __host__ __device__ constexpr int x_bytes(int S) { return S * kMaxAo * 64; }          // S planes of 16 rows x 64 bytes
-__host__ __device__ constexpr int stage_size(int S) { return op_bytes(S) + x_bytes(S); }
-__host__ __device__ constexpr int ring(int S) { return S == oz::S_WIDE ? 2 : S == 5 ? 3 : 5; }
-__host__ __device__ constexpr int smem_size(int S) { return (1 + ring(S)) * stage_size(S) + 1024; }
+__host__ __device__ constexpr int static_size(int S) { return op_bytes(S) + x_bytes(S); }   // RG and Lm
+// nu per stage: half the copies to issue, 64-byte rows fetched two nu at a time, where two stages fit (k_oasm of the graphene
+// slab 1.08 -> 1.04 ms a point with 5 planes, 0.97 -> 0.92 with 3).
+__host__ __device__ constexpr int nus(int S) { return S == oz::S_WIDE ? 1 : 2; }
+__host__ __device__ constexpr int stage_size(int S) { return nus(S) * static_size(S); }
+__host__ __device__ constexpr int ring(int S) { return S == 3 ? 3 : 2; }
+__host__ __device__ constexpr int smem_size(int S) { return static_size(S) + ring(S) * stage_size(S) + 512; }
 __host__ __device__ constexpr int slot_cols(int S) { return 2 * S * kMaxAo; }         // TMEM columns of one nu: two terms, S diagonals, 16 i
 __host__ __device__ constexpr int slots(int S) { return 512 / slot_cols(S); }
 
@@ -236,12 +241,13 @@ __global__ void __launch_bounds__(kThreads, 1)
            const int *__restrict__ nexp, const int *__restrict__ xexp, int *rexp, int *err) {
   using E_ = Elem<S>;
   constexpr int NST = ring(S), NSL = slots(S), SL = slot_cols(S);
-  constexpr uint32_t OPB = op_bytes(S), XB_ = x_bytes(S), STAGE = stage_size(S);
+  constexpr int NU = nus(S);
+  constexpr uint32_t OPB = op_bytes(S), XB_ = x_bytes(S), FIXED = static_size(S), STAGE = stage_size(S);
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t full[NST], empty[NST], tfull[NSL], tempty[NSL], mdone;
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
-  __shared__ int s_e1[kMaxAo], s_f2[128], s_kap[128], s_urow[128], s_box[kTileGroups];
+  __shared__ int s_e1[kMaxAo], s_box[kTileGroups];
   __shared__ int s_groups;
   // U and its tiles run fastest: the CTAs in flight share the N planes of a few V in the L2
   const int uv = blockIdx.x / tb.max_tiles;
@@ -272,8 +278,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       return;
     }
   }
-  uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 511) & ~(uintptr_t)511);   // 64-byte swizzle: 512-byte atoms
   uint8_t *sRG = smem, *sLm = smem + OPB;   // static operands, then the ring
+  // exponent, packed and union column of the tile's rows, in the first stage until the epilogue has read them
+  int *s_f2 = reinterpret_cast<int *>(smem + FIXED), *s_kap = s_f2 + 128, *s_urow = s_kap + 128;
   if (tid == 0) {
     for (int s = 0; s < NST; ++s) {
       mbar_init(&full[s], 1);
@@ -357,22 +365,32 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
+  int kap = -1, f2 = 0, urow = 0;
+  if (warp < kEpi) {
+    const int r = (warp & 3) * 32 + lane;
+    kap = s_kap[r];
+    f2 = s_f2[r];
+    urow = s_urow[r];
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the copies come after these reads
+  __syncthreads();
   const long long nu0 = (long long)p * a.naux + a.aux_off[V];
   if (warp == kEpi) {
     if (elect_one()) {   // TMA producer: N rows of the tile's groups and the 16 X rows of U, per nu
       const int ng = s_groups;
+      const int nblk = (nauxV + NU - 1) / NU;   // (the nu beyond V's last in a block are loaded, not used)
       int it = 0;
-      for (; it < nauxV; ++it) {
+      for (; it < nblk; ++it) {
         const int st = it % NST;
         if (abort_flag || !mbar_wait(&empty[st], (uint32_t)(((it / NST) & 1) ^ 1), WAIT_NS, &abort_flag)) {
           abort_flag = 1;
           break;
         }
-        uint8_t *sn = smem + STAGE + st * STAGE, *sx = sn + OPB;
-        mbar_expect_tx(&full[st], (uint32_t)ng * S * 512 + XB_);
-        const int row = (int)((nu0 + it) * a.m_all);
-        for (int g = 0; g < ng; ++g) tma_load_3d(sn + g * (S * 512), &nmap, &full[st], 0, row + s_box[g], 0);
-        tma_load_3d(sx, &xmap, &full[st], 0, (int)((nu0 + it) * a.natoms + U) * kMaxAo, 0);
+        uint8_t *sn = smem + FIXED + st * STAGE, *sx = sn + NU * OPB;
+        mbar_expect_tx(&full[st], NU * ((uint32_t)ng * S * 512 + XB_));
+        const int nu = (int)nu0 + it * NU;
+        for (int g = 0; g < ng; ++g) tma_load_4d(sn + g * (NU * S * 512), &nmap, &full[st], 0, s_box[g], 0, nu);
+        tma_load_4d(sx, &xmap, &full[st], 0, U * kMaxAo, 0, nu);
       }
       // after a failure: wait for the copies still in flight (the last NST issued stages)
       if (abort_flag)
@@ -383,18 +401,19 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int ks = (two + 15) / 16;
       const uint32_t rg = smem_u32(sRG), lm = smem_u32(sLm);
       for (int it = 0; it < nauxV; ++it) {
-        const int st = it % NST, sl = it % NSL;
+        const int blk = it / NU, st = blk % NST, sl = it % NSL;
         if (it >= NSL && (abort_flag || !mbar_wait(&tempty[sl], (uint32_t)((it / NSL - 1) & 1), WAIT_NS, &abort_flag))) {
           abort_flag = 1;
           break;
         }
-        if (abort_flag || !mbar_wait(&full[st], (uint32_t)((it / NST) & 1), WAIT_NS, &abort_flag)) {
+        if (abort_flag || !mbar_wait(&full[st], (uint32_t)((blk / NST) & 1), WAIT_NS, &abort_flag)) {
           abort_flag = 1;
           break;
         }
         tc_fence_after();
-        const uint32_t sn = smem_u32(smem + STAGE + st * STAGE), sx = sn + OPB, d = tmem + sl * SL;
-        const uint64_t dn = smem_desc64(sn, S * 512), dr = smem_desc64(rg, S * 512), dl = smem_desc64(lm), dx = smem_desc64(sx);
+        const uint32_t s0 = smem_u32(smem + FIXED + st * STAGE), sn = s0 + it % NU * (S * 512), sx = s0 + NU * OPB + it % NU * XB_,
+                       d = tmem + sl * SL;
+        const uint64_t dn = smem_desc64(sn, NU * S * 512), dr = smem_desc64(rg, S * 512), dl = smem_desc64(lm), dx = smem_desc64(sx);
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           if (j >= ks) break;
@@ -410,7 +429,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
           }
         }
-        umma_commit(&empty[st]);
+        if (it % NU == NU - 1) umma_commit(&empty[st]);
         umma_commit(&tfull[sl]);
       }
       if (abort_flag) {   // after a failure: wait for the MMAs already issued
@@ -421,7 +440,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else {
     // epilogue: warps 0-7 the even nu, 8-15 the odd ones; thread = row kap, half of the i each
     const int grp = warp >> 3, quad = warp & 3, half = (warp >> 2) & 1;
-    const int r = quad * 32 + lane, kap = s_kap[r], f2 = s_f2[r], urow = s_urow[r];
     const bool any = __any_sync(0xffffffffu, kap >= 0);
     const int per = (nU + 1) / 2, c0 = half * per, c1 = min(nU, c0 + per);
     // exponents: of the lane's N row, and of row i = lane of Lm and X; those of the warp's next nu are fetched while
@@ -515,12 +533,13 @@ void launch(const OArgs &a, const Tables &t, int np, oz::Sliced &nd, oz::Sliced 
   static_assert(smem_size(S) <= 227 * 1024, "k_oasm: shared memory");
   const unsigned rows = (unsigned)(np * a.naux);
   k_split_n<S><<<dim3(rows, (unsigned)((a.m_all + 127) / 128)), 256, 0, s>>>(
-      a, t.aux_atom, (__nv_bfloat16 *)nd.digits, nd.expo, (long long)nd.rows * nd.kpad);
+      a, t.aux_atom, (__nv_bfloat16 *)nd.digits, nd.expo);
   k_split_x<S><<<dim3(rows, (unsigned)((a.nao + 127) / 128)), 256, 0, s>>>(
-      a, t.aux_atom, t.ao_row, (__nv_bfloat16 *)xd.digits, xd.expo, (long long)xd.rows * xd.kpad);
+      a, t.aux_atom, t.ao_row, (__nv_bfloat16 *)xd.digits, xd.expo);
   LR_CUDA(cudaFuncSetAttribute(k_oasm<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_size(S)));
   k_oasm<S><<<(unsigned)t.max_tiles * (unsigned)(np * a.natoms * a.natoms), kThreads, smem_size(S), s>>>(
-      a, t, oz::make_map(nd, 8, S, 64), oz::make_map(xd, kMaxAo, S, 64), nd.expo, xd.expo, expo, err);
+      a, t, oz::make_map_nested(nd.digits, a.m_all, S, (int)rows, 8, nus(S)),
+      oz::make_map_nested(xd.digits, a.natoms * kMaxAo, S, (int)rows, kMaxAo, nus(S)), nd.expo, xd.expo, expo, err);
   launch_counter() += 3;
   LR_CUDA(cudaGetLastError());
 }

@@ -927,20 +927,34 @@ __global__ void __launch_bounds__(32 * (epi_warps(S) + 2), 1)
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 
-}  // namespace
-
-CUtensorMap make_map(const Sliced &o, int box_rows, int box_planes, int row_bytes) {
+// Tensor map of an operand's planes with boxes of 128 bytes (the swizzle width) x box_rows rows x box_planes planes.
+CUtensorMap make_map(const Sliced &o, int box_rows, int box_planes) {
   CUtensorMap m;
   const cuuint64_t eb = (cuuint64_t)elem_bytes(o.S);
   const cuuint64_t dims[3] = {(cuuint64_t)o.kpad, (cuuint64_t)o.rows, (cuuint64_t)planes(o.S)};
   const cuuint64_t strides[2] = {(cuuint64_t)o.kpad * eb, (cuuint64_t)o.kpad * eb * (cuuint64_t)o.rows};
-  const cuuint32_t box[3] = {(cuuint32_t)(row_bytes / eb), (cuuint32_t)box_rows, (cuuint32_t)box_planes};
+  const cuuint32_t box[3] = {(cuuint32_t)(128 / eb), (cuuint32_t)box_rows, (cuuint32_t)box_planes};
   const cuuint32_t estr[3] = {1, 1, 1};
   const CUtensorMapDataType dt = eb == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
   const CUresult r = g_encode(&m, dt, 3, o.digits, dims, strides, box, estr,
                               CU_TENSOR_MAP_INTERLEAVE_NONE,
-                              row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                              CU_TENSOR_MAP_SWIZZLE_128B,
                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) throw Error{LIBRPA_E_CUDA, "cuTensorMapEncodeTiled failed: " + std::to_string((int)r)};
+  return m;
+}
+
+}  // namespace
+
+CUtensorMap make_map_nested(const void *digits, int rows, int planes, int outer, int box_rows, int box_outer) {
+  CUtensorMap m;
+  const cuuint64_t dims[4] = {32, (cuuint64_t)rows, (cuuint64_t)planes, (cuuint64_t)outer};
+  const cuuint64_t strides[3] = {64, 64ull * rows, 64ull * rows * planes};
+  const cuuint32_t box[4] = {32, (cuuint32_t)box_rows, (cuuint32_t)planes, (cuuint32_t)box_outer};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  const CUresult r = g_encode(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(digits), dims, strides, box, estr,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) throw Error{LIBRPA_E_CUDA, "cuTensorMapEncodeTiled failed: " + std::to_string((int)r)};
   return m;
 }
@@ -1184,8 +1198,8 @@ long long gemm_multi(const std::vector<std::pair<const Sliced *, const Sliced *>
   }
   std::vector<MapPair> mp(ops.size());
   for (size_t i = 0; i < ops.size(); ++i) {
-    mp[i].a = make_map(*ops[i].first, BM, 1, 128);
-    mp[i].b = make_map(*ops[i].second, BN, planes(S), 128);
+    mp[i].a = make_map(*ops[i].first, BM, 1);
+    mp[i].b = make_map(*ops[i].second, BN, planes(S));
     mp[i].ea = ops[i].first->expo;
     mp[i].eb = ops[i].second->expo;
   }

@@ -142,9 +142,9 @@ long long gemm_multi(const std::vector<std::pair<const Sliced *, const Sliced *>
 long long gemm(const Sliced &a, const Sliced &b, int M, int N, int batch, const Out &out, int km, int kn,
                int lower_div, int *err, cudaStream_t s, Handle &h);
 
-// Tensor map of an operand's planes with boxes of row_bytes (64 or 128, the swizzle width) x box_rows rows x
-// box_planes planes; after init().
-CUtensorMap make_map(const Sliced &o, int box_rows, int box_planes, int row_bytes);
+// Tensor map of digit planes laid out [outer][plane][rows][32] (BF16, 64-byte rows) with boxes of box_rows rows of all
+// planes of box_outer outer entries; after init().
+CUtensorMap make_map_nested(const void *digits, int rows, int planes, int outer, int box_rows, int box_outer);
 
 // One-time host setup (driver entry point for tensor-map encoding).  Throws on failure.
 void init();
