@@ -2,8 +2,8 @@
 //
 // Operands are split once into BF16 digit planes (k_row_expo + k_digits, or k_plain for plain
 // BF16); the GEMM kernel streams them with TMA (cp.async.bulk.tensor) into a shared-memory ring
-// and multiplies every digit pair with tcgen05.mma (kind::f16, BF16 x BF16 -> FP32, M = 128,
-// N = 64, K = 16) into the TMEM accumulator of its diagonal; flush groups (the largest K range
+// and multiplies every digit pair with tcgen05.mma (kind::f16, BF16 x BF16 -> FP32, M = 128, K = 16,
+// planes stacked along N) into the TMEM accumulator of its diagonal; flush groups (the largest K range
 // whose FP32 sums stay exact) are moved into exact int64 register sums, scaled by
 // 2^(E_A + E_B - 14 - 8(S-1)) into FP64 at the end.  Every wait on an mbarrier is bounded by the
 // global timer; on a timeout the kernel records the failure in *err, waits (bounded) for its own
@@ -418,6 +418,9 @@ struct alignas(128) MapPair {
 //     registers.  The TMEM columns go back to the issuer before the values are converted and stored, so
 //     conversion and stores overlap the next tile's MMAs.  The conversion (~30 integer instructions) is
 //     bound by its latency: four warps per scheduler, 8 to 16 independent sums each.
+// The epilogue of short-K tiles is bound by that chain and, in the trailing updates, by the FP64 pipe (two additions
+// a cycle and SM), so it has no other FP64 instruction, reads the old outputs before it waits for the sums and stores
+// whole sectors: 96 complex matrices of order 1946, K = 128: 7.0 -> 5.1 ms; N step of the slab 0.50 -> 0.44 ms.
 // DIRECT: every tile has a single flush group (K up to 192 with 5 planes: the N and X steps, the trailing updates);
 // outputs are then formed four columns at a time straight from TMEM, in a rolled loop, with no sums kept (a thread's
 // columns unrolled are more instructions than the instruction cache holds).
