@@ -107,13 +107,19 @@ typedef struct {
   int chi0_slices;               /* 0 = from precision; 1..5 = digit planes of the chi0 GEMMs */
   int ec_slices;                 /* 0 = from precision; 1..5 = digit planes of the ln det GEMMs */
   int test_stall_gemms;          /* testing only (0 = off): in the handle's first test_stall_gemms
-                                    tensor-core GEMM launches the MMA issuer of every CTA waits
-                                    (100 us) on a barrier that nothing arrives at, so the bounded-wait
-                                    failure path runs: the call returns LIBRPA_E_TIMEOUT, later
-                                    calls of the handle run normally */
+                                    tensor-core GEMM launches with up to 5 digit planes the MMA issuer of
+                                    every CTA waits (100 us) on a barrier that nothing arrives at, so the
+                                    bounded-wait failure path runs: the call returns LIBRPA_E_TIMEOUT,
+                                    later calls of the handle run normally.  Added to it,
+                                    LIBRPA_TEST_STALL_WIDE x n does the same to the first n launches with
+                                    8 digit planes, LIBRPA_TEST_STALL_OASM x n to the first n
+                                    tensor-core launches of the O assembly */
   int grid_kind;                 /* LIBRPA_GRID_MINIMAX (default) or LIBRPA_GRID_GAUSS_LEGENDRE: the grid
                                     librpa_gpu_chi0 builds when none was set */
 } librpa_gpu_opts;
+
+#define LIBRPA_TEST_STALL_WIDE (1 << 20) /* test_stall_gemms: n of these, n <= 63 */
+#define LIBRPA_TEST_STALL_OASM (1 << 26) /* the same, n <= 31 */
 
 /* Per-stage device times (ms, CUDA events on the handle's stream) and work counts of
  * the most recent librpa_gpu_chi0 / librpa_gpu_ec call. */

@@ -297,7 +297,9 @@ int librpa_gpu_create(librpa_gpu_t *hp, const librpa_gpu_opts *o) {
   librpa_gpu *h = new (std::nothrow) librpa_gpu();
   if (!h) return LIBRPA_E_NOMEM;
   h->opts = *o;
-  h->stalls_left = o->test_stall_gemms;
+  h->stalls_left = o->test_stall_gemms % LIBRPA_TEST_STALL_WIDE;
+  h->stalls_wide = o->test_stall_gemms % LIBRPA_TEST_STALL_OASM / LIBRPA_TEST_STALL_WIDE;
+  h->stalls_oasm = o->test_stall_gemms / LIBRPA_TEST_STALL_OASM;
   {
     // arithmetic per stage (-1 = FP64 pipes, 0 = plain BF16, 1..5 = digit planes, 6 = plain
     // TF32, 7 = 3xTF32): presets, then explicit overrides

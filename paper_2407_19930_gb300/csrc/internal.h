@@ -170,7 +170,10 @@ struct Handle {
   DevBuf work;        // per-call workspace
   double oz_exec_flops = 0;  // MMA flops issued by the last digit-plane GEMM launch
   double oz_alg_flops = 0;   // algorithmic flops (2 M N K over the summed K) of that launch
-  int stalls_left = 0;       // testing only: tensor-core GEMM launches still to take the failure path
+  // testing only: launches still to take the failure path (GEMMs with up to 5 planes, with 8, O assemblies)
+  int stalls_left = 0, stalls_wide = 0, stalls_oasm = 0;
+  static constexpr uint64_t kStallNs = 100000;   // per CTA
+  static uint64_t stall_ns(int &left) { return left > 0 ? (--left, kStallNs) : 0; }
   double flop_chi0_run = 0;  // algorithmic flops of the last contraction (screened work left out)
   bool chi0_done = false, lri_dirty = true;
   Chi0Plan plan;

@@ -792,7 +792,8 @@ bool run_oassemble(Handle &h, const Point *dpts, int np, double *Nw, double *Xw,
     t.aux_atom = (const int *)P.t_aux_atom.p;
     t.ao_row = (const int *)P.t_ao_row.p;
     t.max_tiles = P.oasm_max_tiles;
-    oasm::run(otc, oa, t, np, *tc->nd, *tc->xd, tc->rexp, tc->err, h.stream);
+    oasm::run(otc, oa, t, np, *tc->nd, *tc->xd, tc->rexp, tc->err, Handle::stall_ns(h.stalls_oasm),
+              h.stream);
     return true;
   }
   // arithmetic: FP64 pipes for the FP64 mode, FP32 for the mixed modes, FP32 pairs (~48 bits)

@@ -238,13 +238,13 @@ __device__ __forceinline__ double combine(const uint32_t (&r1)[S][4], const uint
 template <int S>
 __global__ void __launch_bounds__(kThreads, 1)
     k_oasm(OArgs a, Tables tb, const __grid_constant__ CUtensorMap nmap, const __grid_constant__ CUtensorMap xmap,
-           const int *__restrict__ nexp, const int *__restrict__ xexp, int *rexp, int *err) {
+           const int *__restrict__ nexp, const int *__restrict__ xexp, int *rexp, int *err, uint64_t stall_ns) {
   using E_ = Elem<S>;
   constexpr int NST = ring(S), NSL = slots(S), SL = slot_cols(S);
   constexpr int NU = nus(S);
   constexpr uint32_t OPB = op_bytes(S), XB_ = x_bytes(S), FIXED = static_size(S), STAGE = stage_size(S);
   extern __shared__ uint8_t smem_raw[];
-  __shared__ uint64_t full[NST], empty[NST], tfull[NSL], tempty[NSL], mdone;
+  __shared__ uint64_t full[NST], empty[NST], tfull[NSL], tempty[NSL], mdone, never;
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
   __shared__ int s_e1[kMaxAo], s_box[kTileGroups];
@@ -292,6 +292,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&tempty[s], 8);
     }
     mbar_init(&mdone, 1);
+    mbar_init(&never, 1);
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -398,6 +399,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == kEpi + 1) {
     if (elect_one()) {   // MMA issuer
+      if (stall_ns) {   // testing only: a barrier nothing arrives at
+        mbar_wait(&never, 0, stall_ns, &abort_flag);
+        abort_flag = 1;
+      }
       const int ks = (two + 15) / 16;
       const uint32_t rg = smem_u32(sRG), lm = smem_u32(sLm);
       for (int it = 0; it < nauxV; ++it) {
@@ -529,7 +534,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 template <int S>
-void launch(const OArgs &a, const Tables &t, int np, oz::Sliced &nd, oz::Sliced &xd, int *expo, int *err, cudaStream_t s) {
+void launch(const OArgs &a, const Tables &t, int np, oz::Sliced &nd, oz::Sliced &xd, int *expo, int *err, uint64_t stall_ns,
+            cudaStream_t s) {
   static_assert(smem_size(S) <= 227 * 1024, "k_oasm: shared memory");
   const unsigned rows = (unsigned)(np * a.naux);
   k_split_n<S><<<dim3(rows, (unsigned)((a.m_all + 127) / 128)), 256, 0, s>>>(
@@ -539,7 +545,8 @@ void launch(const OArgs &a, const Tables &t, int np, oz::Sliced &nd, oz::Sliced 
   LR_CUDA(cudaFuncSetAttribute(k_oasm<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_size(S)));
   k_oasm<S><<<(unsigned)t.max_tiles * (unsigned)(np * a.natoms * a.natoms), kThreads, smem_size(S), s>>>(
       a, t, oz::make_map_nested(nd.digits, a.m_all, S, (int)rows, 8, nus(S)),
-      oz::make_map_nested(xd.digits, a.natoms * kMaxAo, S, (int)rows, kMaxAo, nus(S)), nd.expo, xd.expo, expo, err);
+      oz::make_map_nested(xd.digits, a.natoms * kMaxAo, S, (int)rows, kMaxAo, nus(S)), nd.expo, xd.expo, expo, err,
+      stall_ns);
   launch_counter() += 3;
   LR_CUDA(cudaGetLastError());
 }
@@ -547,14 +554,14 @@ void launch(const OArgs &a, const Tables &t, int np, oz::Sliced &nd, oz::Sliced 
 }  // namespace
 
 void run(int S, const OArgs &a, const Tables &t, int np, oz::Sliced &nd, oz::Sliced &xd, int *expo, int *err,
-         cudaStream_t s) {
+         uint64_t stall_ns, cudaStream_t s) {
   oz::init();
   if (S == 3)
-    launch<3>(a, t, np, nd, xd, expo, err, s);
+    launch<3>(a, t, np, nd, xd, expo, err, stall_ns, s);
   else if (S == 5)
-    launch<5>(a, t, np, nd, xd, expo, err, s);
+    launch<5>(a, t, np, nd, xd, expo, err, stall_ns, s);
   else
-    launch<oz::S_WIDE>(a, t, np, nd, xd, expo, err, s);
+    launch<oz::S_WIDE>(a, t, np, nd, xd, expo, err, stall_ns, s);
 }
 
 }  // namespace oasm

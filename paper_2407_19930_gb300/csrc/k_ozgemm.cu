@@ -1235,12 +1235,7 @@ long long gemm_multi(const std::vector<std::pair<const Sliced *, const Sliced *>
   int nsm = 0;
   LR_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h.opts.device));
   const int nt = (int)tk.size(), grid = std::min(nt, nsm);
-  // testing only: the handle's first opts.test_stall_gemms launches take the failure path
-  uint64_t stall = 0;
-  if (h.stalls_left > 0 && S != S_WIDE) {
-    --h.stalls_left;
-    stall = 100000;   // 100 us per CTA
-  }
+  const uint64_t stall = Handle::stall_ns(S == S_WIDE ? h.stalls_wide : h.stalls_left);   // testing only
   const Launch l{dm, de, dt, dc, nt, grid, err, stall, s};
   int ms = 0;
   for (const auto &x : tk) ms = std::max(ms, x.first);

@@ -38,6 +38,8 @@ LIBRPA_GRID_GAUSS_LEGENDRE = 1
 LIBRPA_NOALLOC_SCRATCH_BYTES = 16 << 20
 LIBRPA_NOALLOC_MAX_NAUX = 591
 
+LIBRPA_TEST_STALL_WIDE, LIBRPA_TEST_STALL_OASM = 1 << 20, 1 << 26   # units of opts.test_stall_gemms
+
 _CODES = {v: k for k, v in globals().items() if k.startswith("LIBRPA_E_")}
 
 ALLOC_FN = ctypes.CFUNCTYPE(ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p)
