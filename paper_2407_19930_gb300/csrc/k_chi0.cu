@@ -1564,6 +1564,7 @@ void tc_merged(std::vector<Handle *> &hs) {
     Handle &h = *hs[i];
     h.cur_spin = 0;
     rs[i] = tc_views(h, &npb[i]);
+    rs[i].err = rs[0].err;   // one flag for the whole sequence: the GEMMs' and every handle's O assembly
     const std::vector<int> rl = chi0_r_list(h.mesh);
     pts[i] = make_points(h, rl, 0, (int)(h.ntau * rl.size()));
     h.stats.n_points_chi0 = (long long)pts[i].size();
