@@ -26,6 +26,7 @@
 
 #include "internal.h"
 #include "ozgemm.h"
+#include "tc.h"
 
 namespace librpa {
 namespace {
@@ -380,9 +381,36 @@ __global__ void k_real_transpose(const double2 *L, int n, double *Lt) {
   }
 }
 
-__global__ void k_real_part(const double2 *src, size_t count, double *dst) {
-  const size_t x = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (x < count) dst[x] = src[x].x;
+// real parts of n x n matrices, a row per CTA; eq (or NULL): element (i, j) times 2^-(eq[i] + eq[j])
+__global__ void k_real_part(const double2 *src, int n, const int *eq, double *dst) {
+  const size_t row = (size_t)blockIdx.x * n;
+  const int ei = eq ? eq[blockIdx.x % n] : 0;
+  for (int j = threadIdx.x; j < n; j += blockDim.x) {
+    const double v = src[row + j].x;
+    dst[row + j] = eq ? scale_pow2(v, -(ei + eq[j])) : v;
+  }
+}
+
+// Equilibration of the 8-plane route.  A digit plane holds an element to 2^-63 of its row's largest, where FP64 holds
+// every element to 53 bits of its own, so functions of widely different norms would lose the small ones (aux functions
+// scaled over 2^30: ln det off by 4e-12, over 2^40 by 1e-8, against 1e-15 in FP64).  The integrand does not change under
+// V -> D V D, chi0 -> D^-1 chi0 D^-1, so each V(q) is taken with D_i = 2^eq[i] that brings its diagonal into [1, 4):
+// powers of two, exact, and L^H chi0 L is the same matrix.
+__global__ void k_equil_expo(const double2 *const *V, int n, int *eq) {   // eq[q][i]
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double v = V[blockIdx.y][(size_t)i * n + i].x;
+  const int ex = biased_exp(v);
+  eq[(size_t)blockIdx.y * n + i] = v > 0.0 && ex > 0 && ex < 2047 ? -((ex - 1023) >> 1) : 0;
+}
+__global__ void k_equil_scale(double2 *const *V, int n, const int *eq) {   // a row per CTA
+  double2 *row = V[blockIdx.y] + (size_t)blockIdx.x * n;
+  eq += (size_t)blockIdx.y * n;
+  const int ei = eq[blockIdx.x];
+  for (int j = threadIdx.x; j < n; j += blockDim.x) {
+    const int e = ei + eq[j];
+    if (e) row[j] = make_double2(scale_pow2(row[j].x, e), scale_pow2(row[j].y, e));
+  }
 }
 
 struct RGemm {
@@ -735,7 +763,7 @@ size_t al256(size_t b) { return (b + 255) / 256 * 256; }
 // lndet/trace/info, output, and for the tensor-core route the digit planes.
 struct EcLayout {
   size_t o_L, o_W, o_A, o_ptr, o_ld, o_tr, o_ldc, o_trc, o_inf, o_out, o_wo, o_wq, o_err;
-  size_t o_sx = 0, o_sw = 0, o_sl = 0, o_slh = 0, o_pa = 0, o_pb = 0, o_inv = 0, o_pi = 0;
+  size_t o_sx = 0, o_sw = 0, o_sl = 0, o_slh = 0, o_pa = 0, o_pb = 0, o_inv = 0, o_pi = 0, o_eq = 0;
   size_t total = 0;
 };
 
@@ -778,6 +806,7 @@ EcLayout ec_layout(const Handle &h) {
     l.o_inv = take((size_t)bmax * NB * NB * sizeof(double2));
     l.o_pi = take(std::max(oz::sliced_bytes(bmax * NB, 2 * NB, S), oz::sliced_bytes(bmax * NB, NB, oz::S_WIDE)));
   }
+  if (S == oz::S_WIDE) l.o_eq = take((size_t)nq * n * 4);
   l.total = off;
   return l;
 }
@@ -872,6 +901,14 @@ int ec_run(Handle &h, double *ec, double *ec_q, double *ec_w) {
     LR_CUDA(cudaMemcpyAsync(lp[i], (const char *)h.d_vq.p + (size_t)qlist[i] * mat, mat, cudaMemcpyDeviceToDevice, s));
   }
   LR_CUDA(cudaMemcpyAsync(ptrs, lp.data(), nql * 8, cudaMemcpyHostToDevice, s));
+  int *eq = S == oz::S_WIDE ? (int *)(w + lay.o_eq) : nullptr;   // [qlist][n]
+  if (eq) {
+    k_equil_expo<<<dim3((unsigned)((n + 255) / 256), (unsigned)nql), 256, 0, s>>>(ptrs, n, eq);
+    k_equil_scale<<<dim3((unsigned)n, (unsigned)nql), 256, 0, s>>>(ptrs, n, eq);
+    launch_counter() += 2;
+    LR_CUDA(cudaGetLastError());
+  }
+  auto eq_of = [&](int qi) { return eq ? eq + (size_t)qi * n : nullptr; };
   potrf_batched(h, ptrs, lp, n, n, lndet_v, info, tc);
   {
     dim3 g((unsigned)((n2 + 255) / 256), (unsigned)nql);
@@ -902,7 +939,8 @@ int ec_run(Handle &h, double *ec, double *ec_q, double *ec_w) {
         const double2 *L = Lq + (size_t)qi * n2;
         oz::split_complex(L, n, oz::OP_N, false, n, n, 1, 0, sl, s);     // B'^T of W = chi0 L
         oz::split_complex(L, n, oz::OP_H, true, n, n, 1, 0, slh, s);     // A' of L^H W
-        oz::split_complex(chi + (size_t)q * nw * n2, n, oz::OP_N, true, n, n, nw, (long long)n2, sx, s);
+        oz::split_complex(chi + (size_t)q * nw * n2, n, oz::OP_N, true, n, n, nw, (long long)n2, sx, s,
+                          eq_of(qi));
         // W^T, so that the second GEMM reads W column by column as rows.  A = -L^H W reads W only on
         // and below its diagonal tiles (k >= j): the tiles above are not computed and stay zero
         // (the digit planes of W's rows see zeros there)
@@ -990,8 +1028,7 @@ int ec_run(Handle &h, double *ec, double *ec_q, double *ec_w) {
     for (int r = 0; r < nr; ++r) {
       const int qi = order[nx + r], q = qlist[qi];
       k_real_transpose<<<dim3(nt, nt), dim3(32, 8), 0, s>>>(Lq + (size_t)qi * n2, n, Lt);
-      const size_t cnt = (size_t)nw * n2;
-      k_real_part<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(chi + (size_t)q * nw * n2, cnt, Xr);
+      k_real_part<<<(unsigned)(nw * n), 256, 0, s>>>(chi + (size_t)q * nw * n2, n, eq_of(qi), Xr);
       launch_counter() += 2;
       LR_CUDA(cudaGetLastError());
       if (S >= 0) {

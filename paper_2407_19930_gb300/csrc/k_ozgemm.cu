@@ -49,7 +49,16 @@ struct CplxSrc {
   long long ld, bstride;
   int rows_pb, op;
   bool as_a;
+  const int *eq;
   __device__ double2 opget(const double2 *q, int i, int k) const {
+    double2 z = opget_plain(q, i, k);
+    if (eq) {
+      const int e = -(eq[i] + eq[k]);
+      z = make_double2(scale_pow2(z.x, e), scale_pow2(z.y, e));
+    }
+    return z;
+  }
+  __device__ double2 opget_plain(const double2 *q, int i, int k) const {
     if (op == OP_N) return q[(long long)i * ld + k];
     if (op == OP_C) {
       const double2 z = q[(long long)i * ld + k];
@@ -1053,9 +1062,9 @@ void split_real(const double *src, long long ld, bool trans, int rows, int K, in
 }
 
 void split_complex(const double2 *src, long long ld, Op op, bool as_a, int n_out, int n_k, int batch,
-                   long long batch_stride, Sliced &out, cudaStream_t s) {
+                   long long batch_stride, Sliced &out, cudaStream_t s, const int *eq) {
   const int rows_pb = as_a ? 2 * n_out : n_out;
-  CplxSrc c{src, ld, batch_stride, rows_pb, (int)op, as_a};
+  CplxSrc c{src, ld, batch_stride, rows_pb, (int)op, as_a, eq};
   split_any(c, rows_pb * batch, 2 * n_k, 0, out, s);
 }
 

@@ -15,6 +15,14 @@ namespace {
 
 __device__ __forceinline__ int biased_exp(double v) { return (int)((__double_as_longlong(v) >> 52) & 0x7FF); }
 
+// v 2^e, exact while the result is a normal number (integer instructions; else through FP64)
+__device__ __forceinline__ double scale_pow2(double v, int e) {
+  const int ex = biased_exp(v);
+  if (ex > 0 && ex < 2047 && (unsigned)(ex + e - 1) < 2046u)
+    return __longlong_as_double(__double_as_longlong(v) + ((long long)e << 52));
+  return scalbn(v, e);
+}
+
 // balanced base-256 digits of x = v 2^-E (|x| < 1): x ~ sum_s d_s 2^{-7-8(s-1)}, |d_s| <= 128, as FP32 integers.
 // W = x 2^{7+8(S-1)} rounded (half up in magnitude); with 128 added at every lower digit's place the digits are the
 // bytes of the sum less 128, and a byte b becomes a float by the bits of 2^23 + b.
