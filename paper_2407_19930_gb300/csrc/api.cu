@@ -364,6 +364,7 @@ int librpa_gpu_set_structure(librpa_gpu_t h, int natoms, const double lat[9], co
     h->efermi_k.assign((size_t)nspins * nk, 0.0);
     h->have_q.assign(nk, 0);
     h->have_grid = h->grid_user = false;
+    h->ao_e.clear();
     h->chi0_done = false;
     h->lri_dirty = true;
     h->have_structure = true;
@@ -648,6 +649,9 @@ int librpa_gpu_get_green(librpa_gpu_t h, int itau, int iR, double *go, double *g
     const size_t off = ((size_t)itau * h->mesh.size() + iR) * n2;
     if (go) LR_CUDA(cudaMemcpy(go, (double *)h->d_g.p + off, n2 * 8, cudaMemcpyDeviceToHost));
     if (gv) LR_CUDA(cudaMemcpy(gv, (double *)h->d_g.p + slab + off, n2 * 8, cudaMemcpyDeviceToHost));
+    if (!h->ao_e.empty())   // back to the caller's NAOs
+      for (double *g : {go, gv})
+        for (size_t x = 0; g && x < n2; ++x) g[x] = std::ldexp(g[x], h->ao_e[x / h->nao] + h->ao_e[x % h->nao]);
     return LIBRPA_OK;
   });
 }

@@ -112,6 +112,8 @@ struct Handle {
   int chi0_S = -1;  // chi0 GEMMs: -1 = FP64 pipes, 0 = plain BF16, 1..5 = BF16 digit planes, 6 = plain TF32,
                     // 7 = 3xTF32
   int ec_S = -1;    // ln det GEMMs: same encoding
+  // FP64 mode: the stored G and the packed C are those of NAOs rescaled by 2^-ao_e[i] (k_green.cu); empty: as passed
+  std::vector<int> ao_e;
   bool freq_f32 = false;   // tau -> omega and R -> q transforms in FP32 (LIBRPA_SPLIT_FAST)
   cudaStream_t stream = nullptr;
   bool own_stream = false;

@@ -22,6 +22,7 @@
 // G blocks gathered at the lattice vectors above, and O_U[nu][(i,(K,R1,k))] is assembled by a
 // dedicated kernel.  The GEMMs run on the FP64 tensor cores (mma.sync m8n8k4 .f64).
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <functional>
 #include <set>
@@ -592,6 +593,13 @@ void chi0_plan(Handle &h) {
         for (int i = 0; i < nU; ++i)
           for (int k = 0; k < nK; ++k)
             cp[P.cp_off[U] + ((size_t)mu * nU + i) * mU + e.col + k] = C[((size_t)mu * nU + i) * nK + k];
+      if (h.ao_e.empty()) continue;
+      std::vector<double> fi(nU), fk(nK);   // in units of the rescaled NAOs, as G
+      for (int i = 0; i < nU; ++i) fi[i] = std::ldexp(1.0, h.ao_e[h.ao_off[U] + i]);
+      for (int k = 0; k < nK; ++k) fk[k] = std::ldexp(1.0, h.ao_e[h.ao_off[e.K] + k]);
+      for (int mu = 0; mu < h.n_aux[U]; ++mu)
+        for (int i = 0; i < nU; ++i)
+          for (int k = 0; k < nK; ++k) cp[P.cp_off[U] + ((size_t)mu * nU + i) * mU + e.col + k] *= fi[i] * fk[k];
     }
   }
   upload(h, h.d_cpack, cp);

@@ -14,6 +14,7 @@
 
 #include "internal.h"
 #include "ozgemm.h"
+#include "tc.h"
 
 namespace librpa {
 namespace {
@@ -22,6 +23,45 @@ namespace {
 // from kWideMinAo NAOs on (-1: the FP64 pipes)
 constexpr int kWideMinAo = 64;
 int green_planes(const Handle &h) { return h.chi0_S >= 0 ? 5 : h.nao >= kWideMinAo ? oz::S_WIDE : -1; }
+
+// Equilibration of the NAOs for the FP64 mode's digit planes, which hold an element to 2^-63 of its row's largest: in a
+// product over NAOs a row of C grows with the norms of its columns where a row of G falls, so a spread of 2^12 among
+// the norms costs bits that FP64 keeps (2^20: 1e-11 against 4e-15).  G and C are taken in units of NAOs rescaled by the
+// powers of two ao_e of their largest coefficient, exact in both and without effect on chi0.  A spread of up to
+// 2^kAoSpread stays: the final contraction, over pairs of NAOs, loses 2 kAoSpread of the 10 bits to spare.
+constexpr int kAoSpread = 3;
+
+// mx[i] = largest biased exponent of the coefficients of NAO i (rows: spins x k x bands)
+__global__ void k_ao_norm(const double2 *__restrict__ wfc, long long rows, int nao, int *mx) {
+  const int i = blockIdx.x * 32 + threadIdx.x;
+  if (i >= nao) return;
+  int m = 0;
+  for (long long r = blockIdx.y * 8 + threadIdx.y; r < rows; r += gridDim.y * 8) {
+    const double2 c = wfc[r * nao + i];
+    m = max(m, max(biased_exp(c.x), biased_exp(c.y)));
+  }
+  atomicMax(mx + i, m);
+}
+
+std::vector<int> ao_exponents(const std::vector<int> &mx) {
+  int lo = 2047, hi = 0;
+  for (int m : mx) {
+    if (m == 2047) return {};   // an infinity or a NaN
+    if (m > 0) lo = std::min(lo, m);
+    hi = std::max(hi, m);
+  }
+  if (hi - lo <= kAoSpread) return {};
+  std::vector<int> e;
+  for (int m : mx) e.push_back(m > 0 ? std::max(m - hi, -400) : 0);
+  return e;
+}
+
+// G_ij 2^-(e_i + e_j), a row per CTA
+__global__ void k_scale_green(double *G, const int *e, int nao) {
+  double *row = G + (size_t)blockIdx.x * nao;
+  const int ei = e[blockIdx.x % nao];
+  for (int j = threadIdx.x; j < nao; j += blockDim.x) row[j] = scale_pow2(row[j], -(ei + e[j]));
+}
 
 // Y[g][k][n][i] = sqrt(w[g][k][n]) c_in(k) (the weights are >= 0), so that P^g_k = Y^T conj(Y)
 __global__ void k_scale_bands(const double2 *wfc, const double *w, int nk, int nb, int nao, double2 *Y) {
@@ -163,7 +203,7 @@ size_t green_work_bytes(const Handle &h) {
   const size_t nk = h.mesh.size(), nR = nk, nb = h.nao, n2 = (size_t)h.nao * h.nao;
   const size_t b_e = nk * nb * 8, b_w = 2 * b_e, b_p = 2 * nk * n2 * 16, b_t = nk * nR * 16;
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-  size_t b = al(b_w) + al(b_p) + al(b_t) + al(nR * sizeof(int2)) + 256;
+  size_t b = al(b_w) + al(b_p) + al(b_t) + al(nR * sizeof(int2)) + al(h.nao * sizeof(int)) + 256;
   const int S = green_planes(h);
   if (S >= 0)   // digit planes: Y and the digit planes of both GEMM roles
     b += al(b_p) + oz::sliced_bytes((int)(2 * nk * 2 * h.nao), (int)(2 * nb), S) +
@@ -181,8 +221,9 @@ double green_build(Handle &h) {
   const size_t b_e = (size_t)nk * nb * 8, b_w = 2 * b_e, b_p = 2 * (size_t)nk * n2 * 16,
                b_t = (size_t)nk * nR * 16;
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-  const size_t b_rl = (size_t)nR * sizeof(int2);
-  const size_t o_w = 0, o_p = o_w + al(b_w), o_t = o_p + al(b_p), o_rl = o_t + al(b_t), o_m = o_rl + al(b_rl);
+  const size_t b_rl = (size_t)nR * sizeof(int2), b_ao = (size_t)nao * sizeof(int);
+  const size_t o_w = 0, o_p = o_w + al(b_w), o_t = o_p + al(b_p), o_rl = o_t + al(b_t), o_ao = o_rl + al(b_rl),
+               o_m = o_ao + al(b_ao);
   // digit planes: P^g_k = Y^T conj(Y) as one batched digit-plane GEMM per tau (FP64-accurate)
   const int S = green_planes(h);
   const bool tc = S >= 0;
@@ -226,6 +267,17 @@ double green_build(Handle &h) {
   LR_CUDA(cudaMemcpyAsync(d_rl, rl.data(), rl.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
   LR_CUDA(cudaStreamSynchronize(s));   // tw and rl are host temporaries
   LR_CUDA(cudaMemsetAsync(d_max, 0, 16, s));
+  int *d_ao = (int *)(wk + o_ao);
+  std::vector<int> ao_mx(h.chi0_S < 0 ? nao : 0);
+  if (!ao_mx.empty()) {
+    const long long rows = (long long)h.nspins * nk * nb;
+    LR_CUDA(cudaMemsetAsync(d_ao, 0, b_ao, s));
+    k_ao_norm<<<dim3((unsigned)((nao + 31) / 32), (unsigned)std::min<long long>(64, (rows + 31) / 32)), dim3(32, 8), 0, s>>>(
+        d_wfc0, rows, nao, d_ao);
+    ++launch_counter();
+    LR_CUDA(cudaGetLastError());
+    LR_CUDA(cudaMemcpyAsync(ao_mx.data(), d_ao, b_ao, cudaMemcpyDeviceToHost, s));
+  }
   const size_t g_stride = (size_t)ntau * nR * n2;
   for (int sp = 0; sp < h.nspins; ++sp) {   // one spin channel at a time, own KS data, own G
     const double2 *d_wfc = d_wfc0 + (size_t)sp * nk * nb * nao;
@@ -301,6 +353,17 @@ double green_build(Handle &h) {
   LR_CUDA(cudaStreamSynchronize(s));
   if (e_host) throw Error{LIBRPA_E_TIMEOUT, "Green's function: a bounded wait in the tensor-core GEMM ran out"};
   green_screen(h);   // after the imaginary-part check's maxima: they describe the unscreened G
+  const std::vector<int> e = ao_exponents(ao_mx);
+  if (e != h.ao_e) {   // C is packed in the same units
+    h.ao_e = e;
+    h.lri_dirty = true;
+  }
+  if (!e.empty()) {
+    LR_CUDA(cudaMemcpyAsync(d_ao, h.ao_e.data(), b_ao, cudaMemcpyHostToDevice, s));
+    k_scale_green<<<(unsigned)(2 * h.nspins * (size_t)ntau * nR * nao), 128, 0, s>>>((double *)h.d_g.p, d_ao, nao);
+    ++launch_counter();
+    LR_CUDA(cudaGetLastError());
+  }
   double mre, mim;
   std::memcpy(&mre, &mx[0], 8);
   std::memcpy(&mim, &mx[1], 8);

@@ -45,3 +45,39 @@ def test_auxiliary_functions(spread):
     ec2, ec_q2, ec_w2 = _run(s, grid)
     # powers of two change no rounding
     assert ec2 == ec and np.array_equal(ec_q2, ec_q) and np.array_equal(ec_w2, ec_w)
+
+
+@pytest.mark.parametrize("spread", [4, 16, 30])
+def test_atomic_orbitals(spread):
+    inp, grid = _inputs()
+    st = inp.st
+    ec, ec_q, _ = _run(inp, grid)
+    e = np.random.default_rng(6).integers(-spread // 2, spread // 2 + 1, st.nao)
+    a = 2.0 ** e
+    off = np.concatenate([[0], np.cumsum(st.n_ao)])
+    s = copy.copy(inp)
+    s.wfc = inp.wfc * a
+    s.lri = [(I, K, R, C / a[off[I]:off[I + 1], None] / a[off[K]:off[K + 1]]) for I, K, R, C in inp.lri]
+    ec2, ec_q2, _ = _run(s, grid)
+    # products of 63-bit operands whose rows spread over at most 2^6 more than without the rescaling (2^-57 of
+    # an element), each stored with 53 bits: the two energies differ by a few times 2^-53 of the sums over N_aux
+    assert abs(ec2 - ec) <= 1e-12 * abs(ec) and np.abs(ec_q2 - ec_q).max() <= 1e-12 * np.abs(ec_q).max()
+
+
+def test_green_function_in_the_callers_orbitals():
+    inp, grid = _inputs()
+    st = inp.st
+    a = 2.0 ** np.random.default_rng(6).integers(-15, 16, st.nao)
+    s = copy.copy(inp)
+    s.wfc = inp.wfc * a
+    s.lri = [(I, K, R, np.zeros_like(C)) for I, K, R, C in inp.lri]
+    g = []
+    for x in (inp, s):
+        h = L.librpa_gpu_create(L.librpa_gpu_default_opts())
+        try:
+            L.set_inputs(h, x, grid)
+            L.librpa_gpu_chi0(h)
+            g.append([L.librpa_gpu_get_green(h, it, r, st.nao) for it in range(len(grid["tau"])) for r in range(st.nk)])
+        finally:
+            L.librpa_gpu_destroy(h)
+    assert np.array_equal(np.array(g[1]), np.array(g[0]) * a[:, None] * a)   # powers of two
