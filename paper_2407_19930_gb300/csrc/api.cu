@@ -172,6 +172,14 @@ void free_device_state(Handle &h) {
 
 void release_device(Handle &h) { free_device_state(h); }
 
+void drop_scratch(Handle &h) {
+  cudaStreamSynchronize(h.stream);
+  h.resolve_timers();   // of the launches before the failure
+  cudaGetLastError();
+  for (DevBuf *b : {&h.work, &h.plan.ws, &h.plan.cp_nx, &h.plan.cp_f}) h.release(*b);
+  h.lri_dirty = true;
+}
+
 void materialize(Handle &h) {
   if (!h.deferred) return;
   const size_t nq = h.mesh.size(), nk = (size_t)h.nspins * nq, nb = h.nao, per_k = nb * h.nao,
@@ -191,7 +199,9 @@ void materialize(Handle &h) {
   LR_CUDA(cudaStreamSynchronize(h.stream));
 }
 
-size_t estimate_device_bytes(Handle &h) {
+size_t estimate_device_bytes(Handle &h, bool lean) {
+  const bool lean_saved[2] = {h.lean_chi0, h.lean_ec};
+  if (lean) h.lean_chi0 = h.lean_ec = true;
   const int ntau_saved = h.ntau;
   if (!h.have_grid) h.ntau = h.opts.n_tau;
   const size_t nk = h.mesh.size(), ns = h.nspins, nb = h.nao, n2ao = (size_t)h.nao * h.nao,
@@ -208,6 +218,8 @@ size_t estimate_device_bytes(Handle &h) {
   if (h.g_screen > 0)                                             // block mask, atom tables
     b += ns * 2 * (size_t)h.ntau * nk * h.natoms * h.natoms + 8 * (size_t)h.natoms + 512;
   h.ntau = ntau_saved;
+  h.lean_chi0 = lean_saved[0];
+  h.lean_ec = lean_saved[1];
   return b;
 }
 
@@ -365,6 +377,7 @@ int librpa_gpu_set_structure(librpa_gpu_t h, int natoms, const double lat[9], co
     h->have_q.assign(nk, 0);
     h->have_grid = h->grid_user = false;
     h->ao_e.clear();
+    h->lean_chi0 = h->lean_ec = false;
     h->chi0_done = false;
     h->lri_dirty = true;
     h->have_structure = true;
@@ -558,21 +571,24 @@ int librpa_gpu_chi0(librpa_gpu_t h, double *out_re, double *out_im) {
   return guarded(h, [&]() -> int {
     if (int rc = chi0_prepare(*h)) return rc;
     materialize(*h);
-    h->stats = librpa_gpu_stats{};
     long long l0 = launch_counter();
     cudaEvent_t ev[4];
     for (auto &e : ev) LR_CUDA(cudaEventCreate(&e));
     LR_CUDA(cudaEventRecord(ev[0], h->stream));
-    double imag = green_build(*h);
-    LR_CUDA(cudaEventRecord(ev[1], h->stream));
-    if (h->lri_dirty) {
-      chi0_plan(*h);
-      h->lri_dirty = false;
-    }
-    double ms_gemm = 0;
-    chi0_run(*h, &ms_gemm);
-    LR_CUDA(cudaEventRecord(ev[2], h->stream));
-    freq_transform(*h);
+    double imag = 0;
+    with_memory({h}, &Handle::lean_chi0, [&] {
+      h->resolve_timers();
+      h->stats = librpa_gpu_stats{};
+      imag = green_build(*h);
+      LR_CUDA(cudaEventRecord(ev[1], h->stream));
+      if (h->lri_dirty) {
+        chi0_plan(*h);
+        h->lri_dirty = false;
+      }
+      chi0_run(*h, nullptr);
+      LR_CUDA(cudaEventRecord(ev[2], h->stream));
+      freq_transform(*h);
+    });
     LR_CUDA(cudaEventRecord(ev[3], h->stream));
     LR_CUDA(cudaStreamSynchronize(h->stream));
     float t;
@@ -619,7 +635,8 @@ int librpa_gpu_ec(librpa_gpu_t h, double *ec, double *ec_q, double *ec_w) {
     LR_CUDA(cudaEventCreate(&e0));
     LR_CUDA(cudaEventCreate(&e1));
     LR_CUDA(cudaEventRecord(e0, h->stream));
-    int rc = ec_run(*h, ec, ec_q, ec_w);
+    int rc = LIBRPA_OK;
+    with_memory({h}, &Handle::lean_ec, [&] { rc = ec_run(*h, ec, ec_q, ec_w); });
     LR_CUDA(cudaEventRecord(e1, h->stream));
     LR_CUDA(cudaStreamSynchronize(h->stream));
     float t;

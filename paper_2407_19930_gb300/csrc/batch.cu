@@ -58,16 +58,20 @@ void run_own(Handle &h, cudaStream_t ws, double *ec) {
     ~Restore() { h.stream = s; }
   } restore{h, saved};
   materialize(h);
-  h.stats = librpa_gpu_stats{};
-  const double imag = green_build(h);
-  if (h.lri_dirty) {
-    chi0_plan(h);
-    h.lri_dirty = false;
-  }
-  chi0_run(h, nullptr);
-  freq_transform(h);
+  double imag = 0;
+  with_memory({&h}, &Handle::lean_chi0, [&] {
+    h.stats = librpa_gpu_stats{};
+    imag = green_build(h);
+    if (h.lri_dirty) {
+      chi0_plan(h);
+      h.lri_dirty = false;
+    }
+    chi0_run(h, nullptr);
+    freq_transform(h);
+  });
   h.chi0_done = true;
-  const int rc = ec_run(h, ec, nullptr, nullptr);
+  int rc = LIBRPA_OK;
+  with_memory({&h}, &Handle::lean_ec, [&] { rc = ec_run(h, ec, nullptr, nullptr); });
   if (rc == LIBRPA_E_NOT_PD) throw Error{rc, "ec: a Cholesky pivot was <= 0"};
   if (rc) throw Error{rc, "ec: a bounded device wait ran out"};
   h.release(h.d_chi_qw);
@@ -75,6 +79,38 @@ void run_own(Handle &h, cudaStream_t ws, double *ec) {
   h.chi0_done = false;
   h.resolve_timers();
   if (h.opts.check_level >= 1 && !(imag <= 1e-10)) throw Error{LIBRPA_E_NUMERIC, "batch: G(R, tau) has an imaginary part"};
+}
+
+// the sequence of run_tc_group
+void run_tc_group_once(std::vector<Handle *> &g, double *const *ec, int *failed, std::vector<double> &imag) {
+  for (size_t i = 0; i < g.size(); ++i) {
+    *failed = (int)i;
+    Handle &h = *g[i];
+    materialize(h);
+    h.stats = librpa_gpu_stats{};
+    imag[i] = green_build(h);
+    if (h.lri_dirty) {
+      chi0_plan(h);
+      h.lri_dirty = false;
+    }
+  }
+  *failed = 0;
+  chi0_run_tc_merged(g);
+  for (size_t i = 0; i < g.size(); ++i) {
+    *failed = (int)i;
+    Handle &h = *g[i];
+    freq_transform(h);
+    h.chi0_done = true;
+    int rc = LIBRPA_OK;
+    with_memory({&h}, &Handle::lean_ec, [&] { rc = ec_run(h, ec[i], nullptr, nullptr); });
+    if (rc == LIBRPA_E_NOT_PD) throw Error{rc, "ec: a Cholesky pivot was <= 0"};
+    if (rc) throw Error{rc, "ec: a bounded device wait ran out"};
+    h.release(h.d_chi_qw);
+    h.release(h.work);
+    h.chi0_done = false;
+    h.resolve_timers();
+    if (h.opts.check_level >= 1 && !(imag[i] <= 1e-10)) throw Error{LIBRPA_E_NUMERIC, "batch: G(R, tau) has an imaginary part"};
+  }
 }
 
 // A group of tensor-core handles with the same digit-plane count on stream `ws`: G per handle, the
@@ -95,33 +131,7 @@ void run_tc_group(std::vector<Handle *> &g, cudaStream_t ws, double *const *ec, 
     }
   } restore{g, saved};
   std::vector<double> imag(g.size());
-  for (size_t i = 0; i < g.size(); ++i) {
-    *failed = (int)i;
-    Handle &h = *g[i];
-    materialize(h);
-    h.stats = librpa_gpu_stats{};
-    imag[i] = green_build(h);
-    if (h.lri_dirty) {
-      chi0_plan(h);
-      h.lri_dirty = false;
-    }
-  }
-  *failed = 0;
-  chi0_run_tc_merged(g);
-  for (size_t i = 0; i < g.size(); ++i) {
-    *failed = (int)i;
-    Handle &h = *g[i];
-    freq_transform(h);
-    h.chi0_done = true;
-    const int rc = ec_run(h, ec[i], nullptr, nullptr);
-    if (rc == LIBRPA_E_NOT_PD) throw Error{rc, "ec: a Cholesky pivot was <= 0"};
-    if (rc) throw Error{rc, "ec: a bounded device wait ran out"};
-    h.release(h.d_chi_qw);
-    h.release(h.work);
-    h.chi0_done = false;
-    h.resolve_timers();
-    if (h.opts.check_level >= 1 && !(imag[i] <= 1e-10)) throw Error{LIBRPA_E_NUMERIC, "batch: G(R, tau) has an imaginary part"};
-  }
+  with_memory(g, &Handle::lean_chi0, [&] { run_tc_group_once(g, ec, failed, imag); });
 }
 
 }  // namespace
@@ -237,6 +247,7 @@ int librpa_gpu_batch_run(librpa_gpu_batch_t b, double *ec) {
   for (int i : mi) mh.push_back(hs[i]);
   if (!mh.empty()) {
     StreamSwap swap(mh);
+    const std::vector<Handle *> handles(mh.begin(), mh.end());
     cudaStream_t s = mh[0]->stream;
     int cur = 0;
     cudaEvent_t ev[5] = {}, ev_chi0 = nullptr;
@@ -244,48 +255,52 @@ int librpa_gpu_batch_run(librpa_gpu_batch_t b, double *ec) {
       for (auto &e : ev) LR_CUDA(cudaEventCreate(&e));
       LR_CUDA(cudaEventCreate(&ev_chi0));
       const long long l0 = launch_counter();
-      LR_CUDA(cudaEventRecord(ev[0], s));
       std::vector<double> imag(mh.size());
-      for (cur = 0; cur < (int)mh.size(); ++cur) {
-        materialize(*mh[cur]);
-        mh[cur]->stats = librpa_gpu_stats{};
-        imag[cur] = green_build(*mh[cur]);
-      }
-      LR_CUDA(cudaEventRecord(ev[1], s));
-      std::vector<Handle *> merged;
-      for (cur = 0; cur < (int)mh.size(); ++cur) {
-        Handle &h = *mh[cur];
-        if (h.lri_dirty) {
-          chi0_plan(h);
-          h.lri_dirty = false;
+      with_memory(handles, &Handle::lean_chi0, [&] {
+        LR_CUDA(cudaEventRecord(ev[0], s));
+        t[2] = t[3] = 0;
+        for (cur = 0; cur < (int)mh.size(); ++cur) {
+          materialize(*mh[cur]);
+          mh[cur]->stats = librpa_gpu_stats{};
+          imag[cur] = green_build(*mh[cur]);
         }
-        merged.push_back(&h);
-      }
-      cur = 0;
-      replay = chi0_run_merged(merged, b->m);
-      LR_CUDA(cudaEventRecord(ev_chi0, s));
-      // per handle: transforms and ln det, then its chi0(q, i omega) and workspace are released,
-      // so the batch holds every chi0(R, tau) but one handle's transient buffers at a time
-      for (cur = 0; cur < (int)mh.size(); ++cur) {
-        Handle &h = *mh[cur];
-        LR_CUDA(cudaEventRecord(ev[2], s));
-        freq_transform(h);
-        h.chi0_done = true;
-        LR_CUDA(cudaEventRecord(ev[3], s));
-        const int rc = ec_run(h, &ec[mi[cur]], nullptr, nullptr);
-        if (rc == LIBRPA_E_NOT_PD) throw Error{rc, "ec: a Cholesky pivot was <= 0"};
-        if (rc) throw Error{rc, "ec: a bounded device wait ran out"};
-        LR_CUDA(cudaEventRecord(ev[4], s));
-        LR_CUDA(cudaEventSynchronize(ev[4]));
-        float a = 0, c = 0;
-        cudaEventElapsedTime(&a, ev[2], ev[3]);
-        cudaEventElapsedTime(&c, ev[3], ev[4]);
-        t[2] += a;
-        t[3] += c;
-        h.release(h.d_chi_qw);
-        h.release(h.work);
-        h.chi0_done = false;   // chi0(q, i omega) is gone: ec needs a new chi0
-      }
+        LR_CUDA(cudaEventRecord(ev[1], s));
+        std::vector<Handle *> merged;
+        for (cur = 0; cur < (int)mh.size(); ++cur) {
+          Handle &h = *mh[cur];
+          if (h.lri_dirty) {
+            chi0_plan(h);
+            h.lri_dirty = false;
+          }
+          merged.push_back(&h);
+        }
+        cur = 0;
+        replay = chi0_run_merged(merged, b->m);
+        LR_CUDA(cudaEventRecord(ev_chi0, s));
+        // per handle: transforms and ln det, then its chi0(q, i omega) and workspace are released,
+        // so the batch holds every chi0(R, tau) but one handle's transient buffers at a time
+        for (cur = 0; cur < (int)mh.size(); ++cur) {
+          Handle &h = *mh[cur];
+          LR_CUDA(cudaEventRecord(ev[2], s));
+          freq_transform(h);
+          h.chi0_done = true;
+          LR_CUDA(cudaEventRecord(ev[3], s));
+          int rc = LIBRPA_OK;
+          with_memory({&h}, &Handle::lean_ec, [&] { rc = ec_run(h, &ec[mi[cur]], nullptr, nullptr); });
+          if (rc == LIBRPA_E_NOT_PD) throw Error{rc, "ec: a Cholesky pivot was <= 0"};
+          if (rc) throw Error{rc, "ec: a bounded device wait ran out"};
+          LR_CUDA(cudaEventRecord(ev[4], s));
+          LR_CUDA(cudaEventSynchronize(ev[4]));
+          float a = 0, c = 0;
+          cudaEventElapsedTime(&a, ev[2], ev[3]);
+          cudaEventElapsedTime(&c, ev[3], ev[4]);
+          t[2] += a;
+          t[3] += c;
+          h.release(h.d_chi_qw);
+          h.release(h.work);
+          h.chi0_done = false;   // chi0(q, i omega) is gone: ec needs a new chi0
+        }
+      });
       LR_CUDA(cudaStreamSynchronize(s));
       cudaEventElapsedTime(&t[0], ev[0], ev[1]);
       cudaEventElapsedTime(&t[1], ev[1], ev_chi0);

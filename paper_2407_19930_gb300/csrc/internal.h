@@ -114,6 +114,9 @@ struct Handle {
   int ec_S = -1;    // ln det GEMMs: same encoding
   // FP64 mode: the stored G and the packed C are those of NAOs rescaled by 2^-ao_e[i] (k_green.cu); empty: as passed
   std::vector<int> ao_e;
+  // an allocation failed with digit planes in use: the stages up to chi0, or the ln det, take the route of least
+  // memory from then on (FP64 mode: the FP64 pipes; else the O assembly on the FP32 pipes).  set_structure resets both
+  bool lean_chi0 = false, lean_ec = false;
   bool freq_f32 = false;   // tau -> omega and R -> q transforms in FP32 (LIBRPA_SPLIT_FAST)
   cudaStream_t stream = nullptr;
   bool own_stream = false;
@@ -272,9 +275,36 @@ size_t ec_work_bytes(const Handle &h);
 // checks before the chi0 stage (inputs complete, one Fermi level) and the grid from the KS
 // spectrum when none was set; returns LIBRPA_OK or an error code with h.last_error set
 int chi0_prepare(Handle &h);
+// lean: with the routes of least memory (Handle::lean_chi0)
+size_t estimate_device_bytes(Handle &h, bool lean = false);
+// releases the workspaces and the digit planes of C (rebuilt by the next chi0_plan)
+void drop_scratch(Handle &h);
+// f(), and when device memory runs out in it, once more without scratch held over and on the routes of least memory
+template <class F>
+void with_memory(const std::vector<Handle *> &hs, bool Handle::*lean, F &&f) {
+  try {
+    f();
+    return;
+  } catch (const Error &e) {
+    bool tried = true;
+    for (Handle *h : hs) tried = tried && h->*lean;
+    if (e.code != LIBRPA_E_NOMEM || tried) throw;
+  }
+  std::vector<char> was;
+  for (Handle *h : hs) {
+    was.push_back(h->*lean);
+    h->*lean = true;
+    drop_scratch(*h);
+  }
+  try {
+    f();
+  } catch (...) {
+    for (size_t i = 0; i < hs.size(); ++i) hs[i]->*lean = was[i];
+    throw;
+  }
+}
 void materialize(Handle &h);
 void release_device(Handle &h);
-size_t estimate_device_bytes(Handle &h);
 
 // generic batched complex FP64 GEMM (k_zgemm.cu), used by K1 and K5
 struct ZGemm {

@@ -565,7 +565,7 @@ void chi0_shape(const Handle &h, Chi0Plan &P) {
   P.cpnx_rows = P.cpnx_off[nat];
   // the FP64 mode: 8 digit planes, but for the smallest requests the FP64 pipes (see kWideMinFlops)
   const double total = fl * h.ntau * (double)chi0_r_list(h.mesh).size();
-  P.tc_S = h.chi0_S >= 0 ? h.chi0_S : total >= kWideMinFlops ? oz::S_WIDE : -1;
+  P.tc_S = h.chi0_S >= 0 ? h.chi0_S : total >= kWideMinFlops && !h.lean_chi0 ? oz::S_WIDE : -1;
 }
 
 // Digit planes of the O assembly on the tensor cores: 5 (~39 bits) for the FP64-accurate mode, 3 (~23 bits, as
@@ -573,7 +573,7 @@ void chi0_shape(const Handle &h, Chi0Plan &P) {
 int oasm_planes(const Handle &h, const Chi0Plan &P) {
   for (int n : h.n_ao)
     if (n > oasm::kMaxAo) return 0;
-  if (P.tc_S < 0) return 0;
+  if (P.tc_S < 0 || h.lean_chi0) return 0;
   return P.tc_S == oz::S_WIDE ? oz::S_WIDE : P.tc_S == 4 || P.tc_S == 5 ? 5 : 3;
 }
 

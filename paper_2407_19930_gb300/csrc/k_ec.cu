@@ -755,7 +755,7 @@ void potrf_batched_r(Handle &h, double *const *d_mats, const std::vector<double 
 // digit planes of the ln det GEMMs: those of the mode, and 8 in the FP64 mode for matrices of order
 // kWideMinN or more (-1: the FP64 pipes)
 constexpr int kWideMinN = 96;
-int ec_planes(const Handle &h) { return h.ec_S >= 0 ? h.ec_S : h.naux >= kWideMinN ? oz::S_WIDE : -1; }
+int ec_planes(const Handle &h) { return h.ec_S >= 0 ? h.ec_S : h.naux >= kWideMinN && !h.lean_ec ? oz::S_WIDE : -1; }
 
 size_t al256(size_t b) { return (b + 255) / 256 * 256; }
 

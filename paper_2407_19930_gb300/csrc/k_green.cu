@@ -22,7 +22,7 @@ namespace {
 // digit planes of the G build: 5 in the tensor-core modes (FP64-accurate products), 8 in the FP64 mode
 // from kWideMinAo NAOs on (-1: the FP64 pipes)
 constexpr int kWideMinAo = 64;
-int green_planes(const Handle &h) { return h.chi0_S >= 0 ? 5 : h.nao >= kWideMinAo ? oz::S_WIDE : -1; }
+int green_planes(const Handle &h) { return h.chi0_S >= 0 ? 5 : h.nao >= kWideMinAo && !h.lean_chi0 ? oz::S_WIDE : -1; }
 
 // Equilibration of the NAOs for the FP64 mode's digit planes, which hold an element to 2^-63 of its row's largest: in a
 // product over NAOs a row of C grows with the norms of its columns where a row of G falls, so a spread of 2^12 among

@@ -271,6 +271,7 @@ int librpa_gpu_server_submit(librpa_gpu_server_t s, librpa_gpu_t req, long long 
   size_t est = 0;
   int rc = librpa_gpu_estimate_bytes(req, &est);
   if (rc != LIBRPA_OK) return rc;
+  if (est > s->budget) est = estimate_device_bytes(*req, true);   // what it falls back to within that budget
   std::unique_ptr<Ticket> t(new Ticket());
   t->h = req;
   t->est = est;
