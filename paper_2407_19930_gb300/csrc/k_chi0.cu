@@ -1286,13 +1286,15 @@ void fp64_final(Handle &h, const std::vector<Point> &pts, const Fp64Ws &w, std::
 }
 
 // Workspace of the tensor-core route for a batch of npb points: FP64 N, X, O and the digit planes
-// of Bg, Ag and O (bounded by 2 GiB, at least one point).
+// of Bg, Ag and O (bounded by cap bytes, at least one point).
 struct TcWs {
   long long npb;
   size_t b_n, b_x, b_o, b_bg, b_ag, b_od, b_nd = 0, b_xd = 0, total;   // nd, xd: O assembly on the tensor cores
 };
 
-TcWs tc_ws(const Handle &h, const Chi0Plan &P) {
+constexpr long long kTcCap = 2LL << 30;   // (1 GiB, as on the FP64 pipes: a spin-polarised cell of 4 atoms 22.9 -> 25.7 ms)
+
+TcWs tc_ws(const Handle &h, const Chi0Plan &P, long long cap = kTcCap) {
   const int nat = h.natoms, S = P.tc_S;
   const int rows_bg = 2 * nat * P.m_all, rows_ag = 2 * nat * h.nao, rows_o = nat * h.naux;
   const size_t fp = 8 * (size_t)(2 * P.n_sz + 2 * P.x_sz + P.o_sz);
@@ -1303,7 +1305,7 @@ TcWs tc_ws(const Handle &h, const Chi0Plan &P) {
   if (So) per_point += oz::sliced_bytes((int)rows_nd, 32, So) + oz::sliced_bytes((int)rows_xd, 32, So);
   const long long total_pts = (long long)h.ntau * chi0_r_list(h.mesh).size();
   TcWs w;
-  w.npb = std::min(std::max<long long>(1, (2LL << 30) / (long long)per_point), total_pts);
+  w.npb = std::min(std::max<long long>(1, cap / (long long)per_point), total_pts);
   w.b_n = 8 * (size_t)w.npb * 2 * P.n_sz;
   w.b_x = 8 * (size_t)w.npb * 2 * P.x_sz;
   w.b_o = 8 * (size_t)w.npb * P.o_sz;
@@ -1347,10 +1349,10 @@ struct TcRound {
   std::vector<oz::Entry> en, ex, ef;
 };
 
-// workspace of h for its point batches (allocated), the error flag cleared; returns the views
-TcRound tc_views(Handle &h, long long *npb) {
+// workspace of h for its point batches (allocated, of up to cap bytes), the error flag cleared; returns the views
+TcRound tc_views(Handle &h, long long *npb, long long cap = kTcCap) {
   Chi0Plan &P = h.plan;
-  const TcWs tw = tc_ws(h, P);
+  const TcWs tw = tc_ws(h, P, cap);
   *npb = tw.npb;
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
   h.ensure(h.d_chi_tau, (size_t)h.ntau * h.mesh.size() * h.naux * h.naux * sizeof(double));
@@ -1568,10 +1570,13 @@ void tc_merged(std::vector<Handle *> &hs) {
   std::vector<long long> npb(nh);
   std::vector<std::vector<Point>> pts(nh);
   int rounds = 0;
+  // the workspaces of an FP64 batch: at most 16 GiB together, as on the FP64 pipes (chi0_run_merged)
+  const long long cap =
+      h0.plan.tc_S == oz::S_WIDE ? std::min(kTcCap, std::max<long long>(1LL << 27, (16LL << 30) / (long long)nh)) : kTcCap;
   for (size_t i = 0; i < nh; ++i) {
     Handle &h = *hs[i];
     h.cur_spin = 0;
-    rs[i] = tc_views(h, &npb[i]);
+    rs[i] = tc_views(h, &npb[i], cap);
     rs[i].err = rs[0].err;   // one flag for the whole sequence: the GEMMs' and every handle's O assembly
     const std::vector<int> rl = chi0_r_list(h.mesh);
     pts[i] = make_points(h, rl, 0, (int)(h.ntau * rl.size()));

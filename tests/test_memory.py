@@ -69,3 +69,27 @@ def test_slab_within_the_least_memory(precision, budget):
     assert s["bytes_device_peak"] <= budget
     tol = 1e-8 if precision != L.LIBRPA_SPLIT else 1e-4 / 27.2 * inp.st.natoms
     assert max(abs(x - ec[0]) for x in e) < tol
+
+
+def test_fp64_batch_bounds_its_workspaces():
+    """20 structures whose workspaces would each take about 1 GiB or more: at most 16 GiB together, beside what the handles
+    keep (below 0.15 GB each)."""
+    import torch
+    inp = syn.config_mixed()
+    grid = ogrid.make_grid(10, *inp.delta_range)
+    hs, b = [], None
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    try:
+        for _ in range(20):
+            hs.append(L.librpa_gpu_create(L.librpa_gpu_default_opts()))
+            L.set_inputs(hs[-1], inp, grid)
+        b = L.librpa_gpu_batch_create(hs)
+        ec = L.librpa_gpu_batch_run(b)
+        used = free - torch.cuda.mem_get_info()[0]
+    finally:
+        L.librpa_gpu_batch_destroy(b)
+        for h in hs:
+            L.librpa_gpu_destroy(h)
+    assert np.ptp(ec) <= 1e-12 * abs(ec[0])
+    assert used < (16 << 30) + 20 * 0.15e9
