@@ -396,20 +396,23 @@ __global__ void k_real_part(const double2 *src, int n, const int *eq, double *ds
 // scaled over 2^30: ln det off by 4e-12, over 2^40 by 1e-8, against 1e-15 in FP64).  The integrand does not change under
 // V -> D V D, chi0 -> D^-1 chi0 D^-1, so each V(q) is taken with D_i = 2^eq[i] that brings its diagonal into [1, 4):
 // powers of two, exact, and L^H chi0 L is the same matrix.
-__global__ void k_equil_expo(const double2 *const *V, int n, int *eq) {   // eq[q][i]
+// V: all matrices; the b-th taken is V[ql[b]].  eq[b][i]
+__global__ void k_equil_expo(const double2 *V, const int *ql, int n, int *eq) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const double v = V[blockIdx.y][(size_t)i * n + i].x;
+  const double v = V[((size_t)ql[blockIdx.y] * n + i) * n + i].x;
   const int ex = biased_exp(v);
   eq[(size_t)blockIdx.y * n + i] = v > 0.0 && ex > 0 && ex < 2047 ? -((ex - 1023) >> 1) : 0;
 }
-__global__ void k_equil_scale(double2 *const *V, int n, const int *eq) {   // a row per CTA
-  double2 *row = V[blockIdx.y] + (size_t)blockIdx.x * n;
+__global__ void k_equil_copy(const double2 *V, const int *ql, int n, const int *eq, double2 *out) {   // a row per CTA
+  const double2 *src = V + ((size_t)ql[blockIdx.y] * n + blockIdx.x) * n;
+  double2 *dst = out + ((size_t)blockIdx.y * n + blockIdx.x) * n;
   eq += (size_t)blockIdx.y * n;
   const int ei = eq[blockIdx.x];
   for (int j = threadIdx.x; j < n; j += blockDim.x) {
+    const double2 v = src[j];
     const int e = ei + eq[j];
-    if (e) row[j] = make_double2(scale_pow2(row[j].x, e), scale_pow2(row[j].y, e));
+    dst[j] = make_double2(scale_pow2(v.x, e), scale_pow2(v.y, e));
   }
 }
 
@@ -806,7 +809,7 @@ EcLayout ec_layout(const Handle &h) {
     l.o_inv = take((size_t)bmax * NB * NB * sizeof(double2));
     l.o_pi = take(std::max(oz::sliced_bytes(bmax * NB, 2 * NB, S), oz::sliced_bytes(bmax * NB, NB, oz::S_WIDE)));
   }
-  if (S == oz::S_WIDE) l.o_eq = take((size_t)nq * n * 4);
+  if (S == oz::S_WIDE) l.o_eq = take((size_t)nq * (n + 1) * 4);
   l.total = off;
   return l;
 }
@@ -896,18 +899,20 @@ int ec_run(Handle &h, double *ec, double *ec_q, double *ec_w) {
   // Cholesky of every V(q) computed, packed in qlist order (the batched factorisation needs a
   // uniform stride)
   std::vector<double2 *> lp(nql);
+  int *eq = S == oz::S_WIDE ? (int *)(w + lay.o_eq) : nullptr;   // [qlist][n], then the qlist
   for (int i = 0; i < nql; ++i) {
     lp[i] = Lq + (size_t)i * n2;
-    LR_CUDA(cudaMemcpyAsync(lp[i], (const char *)h.d_vq.p + (size_t)qlist[i] * mat, mat, cudaMemcpyDeviceToDevice, s));
+    if (!eq) LR_CUDA(cudaMemcpyAsync(lp[i], (const char *)h.d_vq.p + (size_t)qlist[i] * mat, mat, cudaMemcpyDeviceToDevice, s));
   }
-  LR_CUDA(cudaMemcpyAsync(ptrs, lp.data(), nql * 8, cudaMemcpyHostToDevice, s));
-  int *eq = S == oz::S_WIDE ? (int *)(w + lay.o_eq) : nullptr;   // [qlist][n]
   if (eq) {
-    k_equil_expo<<<dim3((unsigned)((n + 255) / 256), (unsigned)nql), 256, 0, s>>>(ptrs, n, eq);
-    k_equil_scale<<<dim3((unsigned)n, (unsigned)nql), 256, 0, s>>>(ptrs, n, eq);
+    int *ql = eq + (size_t)nq * n;
+    LR_CUDA(cudaMemcpyAsync(ql, qlist.data(), nql * 4, cudaMemcpyHostToDevice, s));
+    k_equil_expo<<<dim3((unsigned)((n + 255) / 256), (unsigned)nql), 256, 0, s>>>((const double2 *)h.d_vq.p, ql, n, eq);
+    k_equil_copy<<<dim3((unsigned)n, (unsigned)nql), 256, 0, s>>>((const double2 *)h.d_vq.p, ql, n, eq, Lq);
     launch_counter() += 2;
     LR_CUDA(cudaGetLastError());
   }
+  LR_CUDA(cudaMemcpyAsync(ptrs, lp.data(), nql * 8, cudaMemcpyHostToDevice, s));
   auto eq_of = [&](int qi) { return eq ? eq + (size_t)qi * n : nullptr; };
   potrf_batched(h, ptrs, lp, n, n, lndet_v, info, tc);
   {

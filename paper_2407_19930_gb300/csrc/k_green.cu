@@ -43,16 +43,17 @@ __global__ void k_ao_norm(const double2 *__restrict__ wfc, long long rows, int n
   atomicMax(mx + i, m);
 }
 
-std::vector<int> ao_exponents(const std::vector<int> &mx) {
+std::vector<int> ao_exponents(const int *mx, int nao) {
   int lo = 2047, hi = 0;
-  for (int m : mx) {
+  for (int i = 0; i < nao; ++i) {
+    const int m = mx[i];
     if (m == 2047) return {};   // an infinity or a NaN
     if (m > 0) lo = std::min(lo, m);
     hi = std::max(hi, m);
   }
   if (hi - lo <= kAoSpread) return {};
   std::vector<int> e;
-  for (int m : mx) e.push_back(m > 0 ? std::max(m - hi, -400) : 0);
+  for (int i = 0; i < nao; ++i) e.push_back(mx[i] > 0 ? std::max(mx[i] - hi, -400) : 0);
   return e;
 }
 
@@ -203,7 +204,7 @@ size_t green_work_bytes(const Handle &h) {
   const size_t nk = h.mesh.size(), nR = nk, nb = h.nao, n2 = (size_t)h.nao * h.nao;
   const size_t b_e = nk * nb * 8, b_w = 2 * b_e, b_p = 2 * nk * n2 * 16, b_t = nk * nR * 16;
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-  size_t b = al(b_w) + al(b_p) + al(b_t) + al(nR * sizeof(int2)) + al(h.nao * sizeof(int)) + 256;
+  size_t b = al(b_w) + al(b_p) + al(b_t) + al(nR * sizeof(int2)) + al(16 + h.nao * sizeof(int));
   const int S = green_planes(h);
   if (S >= 0)   // digit planes: Y and the digit planes of both GEMM roles
     b += al(b_p) + oz::sliced_bytes((int)(2 * nk * 2 * h.nao), (int)(2 * nb), S) +
@@ -222,12 +223,11 @@ double green_build(Handle &h) {
                b_t = (size_t)nk * nR * 16;
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
   const size_t b_rl = (size_t)nR * sizeof(int2), b_ao = (size_t)nao * sizeof(int);
-  const size_t o_w = 0, o_p = o_w + al(b_w), o_t = o_p + al(b_p), o_rl = o_t + al(b_t), o_ao = o_rl + al(b_rl),
-               o_m = o_ao + al(b_ao);
+  const size_t o_w = 0, o_p = o_w + al(b_w), o_t = o_p + al(b_p), o_rl = o_t + al(b_t), o_m = o_rl + al(b_rl);
   // digit planes: P^g_k = Y^T conj(Y) as one batched digit-plane GEMM per tau (FP64-accurate)
   const int S = green_planes(h);
   const bool tc = S >= 0;
-  const size_t o_y = o_m + 256, o_sa = o_y + al(b_p),
+  const size_t o_y = o_m + al(16 + b_ao), o_sa = o_y + al(b_p),
                o_sb = o_sa + oz::sliced_bytes(2 * nk * 2 * nao, 2 * nb, S),
                o_err = o_sb + oz::sliced_bytes(2 * nk * nao, 2 * nb, S);
   h.ensure(h.work, green_work_bytes(h));
@@ -266,17 +266,15 @@ double green_build(Handle &h) {
   int2 *d_rl = (int2 *)(wk + o_rl);
   LR_CUDA(cudaMemcpyAsync(d_rl, rl.data(), rl.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
   LR_CUDA(cudaStreamSynchronize(s));   // tw and rl are host temporaries
-  LR_CUDA(cudaMemsetAsync(d_max, 0, 16, s));
-  int *d_ao = (int *)(wk + o_ao);
-  std::vector<int> ao_mx(h.chi0_S < 0 ? nao : 0);
-  if (!ao_mx.empty()) {
+  LR_CUDA(cudaMemsetAsync(d_max, 0, 16 + b_ao, s));
+  int *d_ao = (int *)(d_max + 2);   // behind the two maxima: one copy brings both
+  const bool equil = h.chi0_S < 0;
+  if (equil) {
     const long long rows = (long long)h.nspins * nk * nb;
-    LR_CUDA(cudaMemsetAsync(d_ao, 0, b_ao, s));
     k_ao_norm<<<dim3((unsigned)((nao + 31) / 32), (unsigned)std::min<long long>(64, (rows + 31) / 32)), dim3(32, 8), 0, s>>>(
         d_wfc0, rows, nao, d_ao);
     ++launch_counter();
     LR_CUDA(cudaGetLastError());
-    LR_CUDA(cudaMemcpyAsync(ao_mx.data(), d_ao, b_ao, cudaMemcpyDeviceToHost, s));
   }
   const size_t g_stride = (size_t)ntau * nR * n2;
   for (int sp = 0; sp < h.nspins; ++sp) {   // one spin channel at a time, own KS data, own G
@@ -346,14 +344,14 @@ double green_build(Handle &h) {
       phase_sum(it);
     }
   }
-  unsigned long long mx[2];
+  std::vector<char> mx(16 + (equil ? b_ao : 0));
   int e_host = 0;
-  LR_CUDA(cudaMemcpyAsync(mx, d_max, 16, cudaMemcpyDeviceToHost, s));
+  LR_CUDA(cudaMemcpyAsync(mx.data(), d_max, mx.size(), cudaMemcpyDeviceToHost, s));
   if (tc) LR_CUDA(cudaMemcpyAsync(&e_host, d_err, 4, cudaMemcpyDeviceToHost, s));
   LR_CUDA(cudaStreamSynchronize(s));
   if (e_host) throw Error{LIBRPA_E_TIMEOUT, "Green's function: a bounded wait in the tensor-core GEMM ran out"};
   green_screen(h);   // after the imaginary-part check's maxima: they describe the unscreened G
-  const std::vector<int> e = ao_exponents(ao_mx);
+  const std::vector<int> e = equil ? ao_exponents((const int *)(mx.data() + 16), nao) : std::vector<int>();
   if (e != h.ao_e) {   // C is packed in the same units
     h.ao_e = e;
     h.lri_dirty = true;
@@ -365,8 +363,8 @@ double green_build(Handle &h) {
     LR_CUDA(cudaGetLastError());
   }
   double mre, mim;
-  std::memcpy(&mre, &mx[0], 8);
-  std::memcpy(&mim, &mx[1], 8);
+  std::memcpy(&mre, mx.data(), 8);
+  std::memcpy(&mim, mx.data() + 8, 8);
   return mre > 0 ? mim / mre : mim;
 }
 

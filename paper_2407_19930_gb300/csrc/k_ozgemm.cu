@@ -49,16 +49,7 @@ struct CplxSrc {
   long long ld, bstride;
   int rows_pb, op;
   bool as_a;
-  const int *eq;
   __device__ double2 opget(const double2 *q, int i, int k) const {
-    double2 z = opget_plain(q, i, k);
-    if (eq) {
-      const int e = -(eq[i] + eq[k]);
-      z = make_double2(scale_pow2(z.x, e), scale_pow2(z.y, e));
-    }
-    return z;
-  }
-  __device__ double2 opget_plain(const double2 *q, int i, int k) const {
     if (op == OP_N) return q[(long long)i * ld + k];
     if (op == OP_C) {
       const double2 z = q[(long long)i * ld + k];
@@ -79,6 +70,15 @@ struct CplxSrc {
     }
     const double2 z = opget(q, k, rr);
     return cp ? z.y : z.x;
+  }
+};
+
+// A'-form rows (as_a) of Z with element (i, k) times 2^-(eq[i] + eq[k])
+struct CplxEqSrc {
+  CplxSrc z;
+  const int *eq;
+  __device__ double get(int r, int kk) const {
+    return scale_pow2(z.get(r, kk), -(eq[(r % z.rows_pb) >> 1] + eq[kk >> 1]));
   }
 };
 
@@ -1064,7 +1064,12 @@ void split_real(const double *src, long long ld, bool trans, int rows, int K, in
 void split_complex(const double2 *src, long long ld, Op op, bool as_a, int n_out, int n_k, int batch,
                    long long batch_stride, Sliced &out, cudaStream_t s, const int *eq) {
   const int rows_pb = as_a ? 2 * n_out : n_out;
-  CplxSrc c{src, ld, batch_stride, rows_pb, (int)op, as_a, eq};
+  CplxSrc c{src, ld, batch_stride, rows_pb, (int)op, as_a};
+  if (eq) {
+    if (!as_a) throw Error{LIBRPA_E_ARG, "split_complex: scaled elements in the B' form"};
+    split_any(CplxEqSrc{c, eq}, rows_pb * batch, 2 * n_k, 0, out, s);
+    return;
+  }
   split_any(c, rows_pb * batch, 2 * n_k, 0, out, s);
 }
 

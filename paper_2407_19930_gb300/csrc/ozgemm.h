@@ -60,7 +60,7 @@ void split_real(const double *src, long long ld, bool trans, int rows, int K, in
 //  complex: op(Z)[i][k] with op in {N, T, H, C}; Z row-major interleaved (re, im), leading dim ld.
 //   as_a = true  -> stacked real matrix A'[2i + c][2k + c'] = [[Re, -Im], [Im, Re]] of op(Z)[i][k]
 //   as_a = false -> B'^T[j][2k + c'] = component c' of op(Z)[k][j]
-//  eq (device, NULL: none): element (i, k) of Z is taken times 2^-(eq[i] + eq[k])
+//  eq (device, as_a only; NULL: none): element (i, k) of Z is taken times 2^-(eq[i] + eq[k])
 void split_complex(const double2 *src, long long ld, Op op, bool as_a, int n_out, int n_k, int batch,
                    long long batch_stride, Sliced &out, cudaStream_t s, const int *eq = nullptr);
 //  gathered Green's-function blocks of the chi0 contraction (see k_chi0.cu for the tables):

@@ -20,7 +20,7 @@ __device__ __forceinline__ double scale_pow2(double v, int e) {
   const int ex = biased_exp(v);
   if (ex > 0 && ex < 2047 && (unsigned)(ex + e - 1) < 2046u)
     return __longlong_as_double(__double_as_longlong(v) + ((long long)e << 52));
-  return scalbn(v, e);
+  return (__double_as_longlong(v) << 1) == 0 ? v : scalbn(v, e);
 }
 
 // balanced base-256 digits of x = v 2^-E (|x| < 1): x ~ sum_s d_s 2^{-7-8(s-1)}, |d_s| <= 128, as FP32 integers.
