@@ -272,6 +272,8 @@ int chi0_prepare(Handle &h) {
     h.ntau = n;
     h.have_grid = true;
   }
+  // a new grid can change the route of the contraction
+  if (!h.lri_dirty && chi0_planes(h, h.plan) != h.plan.tc_S) h.lri_dirty = true;
   return LIBRPA_OK;
 }
 

@@ -232,6 +232,8 @@ void chi0_plan(Handle &h);
 void chi0_run(Handle &h, double *ms_gemm);
 // host part of chi0_plan: neighbour lists, packed-column sizes, workspace offsets, flops
 void chi0_shape(const Handle &h, Chi0Plan &P);
+// operand form of the contraction's GEMMs for the plan's shape and the handle's grid (Chi0Plan::tc_S)
+int chi0_planes(const Handle &h, const Chi0Plan &P);
 // device bytes the chi0 stage holds for this shape (packed C and its digit planes, chi0(R, tau),
 // batch workspace, tables)
 size_t chi0_device_bytes(const Handle &h, const Chi0Plan &P);

@@ -563,9 +563,13 @@ void chi0_shape(const Handle &h, Chi0Plan &P) {
     P.cpnx_off[a + 1] = P.cpnx_off[a] + h.n_aux[a] * h.n_ao[a];
   }
   P.cpnx_rows = P.cpnx_off[nat];
-  // the FP64 mode: 8 digit planes, but for the smallest requests the FP64 pipes (see kWideMinFlops)
-  const double total = fl * h.ntau * (double)chi0_r_list(h.mesh).size();
-  P.tc_S = h.chi0_S >= 0 ? h.chi0_S : total >= kWideMinFlops && !h.lean_chi0 ? oz::S_WIDE : -1;
+  P.tc_S = chi0_planes(h, P);
+}
+
+// the FP64 mode: 8 digit planes, but for the smallest requests the FP64 pipes (see kWideMinFlops)
+int chi0_planes(const Handle &h, const Chi0Plan &P) {
+  const double total = P.flop_per_point * h.ntau * (double)chi0_r_list(h.mesh).size();
+  return h.chi0_S >= 0 ? h.chi0_S : total >= kWideMinFlops && !h.lean_chi0 ? oz::S_WIDE : -1;
 }
 
 // Digit planes of the O assembly on the tensor cores: 5 (~39 bits) for the FP64-accurate mode, 3 (~23 bits, as
