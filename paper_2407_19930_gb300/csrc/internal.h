@@ -98,6 +98,7 @@ struct Chi0Plan {
   int oasm_max_tiles = 0;
   DevBuf t_lamf, t_unif;   // the columns of d_lam and d_uni with folded, packed lattice vectors (GatherSrc)
   bool folded = false;
+  bool c_nonfinite = false;   // C holds an infinity or a NaN
   std::vector<DevBuf *> all() {
     return {&d_lam, &d_uni, &d_kap, &t_n_ao, &t_n_aux, &t_ao_off, &t_aux_off, &t_m, &t_lam_off, &t_kap_off,
             &t_bg_off, &t_ag_off, &t_n_off, &t_x_off, &t_o_off, &t_pts, &ws, &gargs1, &gargs2,
@@ -114,6 +115,7 @@ struct Handle {
   int ec_S = -1;    // ln det GEMMs: same encoding
   // FP64 mode: the stored G and the packed C are those of NAOs rescaled by 2^-ao_e[i] (k_green.cu); empty: as passed
   std::vector<int> ao_e;
+  bool g_nonfinite = false;   // the stored G holds an infinity or a NaN
   // an allocation failed with digit planes in use: the stages up to chi0, or the ln det, take the route of least
   // memory from then on (FP64 mode: the FP64 pipes; else the O assembly on the FP32 pipes).  set_structure resets both
   bool lean_chi0 = false, lean_ec = false;

@@ -356,6 +356,14 @@ __global__ void __launch_bounds__(256, 2) k_oassemble(OArgs a, int NL, const int
   }
 }
 
+// *flag = 1 when v holds an infinity or a NaN
+__global__ void k_nonfinite(const double *v, size_t n, int *flag) {
+  bool bad = false;
+  for (size_t x = (size_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (size_t)gridDim.x * blockDim.x)
+    bad = bad || (__double2hiint(v[x]) & 0x7FF00000) == 0x7FF00000;
+  if (bad) *flag = 1;
+}
+
 template <class T>
 T *upload(Handle &h, DevBuf &b, const std::vector<T> &v) {
   h.ensure(b, std::max<size_t>(1, v.size()) * sizeof(T));
@@ -715,6 +723,18 @@ void chi0_plan(Handle &h) {
     }
     LR_CUDA(cudaStreamSynchronize(h.stream));
   }
+  P.c_nonfinite = false;
+  if (oasm_planes(h, P) > 0) {
+    h.ensure(P.t_oe_k, sizeof(int));   // (scratch here)
+    int *flag = (int *)P.t_oe_k.p, bad = 0;
+    LR_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), h.stream));
+    k_nonfinite<<<608, 256, 0, h.stream>>>((const double *)h.d_cpack.p, (size_t)P.cp_total, flag);
+    ++launch_counter();
+    LR_CUDA(cudaGetLastError());
+    LR_CUDA(cudaMemcpyAsync(&bad, flag, sizeof(int), cudaMemcpyDeviceToHost, h.stream));
+    LR_CUDA(cudaStreamSynchronize(h.stream));
+    P.c_nonfinite = bad != 0;
+  }
 }
 
 namespace {
@@ -804,7 +824,7 @@ bool run_oassemble(Handle &h, const Point *dpts, int np, double *Nw, double *Xw,
     t.aux_atom = (const int *)P.t_aux_atom.p;
     t.ao_row = (const int *)P.t_ao_row.p;
     t.max_tiles = P.oasm_max_tiles;
-    oasm::run(otc, oa, t, np, *tc->nd, *tc->xd, tc->rexp, tc->err, Handle::stall_ns(h.stalls_oasm),
+    oasm::run(otc, oa, t, np, *tc->nd, *tc->xd, tc->rexp, tc->err, h.g_nonfinite || P.c_nonfinite, Handle::stall_ns(h.stalls_oasm),
               h.stream);
     return true;
   }

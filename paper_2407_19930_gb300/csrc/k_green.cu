@@ -91,7 +91,7 @@ __global__ void k_weights(const double *eig, const double *occ, double mu, doubl
 // One thread per (g, i, j) and, by blockIdx.y, per pair R, -R of the list rl (R <= -R: {R, -R}): with t = c + i s the
 // two cells share the sums of p.x c, p.y s, p.x s and p.y c, half the FP64 flops of a cell at a time.
 // FP64-bound: 4 fused multiply-adds per k and pair (graphene slab, 16 k: 976 -> ~500 us a tau).  The largest
-// |Re| and |Im| go through the warp, one atomic each.
+// |Re| and |Im| go through the warp, one atomic each; maxabs[2] becomes 1 when G holds an infinity or a NaN.
 __global__ void __launch_bounds__(256) k_phase_sum(const double2 *__restrict__ P, const double2 *__restrict__ twiddle,
                                                    const int2 *__restrict__ rl, int nk, int nR, int nao, double inv_nk,
                                                    double *__restrict__ G, size_t g_stride, unsigned long long *maxabs) {
@@ -99,6 +99,7 @@ __global__ void __launch_bounds__(256) k_phase_sum(const double2 *__restrict__ P
   const size_t x = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int2 R = rl[blockIdx.y];
   double mre = 0.0, mim = 0.0;
+  bool bad = false;
   if (x < 2 * n2) {
     const int g = (int)(x / n2);
     const size_t ij = x % n2;
@@ -121,11 +122,13 @@ __global__ void __launch_bounds__(256) k_phase_sum(const double2 *__restrict__ P
     double *out = G + (size_t)g * g_stride + ij;
     const double re = (xc - ys) * inv_nk, im = (xs + yc) * inv_nk;
     out[(size_t)R.x * n2] = re;
+    bad = (__double2hiint(re) & 0x7FF00000) == 0x7FF00000;
     mre = fabs(re);
     mim = fabs(im);
     if (R.y != R.x) {
       const double re2 = (xc + ys) * inv_nk, im2 = (yc - xs) * inv_nk;
       out[(size_t)R.y * n2] = re2;
+      bad = bad || (__double2hiint(re2) & 0x7FF00000) == 0x7FF00000;
       mre = fmax(mre, fabs(re2));
       mim = fmax(mim, fabs(im2));
     }
@@ -135,6 +138,7 @@ __global__ void __launch_bounds__(256) k_phase_sum(const double2 *__restrict__ P
     mre = fmax(mre, __shfl_xor_sync(0xffffffffu, mre, o));
     mim = fmax(mim, __shfl_xor_sync(0xffffffffu, mim, o));
   }
+  if (bad) maxabs[2] = 1;
   if ((threadIdx.x & 31) == 0) {   // non-negative doubles order like their bit patterns
     atomicMax(&maxabs[0], __double_as_longlong(mre));
     atomicMax(&maxabs[1], __double_as_longlong(mim));
@@ -204,7 +208,7 @@ size_t green_work_bytes(const Handle &h) {
   const size_t nk = h.mesh.size(), nR = nk, nb = h.nao, n2 = (size_t)h.nao * h.nao;
   const size_t b_e = nk * nb * 8, b_w = 2 * b_e, b_p = 2 * nk * n2 * 16, b_t = nk * nR * 16;
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-  size_t b = al(b_w) + al(b_p) + al(b_t) + al(nR * sizeof(int2)) + al(16 + h.nao * sizeof(int));
+  size_t b = al(b_w) + al(b_p) + al(b_t) + al(nR * sizeof(int2)) + al(24 + h.nao * sizeof(int));
   const int S = green_planes(h);
   if (S >= 0)   // digit planes: Y and the digit planes of both GEMM roles
     b += al(b_p) + oz::sliced_bytes((int)(2 * nk * 2 * h.nao), (int)(2 * nb), S) +
@@ -227,7 +231,7 @@ double green_build(Handle &h) {
   // digit planes: P^g_k = Y^T conj(Y) as one batched digit-plane GEMM per tau (FP64-accurate)
   const int S = green_planes(h);
   const bool tc = S >= 0;
-  const size_t o_y = o_m + al(16 + b_ao), o_sa = o_y + al(b_p),
+  const size_t o_y = o_m + al(24 + b_ao), o_sa = o_y + al(b_p),
                o_sb = o_sa + oz::sliced_bytes(2 * nk * 2 * nao, 2 * nb, S),
                o_err = o_sb + oz::sliced_bytes(2 * nk * nao, 2 * nb, S);
   h.ensure(h.work, green_work_bytes(h));
@@ -266,8 +270,8 @@ double green_build(Handle &h) {
   int2 *d_rl = (int2 *)(wk + o_rl);
   LR_CUDA(cudaMemcpyAsync(d_rl, rl.data(), rl.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
   LR_CUDA(cudaStreamSynchronize(s));   // tw and rl are host temporaries
-  LR_CUDA(cudaMemsetAsync(d_max, 0, 16 + b_ao, s));
-  int *d_ao = (int *)(d_max + 2);   // behind the two maxima: one copy brings both
+  LR_CUDA(cudaMemsetAsync(d_max, 0, 24 + b_ao, s));
+  int *d_ao = (int *)(d_max + 3);   // behind the maxima and the flag of k_phase_sum: one copy brings them all
   const bool equil = h.chi0_S < 0;
   if (equil) {
     const long long rows = (long long)h.nspins * nk * nb;
@@ -344,14 +348,14 @@ double green_build(Handle &h) {
       phase_sum(it);
     }
   }
-  std::vector<char> mx(16 + (equil ? b_ao : 0));
+  std::vector<char> mx(24 + (equil ? b_ao : 0));
   int e_host = 0;
   LR_CUDA(cudaMemcpyAsync(mx.data(), d_max, mx.size(), cudaMemcpyDeviceToHost, s));
   if (tc) LR_CUDA(cudaMemcpyAsync(&e_host, d_err, 4, cudaMemcpyDeviceToHost, s));
   LR_CUDA(cudaStreamSynchronize(s));
   if (e_host) throw Error{LIBRPA_E_TIMEOUT, "Green's function: a bounded wait in the tensor-core GEMM ran out"};
   green_screen(h);   // after the imaginary-part check's maxima: they describe the unscreened G
-  const std::vector<int> e = equil ? ao_exponents((const int *)(mx.data() + 16), nao) : std::vector<int>();
+  const std::vector<int> e = equil ? ao_exponents((const int *)(mx.data() + 24), nao) : std::vector<int>();
   if (e != h.ao_e) {   // C is packed in the same units
     h.ao_e = e;
     h.lri_dirty = true;
@@ -365,6 +369,7 @@ double green_build(Handle &h) {
   double mre, mim;
   std::memcpy(&mre, mx.data(), 8);
   std::memcpy(&mim, mx.data() + 8, 8);
+  h.g_nonfinite = mx[16] != 0;
   return mre > 0 ? mim / mre : mim;
 }
 

@@ -61,8 +61,9 @@ __device__ __forceinline__ void tc_digits(float h, float l, float sc7, float sc1
 
 // The element type of the operands: (hi, lo) FP32 pairs with up to 5 planes (N and X arrive so from their GEMMs, G as
 // FP64 turned into pairs; the low part joins the digits after the second, error below 2^-39 of the row
-// maximum), FP64 numbers with 8 planes.
-template <int S>
+// maximum), FP64 numbers with 8 planes.  NANS: G or C holds an infinity or a NaN (known on the host); the exponent of a row
+// with one is then 1025, as it always is with 8 planes (in every kernel this test costs 2% of the slab's SPLIT energy).
+template <int S, bool NANS>
 struct Elem {
   using T = float2;
   __device__ static T zero() { return make_float2(0.f, 0.f); }
@@ -73,9 +74,13 @@ struct Elem {
   }
   using M = float;   // running maximum
   __device__ static M m0() { return 0.f; }
-  __device__ static M mx(M m, T v) { return fmaxf(m, fabsf(v.x)); }
-  __device__ static M both(M m, int o) { return fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o)); }
-  __device__ static int expo(M m) { return tc_expo(m); }
+  __device__ static M mx(M m, T v) { return larger(m, fabsf(v.x)); }
+  __device__ static M both(M m, int o) { return larger(m, __shfl_xor_sync(0xffffffffu, m, o)); }
+  __device__ static int expo(M m) { return NANS && !(m < __int_as_float(0x7F800000)) ? 1025 : tc_expo(m); }
+  __device__ static float larger(float a, float b) {
+    if (!NANS) return fmaxf(a, b);
+    return a != a || a > b ? a : b;   // NaN if either is
+  }
   // digits of 8 elements, 16 bytes per plane
   __device__ static void digits8(const T *v, int E, uint4 *w) {
     const float sc7 = tc_pow2(7 - E), sc15 = tc_pow2(15 - E);
@@ -88,8 +93,8 @@ struct Elem {
                         pack_bf16(d[6][s], d[7][s]));
   }
 };
-template <>
-struct Elem<oz::S_WIDE> {
+template <bool NANS>
+struct Elem<oz::S_WIDE, NANS> {
   using T = double;
   __device__ static T zero() { return 0.0; }
   __device__ static T load(const double *p) { return *p; }
@@ -115,10 +120,10 @@ struct Elem<oz::S_WIDE> {
 
 // Digit planes of N: laid out [(p, nu)][plane][union column][t], t = (g, j); row exponents [(p, nu)][union column].  Two lanes per row (16 t each), 16 consecutive
 // columns per warp; block = 128 columns of one (p, nu).
-template <int S>
+template <int S, bool NANS>
 __global__ void __launch_bounds__(256) k_split_n(OArgs a, const int *__restrict__ aux_atom, __nv_bfloat16 *dig,
                                                  int *expo) {
-  using E_ = Elem<S>;
+  using E_ = Elem<S, NANS>;
   const int p = blockIdx.x / a.naux, nug = blockIdx.x % a.naux, V = aux_atom[nug], nu = nug - a.aux_off[V];
   const int lane = threadIdx.x & 31, h = lane >> 4;
   const int col = blockIdx.y * 128 + (threadIdx.x >> 5) * 16 + (lane & 15);
@@ -151,10 +156,10 @@ __global__ void __launch_bounds__(256) k_split_n(OArgs a, const int *__restrict_
 
 // Digit planes of X: [(p, nu)][plane][16 U + i][t]; two lanes per row.  Rows i >= n_U are left as they are (the MMA
 // columns they give are not read).
-template <int S>
+template <int S, bool NANS>
 __global__ void __launch_bounds__(256) k_split_x(OArgs a, const int *__restrict__ aux_atom,
                                                  const int *__restrict__ ao_row, __nv_bfloat16 *dig, int *expo) {
-  using E_ = Elem<S>;
+  using E_ = Elem<S, NANS>;
   const int p = blockIdx.x / a.naux, nug = blockIdx.x % a.naux, V = aux_atom[nug], nu = nug - a.aux_off[V];
   const int lane = threadIdx.x & 31, h = lane >> 4;
   const int ao = blockIdx.y * 128 + (threadIdx.x >> 5) * 16 + (lane & 15);
@@ -235,11 +240,12 @@ __device__ __forceinline__ double combine(const uint32_t (&r1)[S][4], const uint
   }
 }
 
-template <int S>
+// NANS (see Elem; with 8 planes always): outputs of rows with the exponent 1025 are NaN, whatever their digits gave
+template <int S, bool NANS>
 __global__ void __launch_bounds__(kThreads, 1)
     k_oasm(OArgs a, Tables tb, const __grid_constant__ CUtensorMap nmap, const __grid_constant__ CUtensorMap xmap,
            const int *__restrict__ nexp, const int *__restrict__ xexp, int *rexp, int *err, uint64_t stall_ns) {
-  using E_ = Elem<S>;
+  using E_ = Elem<S, NANS>;
   constexpr int NST = ring(S), NSL = slots(S), SL = slot_cols(S);
   constexpr int NU = nus(S);
   constexpr uint32_t OPB = op_bytes(S), XB_ = x_bytes(S), FIXED = static_size(S), STAGE = stage_size(S);
@@ -495,7 +501,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int x = x0; x < x0 + N; ++x) {
               const int e1 = e[x] >> 16, e2 = (int)(short)e[x];
               o[x - x0] = combine<S>(r1, r2, x, e1 + f1, e2 + f2);
-              if (S == oz::S_WIDE && max(max(e1, f1), max(e2, f2)) > 1024)
+              if ((S == oz::S_WIDE || NANS) && max(max(e1, f1), max(e2, f2)) > 1024)
                 o[x - x0] = __longlong_as_double(0x7FF8000000000000ll);
             }
 #pragma unroll
@@ -533,17 +539,17 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == kEpi) tmem_dealloc(tmem, 512);
 }
 
-template <int S>
+template <int S, bool NANS = false>
 void launch(const OArgs &a, const Tables &t, int np, oz::Sliced &nd, oz::Sliced &xd, int *expo, int *err, uint64_t stall_ns,
             cudaStream_t s) {
   static_assert(smem_size(S) <= 227 * 1024, "k_oasm: shared memory");
   const unsigned rows = (unsigned)(np * a.naux);
-  k_split_n<S><<<dim3(rows, (unsigned)((a.m_all + 127) / 128)), 256, 0, s>>>(
+  k_split_n<S, NANS><<<dim3(rows, (unsigned)((a.m_all + 127) / 128)), 256, 0, s>>>(
       a, t.aux_atom, (__nv_bfloat16 *)nd.digits, nd.expo);
-  k_split_x<S><<<dim3(rows, (unsigned)((a.nao + 127) / 128)), 256, 0, s>>>(
+  k_split_x<S, NANS><<<dim3(rows, (unsigned)((a.nao + 127) / 128)), 256, 0, s>>>(
       a, t.aux_atom, t.ao_row, (__nv_bfloat16 *)xd.digits, xd.expo);
-  LR_CUDA(cudaFuncSetAttribute(k_oasm<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_size(S)));
-  k_oasm<S><<<(unsigned)t.max_tiles * (unsigned)(np * a.natoms * a.natoms), kThreads, smem_size(S), s>>>(
+  LR_CUDA(cudaFuncSetAttribute(k_oasm<S, NANS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_size(S)));
+  k_oasm<S, NANS><<<(unsigned)t.max_tiles * (unsigned)(np * a.natoms * a.natoms), kThreads, smem_size(S), s>>>(
       a, t, oz::make_map_nested(nd.digits, a.m_all, S, (int)rows, 8, nus(S)),
       oz::make_map_nested(xd.digits, a.natoms * kMaxAo, S, (int)rows, kMaxAo, nus(S)), nd.expo, xd.expo, expo, err,
       stall_ns);
@@ -554,9 +560,13 @@ void launch(const OArgs &a, const Tables &t, int np, oz::Sliced &nd, oz::Sliced 
 }  // namespace
 
 void run(int S, const OArgs &a, const Tables &t, int np, oz::Sliced &nd, oz::Sliced &xd, int *expo, int *err,
-         uint64_t stall_ns, cudaStream_t s) {
+         bool nans, uint64_t stall_ns, cudaStream_t s) {
   oz::init();
-  if (S == 3)
+  if (S == 3 && nans)
+    launch<3, true>(a, t, np, nd, xd, expo, err, stall_ns, s);
+  else if (S == 5 && nans)
+    launch<5, true>(a, t, np, nd, xd, expo, err, stall_ns, s);
+  else if (S == 3)
     launch<3>(a, t, np, nd, xd, expo, err, stall_ns, s);
   else if (S == 5)
     launch<5>(a, t, np, nd, xd, expo, err, stall_ns, s);

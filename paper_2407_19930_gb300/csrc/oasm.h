@@ -66,10 +66,10 @@ inline long long x_rows(int naux, int natoms) { return (long long)naux * natoms 
 
 // O for np points with S digit planes (3, 5 or 8): splits N and X into nd and xd, then one launch over every
 // (point, U, V, tile).  expo: row exponents of O's digit planes (rows (p, U, nu), initialised to -1022), built by
-// atomicMax.  err: set to 1 when a bounded wait ran out.  stall_ns > 0 (testing only): the failure path, as in
+// atomicMax.  err: set to 1 when a bounded wait ran out.  nans: G or C may hold an infinity or a NaN.  stall_ns > 0 (testing only): the failure path, as in
 // k_ozgemm.
 void run(int S, const OArgs &a, const Tables &t, int np, oz::Sliced &nd, oz::Sliced &xd, int *expo, int *err,
-         uint64_t stall_ns, cudaStream_t s);
+         bool nans, uint64_t stall_ns, cudaStream_t s);
 
 }  // namespace oasm
 }  // namespace librpa
