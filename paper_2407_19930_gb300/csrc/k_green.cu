@@ -123,8 +123,8 @@ __global__ void __launch_bounds__(256) k_phase_sum(const double2 *__restrict__ P
     const double re = (xc - ys) * inv_nk, im = (xs + yc) * inv_nk;
     out[(size_t)R.x * n2] = re;
     bad = (__double2hiint(re) & 0x7FF00000) == 0x7FF00000;
-    mre = fabs(re);
-    mim = fabs(im);
+    mre = fmax(0.0, fabs(re));   // (a NaN is left out, as everywhere in these maxima)
+    mim = fmax(0.0, fabs(im));
     if (R.y != R.x) {
       const double re2 = (xc + ys) * inv_nk, im2 = (yc - xs) * inv_nk;
       out[(size_t)R.y * n2] = re2;

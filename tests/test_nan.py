@@ -45,3 +45,19 @@ def test_coefficient(precision, value):
     assert not np.isfinite(tau[..., bad]).any()
     tol = {L.LIBRPA_FP64: 1e-10, L.LIBRPA_FP64_TC: 1e-10, L.LIBRPA_SPLIT: 1e-5}[precision]   # as without the NaN
     assert np.abs(tau - ref)[..., ~bad].max() < tol * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("precision", [L.LIBRPA_FP64, L.LIBRPA_FP64_TC])
+def test_orbitals_without_a_number(precision):
+    """Kohn-Sham coefficients that are all NaN give results that are NaN, not an error of the imaginary part."""
+    inp, grid = _inputs()
+    inp.wfc = np.full_like(inp.wfc, np.nan)
+    o = L.librpa_gpu_default_opts()
+    o.precision = precision
+    h = L.librpa_gpu_create(o)
+    try:
+        L.set_inputs(h, inp, grid)
+        L.librpa_gpu_chi0(h)
+        assert np.isnan(L.librpa_gpu_get_chi0_tau(h, 0, 0, inp.st.naux)).all()
+    finally:
+        L.librpa_gpu_destroy(h)
