@@ -34,7 +34,7 @@ def _sources():
 
 def _deps():
     return (_sources() + glob.glob(os.path.join(SRC, "*.h")) + glob.glob(os.path.join(INC, "*.h")) +
-            [os.path.join(HERE, "probe", "peaks.cu")])
+            PROBE_SRC)
 
 
 def up_to_date() -> bool:
@@ -78,14 +78,14 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
-PROBE_SRC = os.path.join(HERE, "probe", "peaks.cu")
+PROBE_SRC = [os.path.join(HERE, "probe", f) for f in ("peaks.cu", "rsqrt.cu")]
 PROBE_LIB = os.path.join(BUILD, "libpeaks.so")
 
 
 def _build_probe(nvcc: str) -> str:
-    """The FP64 peak probes the benchmark measures its roofline against (a library of its own,
-    outside the C ABI)."""
-    cmd = [nvcc, *ARCH, "-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-shared", PROBE_SRC, "-o", PROBE_LIB]
+    """The FP64 peak probes the benchmark measures its roofline against and the probe of the pivots' square roots
+    (a library of its own, outside the C ABI)."""
+    cmd = [nvcc, *ARCH, "-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-shared", *PROBE_SRC, "-o", PROBE_LIB]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError("compile failed: %s\n%s%s" % (" ".join(cmd), r.stdout, r.stderr))

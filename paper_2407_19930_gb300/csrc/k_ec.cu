@@ -26,6 +26,7 @@
 
 #include "internal.h"
 #include "ozgemm.h"
+#include "rsqrt.h"
 #include "tc.h"
 
 namespace librpa {
@@ -40,20 +41,6 @@ constexpr int NB = 64;
 // 8 x 8 triangle 64 threads factor, an element each, and every other product runs over many threads.
 constexpr int KB = 8;   // columns per block
 
-// 1 / sqrt(d) for a normal d > 0 in five FP64 instructions: FP32 seed r0 of the mantissa and one step of third order
-// in e = 1 - d r0^2 (r0 (1 + e / 2 + 3 e^2 / 8), error ~e^3 < 2^-60), conversions and scaling by integer instructions
-__device__ __forceinline__ double fast_rsqrt(double d) {
-  const int hi = __double2hiint(d), ex = hi >> 20;
-  if (ex < 1 || ex > 2046) return rsqrt(d);
-  const int q = (ex - 1023) & ~1;   // d 2^-q in [1, 4)
-  const double x = __hiloint2double(hi - (q << 20), __double2loint(d));
-  const float f = __int_as_float(((ex - q - 896) << 23) | ((hi & 0xFFFFF) << 3));
-  const int rb = __float_as_int(rsqrtf(f));
-  const double r0 = __hiloint2double((rb >> 3) + (896 << 20), rb << 29);
-  const double e = fma(-(x * r0), r0, 1.0);
-  const double r = fma(r0 * e, fma(0.375, e, 0.5), r0);
-  return __hiloint2double(__double2hiint(r) - ((q / 2) << 20), __double2loint(r));
-}
 __device__ __forceinline__ void bar_64() { asm volatile("bar.sync 1, 64;" ::: "memory"); }   // threads 0..63
 
 // element arithmetic: T = double2 (complex) or double
@@ -125,9 +112,7 @@ __global__ void __launch_bounds__(256) k_potrf_diag(T *const *mats, int n, int l
         const double ri = fast_rsqrt(d);
         if (k == j) {
           if (r == j) {
-            double sq = d * ri;
-            sq = fma(0.5 * ri, fma(-sq, sq, d), sq);   // sqrt(d)
-            set_re(e, sq);
+            set_re(e, sqrt_from(d, ri));
             rinv[j0 + j] = ri;
             piv[j0 + j] = d;
             if (!ok) bad = 1;
