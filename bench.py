@@ -466,16 +466,7 @@ def run_gpu(args):
     fp64_src = ("measured in this run: DMMA m8n8k4 register probe (probe/peaks.cu), SM clock median %s MHz"
                 % ((peaks_run.get("clocks") or {}).get("sm_mhz") if peaks_run else None)) if dmma else \
         "derived: %s BF16 dense burst x nominal FP64/BF16 (1.25/2250)" % src
-    # dominant kernel by device time within the step
-    kern = {"k_dgemm_nt": (s["ms_gemm_chi0"], s["flop_gemm_chi0"], s["n_gemm_chi0"], "paper_2407_19930_gb300/csrc/k_chi0.cu"),
-            "k_zgemm": (s["ms_gemm_ec"], s["flop_gemm_ec"], s["n_gemm_ec"], "paper_2407_19930_gb300/csrc/k_zgemm.cu")}
-    name = max(kern, key=lambda k: kern[k][0])
-    ms, fl, nl, srcf = kern[name]
-    achieved = fl / (ms * 1e-3) / 1e12 if ms > 0 else None
-    tr = TRAFFIC.get(name)
-    # the captured traffic is the graphene slab's (its per-launch work is the same at every k-mesh)
-    traffic = tr["bytes_per_launch"] if (tr and args.workload == "graphene" and
-                                         tr["src_sha"] == _src_sha(tr["src"], tr["begin"], tr["end"])) else None
+    fp64_note = "FP64 tensor path, %s; derived from the BF16 peak: %.3f" % (fp64_src, fp64_derived)
     step_ms = t / args.steps * 1e3 * ws / ws
     chi0_tflops = s["flop_chi0"] / (s["ms_chi0"] * 1e-3) / 1e12
     line = {
@@ -496,16 +487,11 @@ def run_gpu(args):
         "chi0_tflops": chi0_tflops,
         "stage_ms": {"green": s["ms_green"], "chi0": s["ms_chi0"], "freq": s["ms_freq"], "ec": s["ms_ec"]},
         "ec_ha": ec,
-        "roofline": {"kernel": name, "bound": "tensor", "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s",
-                     "frac": achieved / fp64_peak if achieved else None, "traffic": traffic,
-                     "peak_note": "FP64 tensor path, %s; derived from the BF16 peak: %.3f" % (fp64_src, fp64_derived),
-                     "launches": nl, "flop": fl},
+        "roofline": roofline(s, peaks, src, fp64_peak, fp64_note, args.workload == "graphene"),
         "clocks": clk,
     }
     if peaks_run:
         line["peaks_measured"] = peaks_run
-    if args.precision != "fp64":
-        line["roofline"] = tc_roofline(s, peaks, src)
     if modes:
         line["modes"] = modes
     if ws == 1 and args.serve_sample > 0:
@@ -553,6 +539,22 @@ def run_gpu(args):
     if dist:
         dist.destroy_process_group()
     return 0
+
+
+def roofline(s, peaks, src, fp64_peak, fp64_note, slab):
+    """Roofline of the GEMM leg (chi0 or ln det) with the longer device time, against the peak of the pipe it ran on: digit
+    planes (their MMA flops are in the stats, in the FP64 mode too) or the FP64 tensor path."""
+    leg, name = ("chi0", "k_dgemm_nt") if s["ms_gemm_chi0"] >= s["ms_gemm_ec"] else ("ec", "k_zgemm, k_dgemm_tri")
+    if s["flop_exec_gemm_" + leg] > 0:
+        return tc_roofline(s, peaks, src)
+    ms, fl = s["ms_gemm_" + leg], s["flop_gemm_" + leg]
+    achieved = fl / (ms * 1e-3) / 1e12 if ms > 0 else None
+    tr = TRAFFIC.get(name)
+    # the captured traffic is the graphene slab's (its per-launch work is the same at every k-mesh)
+    traffic = tr["bytes_per_launch"] if tr and slab and tr["src_sha"] == _src_sha(tr["src"], tr["begin"], tr["end"]) else None
+    return {"kernel": name, "bound": "tensor", "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s",
+            "frac": achieved / fp64_peak if achieved else None, "traffic": traffic, "peak_note": fp64_note,
+            "launches": s["n_gemm_" + leg], "flop": fl}
 
 
 def tc_roofline(s, peaks, src):
@@ -609,7 +611,7 @@ def time_mode(L, inp, stream, device, ntau, mode, ec_ref, torch):
            "stage_ms": {"green": s["ms_green"], "chi0": s["ms_chi0"], "freq": s["ms_freq"], "ec": s["ms_ec"]},
            "ec_ha": ec, "ec_diff_vs_fp64_mev_per_atom": dmev, "within_0.1_mev_per_atom": dmev <= 0.1,
            "steps": 1, "warmup": 1}
-    if prec != "fp64":
+    if prec != "fp64" or s["flop_exec_gemm_chi0"] > 0:
         out["roofline"] = tc_roofline(s, peaks, src)
     if theta > 0:
         out["screening"] = {"threshold": theta, "points_contracted": s["n_points_chi0"],

@@ -646,7 +646,7 @@ int librpa_gpu_ec(librpa_gpu_t h, double *ec, double *ec_q, double *ec_w) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     h->stats.ms_ec = t;
-    h->stats.ms_gemm_ec = h->stats.flop_gemm_ec = 0;
+    h->stats.ms_gemm_ec = h->stats.flop_gemm_ec = h->stats.flop_exec_gemm_ec = 0;
     h->stats.n_gemm_ec = 0;
     h->resolve_timers();
     h->stats.launches += launch_counter() - l0;

@@ -576,6 +576,7 @@ void potrf_batched(Handle &h, double2 *const *d_mats, const std::vector<double2 
       LR_CUDA(cudaEventRecord(tm.a, s));
       oz::gemm(tc->pa, tc->pi, 2 * rest, nb, B, o, 0, 0, 0, tc->err, s, h);
       LR_CUDA(cudaEventRecord(tm.b, s));
+      tm.exec_flops = h.oz_exec_flops;
       h.timed.push_back(tm);
     } else {
       launch_trsm<double2>(d_mats, B, n, ld, p0, rest, s);
@@ -602,6 +603,7 @@ void potrf_batched(Handle &h, double2 *const *d_mats, const std::vector<double2 
       LR_CUDA(cudaEventRecord(tm.a, s));
       oz::gemm(tc->pa, tc->pb, 2 * rest, rest, B, o, 0, 0, 2, tc->err, s, h);
       LR_CUDA(cudaEventRecord(tm.b, s));
+      tm.exec_flops = h.oz_exec_flops;
       h.timed.push_back(tm);
       continue;
     }
@@ -701,6 +703,7 @@ void potrf_batched_r(Handle &h, double *const *d_mats, const std::vector<double 
       LR_CUDA(cudaEventRecord(tm.a, s));
       oz::gemm(tc->pa, tc->pi, rest, nb, B, o, 0, 0, 0, tc->err, s, h);
       LR_CUDA(cudaEventRecord(tm.b, s));
+      tm.exec_flops = h.oz_exec_flops;
       h.timed.push_back(tm);
     } else {
       launch_trsm<double>(d_mats, B, n, ld, p0, rest, s);
