@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   constexpr int NU = nus(S);
   constexpr uint32_t OPB = op_bytes(S), XB_ = x_bytes(S), FIXED = static_size(S), STAGE = stage_size(S);
   extern __shared__ uint8_t smem_raw[];
-  __shared__ uint64_t full[NST], empty[NST], tfull[NSL], tempty[NSL], mdone, never;
+  __shared__ uint64_t full[NST], empty[NST], tfull[2][NSL], tempty[NSL], mdone, never;
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
   __shared__ int s_e1[kMaxAo], s_box[kTileGroups];
@@ -294,7 +294,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&empty[s], 1);
     }
     for (int s = 0; s < NSL; ++s) {
-      mbar_init(&tfull[s], 1);
+      mbar_init(&tfull[0][s], 1);
+      mbar_init(&tfull[1][s], 1);
       mbar_init(&tempty[s], 8);
     }
     mbar_init(&mdone, 1);
@@ -441,7 +442,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
         if (it % NU == NU - 1) umma_commit(&empty[st]);
-        umma_commit(&tfull[sl]);
+        umma_commit(&tfull[it & 1][sl]);
       }
       if (abort_flag) {   // after a failure: wait for the MMAs already issued
         umma_commit(&mdone);
@@ -449,7 +450,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
   } else {
-    // epilogue: warps 0-7 the even nu, 8-15 the odd ones; thread = row kap, half of the i each
+    // epilogue: warps 0-7 the even nu, 8-15 the odd ones; thread = row kap, half of the i each.  A slot has a tfull barrier
+    // for each of the two groups, which waits for every phase of its own: with an odd number of slots the groups take a
+    // slot in turn, and of one barrier a group would wait for every other phase, the parity of the one before passing for it.
     const int grp = warp >> 3, quad = warp & 3, half = (warp >> 2) & 1;
     const bool any = __any_sync(0xffffffffu, kap >= 0);
     const int per = (nU + 1) / 2, c0 = half * per, c1 = min(nU, c0 + per);
@@ -465,7 +468,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int e_lane = (int)((unsigned)e1_lane << 16) | (e2n & 0xFFFF);   // both, one shuffle per i (|e| <= 1100)
       f1n = next_f1(it + 2);
       e2n = next_e2(it + 2);
-      bool ok = !abort_flag && mbar_wait(&tfull[sl], (uint32_t)((it / NSL) & 1), WAIT_NS, &abort_flag);
+      bool ok = !abort_flag && mbar_wait(&tfull[grp][sl], (uint32_t)(it / (NSL % 2 ? 2 * NSL : NSL) & 1), WAIT_NS, &abort_flag);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) {
         abort_flag = 1;
