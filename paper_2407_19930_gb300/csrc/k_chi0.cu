@@ -1893,6 +1893,10 @@ size_t chi0_device_bytes(const Handle &h, const Chi0Plan &P) {
   size_t cols = 0;
   for (int a = 0; a < h.natoms; ++a) cols += P.m[a];
   b += (2 * cols + (size_t)P.m_all) * 6 * sizeof(int) + 16 * (size_t)(h.natoms + 1) * 8 + 12 * 256;
+  b += (cols + P.m_all) * sizeof(int2) + 2 * 256;   // folded columns
+  if (oasm_planes(h, P) > 0)   // row groups (a tile's padded to 16) and tiles of the O assembly, atom of each ABF, row of each NAO
+    b += (cols + oasm::kTileGroups * (size_t)h.natoms) * sizeof(oasm::Group) + (h.natoms + 1 + (size_t)h.naux + h.nao) * sizeof(int) +
+         4 * 256;
   return b;
 }
 

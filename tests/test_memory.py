@@ -93,3 +93,28 @@ def test_fp64_batch_bounds_its_workspaces():
             L.librpa_gpu_destroy(h)
     assert np.ptp(ec) <= 1e-12 * abs(ec[0])
     assert used < (16 << 30) + 20 * 0.15e9
+
+
+def test_server_admits_what_fits_without_planes():
+    inp, grid = _inputs()
+    o = L.librpa_gpu_default_opts()
+    h = L.librpa_gpu_create(o)
+    try:
+        L.set_inputs(h, inp, grid)
+        budget = int(L.librpa_gpu_estimate_bytes(h)) - (64 << 20)
+        L.librpa_gpu_chi0(h)
+        ec = L.librpa_gpu_ec(h)[0]
+    finally:
+        L.librpa_gpu_destroy(h)
+    s = L.librpa_gpu_server_create(slots=1, hbm_budget=budget)
+    r = None
+    try:
+        r = L.librpa_gpu_server_request(s, o)
+        L.set_inputs(r, inp, grid)
+        res = L.librpa_gpu_server_wait(s, L.librpa_gpu_server_submit(s, r), 120.0)
+        assert res["status"] == L.LIBRPA_OK and abs(res["ec"] - ec) < 1e-8
+        assert res["bytes_peak"] <= res["bytes_reserved"] <= budget
+    finally:
+        L.librpa_gpu_server_destroy(s)
+        if r:
+            L.librpa_gpu_destroy(r)
