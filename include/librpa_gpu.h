@@ -67,14 +67,25 @@ extern "C" {
  * split writes x = hi + lo with hi = tf32(x), lo = tf32(x - hi) and sums hi hi + hi lo + lo hi
  * in FP32 (about 21 bits).  In every mode other than LIBRPA_FP64 the O assembly of the chi0
  * contraction also runs on digit planes (5 for LIBRPA_FP64_TC, 3 otherwise), the ln det GEMMs
- * (including the Cholesky panel products and trailing updates) and the G(tau) products
- * C diag(w) C^H on 5 planes.  LIBRPA_SPLIT_FAST alone leaves that rule: its ln det GEMMs use 4
- * planes (~31 bits) and its tau -> omega and R -> q transforms compute in FP32 (the transform
- * weights and phases rounded to FP32), for an E_c still within 0.1 meV/atom.  So LIBRPA_FP64_TC is a ~39-bit mode, not FP64: its results match
- * the FP64 path to chi0(R, tau) 1e-10 normwise and E_c 1e-8 Ha, not bit for bit.  The
- * exponentials of G(tau), the transform weights, the Cholesky factorisations' diagonal blocks
- * and the E_c sum always stay FP64. */
-#define LIBRPA_FP64 0     /* every step in FP64 on the FP64 pipes (DMMA / DFMA) */
+ * (including the Cholesky panel products, on 8 planes for real matrices, and trailing updates) and
+ * the G(tau) products C diag(w) C^H on 5 planes.
+ *   LIBRPA_FP64 computes on the FP64 pipes (DMMA / DFMA) in small requests, and with 8 digit planes
+ * where a stage is large: the contraction from 5e8 flops on (2 M N K of its GEMMs and the O assembly,
+ * over all (R, tau) points), G from 64 NAOs on, the ln det from N_aux 96 on.  8 planes are 63 bits
+ * relative to the largest element of an operand row, their sums are exact and rounded to FP64 once.
+ * So accuracy there is relative to a row: an element more than 2^-10 below its row's largest keeps
+ * fewer than 53 bits, one below 2^-63 of it counts as zero.  NAOs and auxiliary functions are taken in
+ * units of powers of two that bring their norms together, so that results do not depend on how
+ * the caller scales the functions.  A row that holds an infinity or a NaN makes its outputs NaN.  When
+ * device memory does not hold the planes, the FP64 pipes are used; the other modes then run the O
+ * assembly in FP32 arithmetic (pairs of numbers in LIBRPA_FP64_TC).
+ *   LIBRPA_FP64_TC is a ~39-bit mode, not FP64: its results match the FP64 path to chi0(R, tau) 1e-10
+ * normwise and E_c 1e-8 Ha, not bit for bit.  LIBRPA_SPLIT_FAST alone runs its ln det GEMMs on 4
+ * planes (~31 bits) and its tau -> omega and R -> q transforms in FP32 (the transform weights and
+ * phases rounded to FP32), for an E_c still within 0.1 meV/atom.  Else, in every mode, the
+ * exponentials of G(tau), the transforms, the Cholesky factorisations' diagonal blocks and the E_c
+ * sum are FP64. */
+#define LIBRPA_FP64 0     /* FP64; the products of large stages on 8 digit planes (63 bits) */
 #define LIBRPA_FP64_TC 1  /* chi0, G and ln det GEMMs with 5 digit planes (~39 bits) on the tensor cores */
 #define LIBRPA_SPLIT 2    /* chi0 GEMMs with 3 digit planes (mixed), ln det GEMMs with 5 */
 #define LIBRPA_BF16 3     /* chi0 GEMMs in plain BF16 (FP32 accumulation), ln det GEMMs with 5 */
@@ -130,16 +141,16 @@ typedef struct {
   double ms_ec;            /* K5 + K6: Cholesky, ln det, E_c */
   double flop_chi0;        /* algorithmic FP64 flops of K2 (no padding), see the design notes */
   double flop_ec;          /* algorithmic FP64 flops of K5 */
-  double ms_gemm_chi0;     /* device time of the FP64 MMA GEMM launches of K2 (sum of per-launch events) */
+  double ms_gemm_chi0;     /* device time of the GEMM launches of K2 (sum of per-launch events) */
   double flop_gemm_chi0;   /* algorithmic flops of those launches (2 M N K, no padding) */
   long long n_gemm_chi0;   /* number of those launches */
-  double ms_gemm_ec;       /* device time of the complex GEMM launches of K5 */
+  double ms_gemm_ec;       /* device time of the GEMM launches of K5 */
   double flop_gemm_ec;     /* algorithmic flops of those launches (8 per complex MAC on the triangle) */
   long long n_gemm_ec;     /* number of those launches */
   long long launches;      /* kernels launched by the call */
   size_t bytes_device;     /* device bytes held by the handle */
   double flop_exec_gemm_chi0; /* tensor-core MMA flops issued by the timed chi0 GEMMs (digit-plane
-                                 products, tile padding and all); 0 in the FP64 mode */
+                                 products, tile padding and all); 0 on the FP64 pipes */
   double flop_exec_gemm_ec;   /* the same for the timed ln det GEMMs */
   size_t bytes_device_peak;   /* largest device footprint of the handle so far */
   long long n_points_chi0;    /* (R, tau) points contracted, summed over spin channels */
@@ -284,7 +295,7 @@ int librpa_gpu_get_grid(librpa_gpu_t h, int *n, double *tau, double *omega, doub
  * [nq][nomega][N_aux][N_aux] (N_aux^2 * nq * nomega doubles).  The device copies of
  * G, chi0(R, tau) and chi0(q, i omega) stay on the device for librpa_gpu_ec and the
  * librpa_gpu_get_* calls until the next librpa_gpu_chi0 or set_structure.
- * Errors: E_STATE, E_NOMEM, E_CUDA, E_NUMERIC. */
+ * Errors: E_STATE, E_NOMEM, E_CUDA, E_NUMERIC, E_TIMEOUT (digit planes only). */
 int librpa_gpu_chi0(librpa_gpu_t h, double *out_re, double *out_im);
 
 /* RPA correlation energy (Sec. 2, Eq. for E_c with Pi = chi0 V and Tr ln = ln det):
@@ -294,7 +305,7 @@ int librpa_gpu_chi0(librpa_gpu_t h, double *out_re, double *out_im);
  *   ec    -> E_c in Ha per cell;
  *   ec_q  -> [nq] per-q contributions (nullable);  ec_w -> [nomega] per-frequency (nullable).
  * Requires librpa_gpu_chi0 and set_coulomb for every q.
- * Errors: E_STATE, E_NOT_PD, E_NOMEM, E_CUDA. */
+ * Errors: E_STATE, E_NOT_PD, E_NOMEM, E_CUDA, E_TIMEOUT (digit planes only). */
 int librpa_gpu_ec(librpa_gpu_t h, double *ec, double *ec_q, double *ec_w);
 
 /* No-allocation variant of the ln det stage, for callers that cannot call cudaMalloc:
@@ -367,9 +378,10 @@ int librpa_gpu_get_stats(librpa_gpu_t h, librpa_gpu_stats *s);
  * The FP64-mode, single-channel handles run on the first such handle's stream, and their
  * chi0 contraction runs in rounds: round r takes the r-th batch of (R, tau) points of every
  * one of them, and runs its GEMMs as single grouped launches over all those tiles, which
- * have uneven shapes.  The GEMM tile shape is picked by timing the variants on the first
- * run; from the second run on, that launch sequence is replayed from a CUDA graph.  The
- * single-channel tensor-core handles without screening are grouped by digit-plane count; a
+ * have uneven shapes: the handles on digit planes (see LIBRPA_FP64) in one sequence, within
+ * 16 GiB of workspaces together, and the small ones on the FP64 pipes in another, whose GEMM tile
+ * shape is picked by timing the variants on the first run and which is replayed from a CUDA
+ * graph from the second run on.  The single-channel tensor-core handles without screening are grouped by digit-plane count; a
  * group's chi0 contraction runs in rounds whose N-step, X-step and final GEMMs are each one
  * launch over all the group's tiles.  Those groups and the other handles (nspins = 2,
  * screening) run at the same time on up to four library-owned streams (one host thread each).  While a batch exists, run its
@@ -379,7 +391,7 @@ typedef struct librpa_gpu_batch *librpa_gpu_batch_t;
 
 typedef struct {
   int n, n_merged;         /* handles; handles whose chi0 ran in the merged launches */
-  int graph;               /* 1 if the last run replayed the captured graph */
+  int graph;               /* 1 if the last run replayed the captured graph (handles on the FP64 pipes) */
   int var_nx, var_fin;     /* FP64 GEMM tile variants chosen: 0 = 64x64, 1 = 32x64, 2 = 64x32,
                               3 = 32x32, 4 = 128x64 (M x N); -1 = none */
   int failed_index;        /* handle of the last error (its last_error has the message), or -1 */
@@ -447,7 +459,8 @@ typedef struct {
 } librpa_gpu_server_stats;
 
 /* Upper bound of the device bytes h will hold during chi0 + ec, from its structure, LRI
- * blocks, precision and grid size (the user grid, else opts.n_tau).  Needs no GPU.
+ * blocks, precision and grid size (the user grid, else opts.n_tau), on digit planes where the
+ * precision has them (a request also runs in less, see LIBRPA_FP64).  Needs no GPU.
  * Errors: E_STATE (no structure), E_ARG. */
 int librpa_gpu_estimate_bytes(librpa_gpu_t h, size_t *bytes);
 
@@ -463,7 +476,7 @@ int librpa_gpu_server_request(librpa_gpu_server_t s, const librpa_gpu_opts *o, l
 
 /* Queue a filled request; *ticket identifies it.  The caller must not use req until
  * librpa_gpu_server_wait has returned its result.  Errors: E_STATE (inputs missing),
- * E_NOMEM (its estimate exceeds the whole budget), E_ARG. */
+ * E_NOMEM (not even its routes of least memory fit the whole budget), E_ARG. */
 int librpa_gpu_server_submit(librpa_gpu_server_t s, librpa_gpu_t req, long long *ticket);
 
 /* Wait up to timeout_s seconds (< 0: no limit) for a request's result.  Returns

@@ -110,7 +110,7 @@ struct Chi0Plan {
 // ----------------------------------------------------------------- handle
 struct Handle {
   librpa_gpu_opts opts{};
-  int chi0_S = -1;  // chi0 GEMMs: -1 = FP64 pipes, 0 = plain BF16, 1..5 = BF16 digit planes, 6 = plain TF32,
+  int chi0_S = -1;  // chi0 GEMMs: -1 = FP64 (8 digit planes or the FP64 pipes, see chi0_planes), 0 = plain BF16, 1..5 = BF16 digit planes, 6 = plain TF32,
                     // 7 = 3xTF32
   int ec_S = -1;    // ln det GEMMs: same encoding
   // FP64 mode: the stored G and the packed C are those of NAOs rescaled by 2^-ao_e[i] (k_green.cu); empty: as passed

@@ -485,7 +485,10 @@ double dgemm_batched(Handle &h, const std::vector<DGemm> &batch, cudaStream_t s,
 }  // namespace
 
 // FP64 mode: requests whose contraction takes this many flops or more run on 8 digit planes on the
-// tensor cores, smaller ones on the FP64 pipes.
+// tensor cores, smaller ones on the FP64 pipes.  Both sides measured (1 k point, 8 points, ms on the pipes / planes):
+// 1.1e6 flops 0.15 / 0.17, 3.9e6 0.22 / 0.19, 8.7e7 0.93 / 0.38, 4.7e8 2.5 / 0.30, 1.2e9 4.4 / 0.41, 1e10 18.2 / 1.1, 2.9e10
+// 32.9 / 3.4.  The line lies above the crossover: smaller requests keep the arithmetic of the pipes (and, in batches, the
+// replayed graph) at up to 2.2 ms more.
 constexpr double kWideMinFlops = 5e8;
 
 void chi0_shape(const Handle &h, Chi0Plan &P) {

@@ -20,7 +20,9 @@ namespace librpa {
 namespace {
 
 // digit planes of the G build: 5 in the tensor-core modes (FP64-accurate products), 8 in the FP64 mode
-// from kWideMinAo NAOs on (-1: the FP64 pipes)
+// from kWideMinAo NAOs on (-1: the FP64 pipes).  Both sides measured (1 k point, 8 points, ms on the pipes / planes): 9 NAOs
+// 0.40 / 0.42, 13 0.67 / 0.42, 27 0.95 / 0.46, 53 1.81 / 0.51, 74 2.34 / 0.55; the line lies above the crossover, as that of
+// the contraction.
 constexpr int kWideMinAo = 64;
 int green_planes(const Handle &h) { return h.chi0_S >= 0 ? 5 : h.nao >= kWideMinAo && !h.lean_chi0 ? oz::S_WIDE : -1; }
 

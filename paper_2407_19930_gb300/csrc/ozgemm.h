@@ -31,7 +31,7 @@ namespace oz {
 // three products hi hi + hi lo + lo hi summed in one FP32 accumulator (the "3xTF32" split)
 // S_WIDE: 8 digit planes (63 bits per operand, below the rounding of FP64), whose diagonal sums are
 // carried in two int64 words: the products of the FP64 mode
-constexpr int BM = 128, BN = 64, BK = 64, SMAX = 5, S_TF32 = 6, S_TF32X3 = 7, S_WIDE = 8;
+constexpr int BM = 128, SMAX = 5, S_TF32 = 6, S_TF32X3 = 7, S_WIDE = 8;
 __host__ __device__ constexpr bool is_digits(int S) { return (S >= 1 && S <= SMAX) || S == S_WIDE; }
 __host__ __device__ constexpr int planes(int S) { return is_digits(S) ? S : S == S_TF32X3 ? 2 : 1; }
 inline int elem_bytes(int S) { return S == S_TF32 || S == S_TF32X3 ? 4 : 2; }
@@ -107,7 +107,7 @@ struct Out {
 };
 
 // One GEMM of a grouped launch: C = alpha A[a_row0 .. + M) B[b_row0 .. + N)^T + beta C over
-// K columns.  K range per output tile starts at (m0 * km + n0 * kn) rounded down to BK
+// K columns.  K range per output tile starts at (m0 * km + n0 * kn) rounded down to the K step
 // (triangular operands); lower_div > 0 skips the tiles strictly above the diagonal, those with
 // n0 * lower_div >= m0 + BM (lower_div stacked rows per output row: 2 for complex outputs).
 constexpr int kNoShift = 1 << 30;
